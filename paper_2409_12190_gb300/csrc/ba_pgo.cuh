@@ -34,6 +34,7 @@
 #include <stdint.h>
 
 #include "ba_band.cuh"
+#include "ba_gridx.cuh"
 #include "ba_kernels.cuh"
 
 namespace ba {
@@ -510,7 +511,7 @@ __device__ __forceinline__ void grid_total(const double* __restrict__ part, int 
 
 struct PcgArgs {
   int N;
-  int npb;             // nodes per block pass (blockDim.x = 6 npb)
+  int npb;             // nodes per block pass (blockDim.x >= 6 npb, a multiple of 32)
   const int32_t* rowptr;
   const int2* inc2;    // per incidence slot: (edge, other node)
   const double* B;
@@ -528,6 +529,7 @@ struct PcgArgs {
   int maxiter;
   double tol;
   GridBar* bar;
+  GridX gx;  // k_pgo_pcg_res: the blocks' sums
   DevState* st;
 };
 
@@ -726,22 +728,33 @@ static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg(PcgArgs a
 }
 
 // Shared memory of k_pgo_pcg_res for a block of `slots` incidence slots:
-// their B blocks (36), neighbour directions (6) and neighbour indices.
-__host__ __device__ constexpr size_t pgo_res_smem(int slots) { return (size_t)slots * (36 * 8 + 6 * 8 + 4); }
+// their B blocks (36), neighbour directions (6), differences (6), neighbour
+// indices and owning nodes.
+__host__ __device__ constexpr size_t pgo_res_smem(int slots) { return (size_t)slots * (36 * 8 + 12 * 8 + 4 + 1); }
+// 64-bit words the kernel exchanges through, zero before the launch: the
+// slots of `blocks` blocks, then z of N nodes.
+constexpr size_t pgo_res_words(int blocks, int N) { return gx_bytes(blocks) / 8 + 12 * (size_t)N; }
 
 // The same iteration as k_pgo_pcg when every block holds exactly one group
 // of npb nodes (gridDim.x = ceil(N / npb)): each thread keeps its entry of
-// x, r, z, p, D and its row of M for the whole solve in registers, the
-// block's B blocks and neighbour indices are staged in shared memory once,
-// and per iteration only the neighbours' z and p_old cross global memory.
-// Same arithmetic, in the same order, as k_pgo_pcg.
+// x, r, z, p, D and its row of M for the whole solve in registers, and the
+// block's B blocks and its neighbours' directions stay in shared memory
+// (p_other = z_other + beta p_other is formed where it is needed), so per
+// iteration only z and the two exchanges' sums cross global memory, without
+// fences (ba_gridx.cuh); the neighbours' z are fetched while the second
+// exchange is under way.
+//
+// What bounds it: latency, and the FP64 pipe (16 cycles a warp instruction):
+// the product takes one thread per (slot, row), five slots a warp, and the
+// differences p - p_other are formed once per slot instead of once per row.
+// A 2,500-pose sphere (147 blocks), two trials of 100 iterations with all
+// else of them: 4.00 ms with counter barriers and a thread per (node, row),
+// 2.54 ms now (about 18 and 11 us an iteration).
 static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg_res(PcgArgs a) {
   extern __shared__ __align__(16) unsigned char pgo_smem[];
   __shared__ double sr[PGO_PCG_NODES][6];
-  const unsigned int G = gridDim.x;
   const int N = a.N;
   const int npb = a.npb;
-  const long long n6 = 6LL * N;
   const int ln = threadIdx.x / 6, row = threadIdx.x % 6;
   const int n0 = blockIdx.x * npb;
   const int n = n0 + ln;
@@ -752,14 +765,19 @@ static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg_res(PcgAr
   const int s_lo = __ldg(a.rowptr + n0), s_hi = __ldg(a.rowptr + nend);
   const int nsl = s_hi - s_lo;
   double* sB = reinterpret_cast<double*>(pgo_smem);  // [nsl][36]
-  double* sp = sB + 36LL * nsl;                      // [nsl][6]
-  int* sother = reinterpret_cast<int*>(sp + 6LL * nsl);
+  double* sp = sB + 36LL * nsl;                      // [nsl][6]: the neighbours' directions
+  double* su = sp + 6LL * nsl;                       // [nsl][6]: their z, then p - p_other, then B (p - p_other)
+  int* sother = reinterpret_cast<int*>(su + 6LL * nsl);
+  unsigned char* sown = reinterpret_cast<unsigned char*>(sother + nsl);  // the slot's node within the block
   for (int e = threadIdx.x; e < nsl * 36; e += blockDim.x) {
     const int sl = e / 36, k = e % 36;
     sB[e] = __ldg(a.B + 36LL * __ldg(&a.inc2[s_lo + sl].x) + k);
   }
+  for (int e = threadIdx.x; e < nsl * 6; e += blockDim.x) sp[e] = 0.0;
   for (int sl = threadIdx.x; sl < nsl; sl += blockDim.x) sother[sl] = __ldg(&a.inc2[s_lo + sl].y);
   const int my_lo = live ? __ldg(a.rowptr + n) - s_lo : 0, my_hi = live ? __ldg(a.rowptr + n + 1) - s_lo : 0;
+  if (live && row == 0)
+    for (int sl = my_lo; sl < my_hi; ++sl) sown[sl] = (unsigned char)ln;
   double Mrow[6];
   double Da = 0.0, ra = 0.0, xa = 0.0, za = 0.0, pa = 0.0;
   if (live) {
@@ -781,74 +799,88 @@ static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg_res(PcgAr
     }
     return;
   }
-  double* pold = a.p;
-  double* pcur = a.p + n6;
+  // z of every node as other blocks read it; the neighbours' z of this block's
+  // slots into su (all warps but the first)
+  unsigned long long* zx = a.gx.slots + gx_bytes(gridDim.x) / 8;
+  auto fetch_z = [&](unsigned int epoch) {
+    return gx_gather<8>(a.gx, zx, epoch, nsl * 6, threadIdx.x - 32, blockDim.x - 32,
+                        [&](int e) { return 6 * sother[e / 6] + e % 6; }, su);
+  };
   double rz_part = 0.0;
   if (live) {
     double zz = 0.0;
 #pragma unroll
     for (int k = 0; k < 6; ++k) zz += Mrow[k] * sr[ln][k];
     za = zz;
-    a.z[o] = za;
-    pold[o] = 0.0;
+    gx_put(zx + 2 * o, 1, za);
     rz_part = za * ra;
   }
-  {
-    double v[1] = {rz_part};
-    block_sum_all<1>(v);
-    if (threadIdx.x == 0) a.part[4LL * blockIdx.x] = v[0];
-  }
-  if (!grid_barrier(a.bar, G)) return;
   double rz;
   {
-    double v[1] = {0.0};
-    for (int i = threadIdx.x; i < (int)G; i += blockDim.x) v[0] += __ldcg(a.part + 4LL * i);
-    block_sum_all<1>(v);
+    double v[1] = {rz_part};
+    if (!grid_exchange<1, PGO_PCG_THREADS>(a.gx, 1, 1, v, [&] { return fetch_z(1); })) return;
     rz = v[0];
   }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int wsl = lane / 6, wrow = lane % 6;  // five slots a warp, lanes 30 and 31 idle
   double beta = 0.0;
   double rel = 1.0;
   int it = 0;
   while (it < a.maxiter) {
-    // phase A: p = z + beta p_old; q = (H + D) p; p . q
+    // phase A: p = z + beta p; q = (H + D) p; p . q
     pa = za + beta * pa;
-    if (live) {
-      sr[ln][row] = pa;
-      pcur[o] = pa;
-    }
-    for (int e = threadIdx.x; e < nsl * 6; e += blockDim.x) {
-      const int sl = e / 6, k = e % 6;
-      const long long g = 6LL * sother[sl] + k;
-      sp[e] = __ldcg(a.z + g) + beta * __ldcg(pold + g);
+    if (live) sr[ln][row] = pa;
+    __syncthreads();
+    // U groups of five slots a warp: lane (slot, k) forms p - p_other, then
+    // lane (slot, row) the row's product
+    constexpr int U = 2;
+    for (int s0 = warp * 5 * U; s0 < nsl; s0 += nw * 5 * U) {
+      int sl[U];
+      bool on[U];
+      double po[U], pi[U], acc[U];
+#pragma unroll
+      for (int g = 0; g < U; ++g) {
+        sl[g] = s0 + 5 * g + wsl;
+        on[g] = wsl < 5 && sl[g] < nsl;
+        po[g] = on[g] ? su[6 * sl[g] + wrow] + beta * sp[6 * sl[g] + wrow] : 0.0;
+        pi[g] = on[g] ? sr[sown[sl[g]]][wrow] : 0.0;
+      }
+#pragma unroll
+      for (int g = 0; g < U; ++g)
+        if (on[g]) {
+          sp[6 * sl[g] + wrow] = po[g];
+          su[6 * sl[g] + wrow] = pi[g] - po[g];
+        }
+      __syncwarp();
+#pragma unroll
+      for (int g = 0; g < U; ++g) {
+        acc[g] = 0.0;
+        if (on[g]) {
+          const double2* Br = reinterpret_cast<const double2*>(sB + 36LL * sl[g] + 6 * wrow);
+          const double2* u = reinterpret_cast<const double2*>(su + 6LL * sl[g]);
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            const double2 b = Br[k], w = u[k];
+            acc[g] += b.x * w.x;
+            acc[g] += b.y * w.y;
+          }
+        }
+      }
+      __syncwarp();  // the slots' lanes have read their differences
+#pragma unroll
+      for (int g = 0; g < U; ++g)
+        if (on[g]) su[6 * sl[g] + wrow] = acc[g];
     }
     __syncthreads();
     double qa = 0.0;
     if (free_n) {
-      double pi[6];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) pi[k] = sr[ln][k];
-      for (int sl = my_lo; sl < my_hi; ++sl) {
-        const double* Br = sB + 36LL * sl + 6 * row;
-        const double* po = sp + 6LL * sl;
-        double acc = 0.0;
-#pragma unroll
-        for (int k = 0; k < 6; ++k) acc += Br[k] * (pi[k] - po[k]);
-        qa += acc;
-      }
+      for (int sl = my_lo; sl < my_hi; ++sl) qa += su[6 * sl + row];
       qa += Da * pa;
     }
-    double pq_part = live ? pa * qa : 0.0;
-    {
-      double v[1] = {pq_part};
-      block_sum_all<1>(v);
-      if (threadIdx.x == 0) a.part[4LL * blockIdx.x + 1] = v[0];
-    }
-    if (!grid_barrier(a.bar, G)) return;
     double pq;
     {
-      double v[1] = {0.0};
-      for (int i = threadIdx.x; i < (int)G; i += blockDim.x) v[0] += __ldcg(a.part + 4LL * i + 1);
-      block_sum_all<1>(v);
+      double v[1] = {live ? pa * qa : 0.0};
+      if (!grid_exchange<1, PGO_PCG_THREADS>(a.gx, 0, it + 1, v)) return;
       pq = v[0];
     }
     if (!(pq > 0.0)) break;
@@ -867,27 +899,14 @@ static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg_res(PcgAr
 #pragma unroll
       for (int k = 0; k < 6; ++k) zz += Mrow[k] * sr[ln][k];
       za = zz;
-      a.z[o] = za;
+      gx_put(zx + 2 * o, it + 2, za);
       rzp = za * ra;
     }
     ++it;
-    {
-      double v[2] = {rr_part, rzp};
-      block_sum_all<2>(v);
-      if (threadIdx.x == 0) {
-        a.part[4LL * blockIdx.x + 2] = v[0];
-        a.part[4LL * blockIdx.x + 3] = v[1];
-      }
-    }
-    if (!grid_barrier(a.bar, G)) return;
     double rr, rz_new;
     {
-      double v[2] = {0.0, 0.0};
-      for (int i = threadIdx.x; i < (int)G; i += blockDim.x) {
-        v[0] += __ldcg(a.part + 4LL * i + 2);
-        v[1] += __ldcg(a.part + 4LL * i + 3);
-      }
-      block_sum_all<2>(v);
+      double v[2] = {rr_part, rzp};
+      if (!grid_exchange<2, PGO_PCG_THREADS>(a.gx, 1, it + 1, v, [&] { return fetch_z(it + 1); })) return;
       rr = v[0];
       rz_new = v[1];
     }
@@ -895,9 +914,6 @@ static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg_res(PcgAr
     if (sqrt(rr) <= a.tol * bnorm) break;
     beta = rz_new / rz;
     rz = rz_new;
-    double* t = pold;
-    pold = pcur;
-    pcur = t;
   }
   if (live) a.x[o] = xa;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
