@@ -64,8 +64,12 @@ enum { BA_JAC_AUTO = 0, BA_JAC_RECOMPUTE = 1, BA_JAC_STORE = 2 };
 
 /* How each LM trial solves the reduced camera system S dc = b (Sec. IV-C:
  * the paper offers PCG and a sparse direct solver, a Cholesky
- * factorisation).  BA_SOLVER_PCG: block-Jacobi PCG with the implicit S x
- * product (pcg_maxiter, pcg_tol).  BA_SOLVER_CHOLESKY: S formed explicitly
+ * factorisation).  BA_SOLVER_PCG: block-Jacobi PCG (pcg_maxiter,
+ * pcg_tol) with the implicit S x product or, where the observation structure
+ * makes that faster, on S formed once per trial (only the blocks of camera
+ * pairs with common points; chosen at create, the same for every trial; a
+ * bounded wait of its one launch that runs out, about a second, leaves dc = 0
+ * for the trial).  BA_SOLVER_CHOLESKY: S formed explicitly
  * as a dense 9C x 9C FP64 matrix and factored by a tiled Cholesky on the
  * GPU (the factorisation and both triangular solves in one cooperative
  * launch), for problems with 9C <= BA_DENSE_MAX_DIM (the matrix and its

@@ -299,17 +299,22 @@ void enqueue_dense_solve(ba_problem* h, const double* lam_ptr) {
   cudaStream_t s = h->s;
   const int n = 9 * h->C;
   Prof pr(h, BA_K_OTHER);
+  if (h->sx.direct) {
+    schur_form(h);
+    cudaMemsetAsync(h->bT, 0, h->bT_bytes, s);
+    schur_to_band(h, lam_ptr);
+  } else {
   k_dense_w<T, MF><<<nblk(h->P, DENSE_THREADS), DENSE_THREADS, 0, s>>>(
       h->P, h->rowptr_pt, h->pm_cam, h->pm2cm, (const T*)h->Jcm, (const T*)h->cm_sw, (const T*)h->camtab,
       (const T*)h->pts, h->st, h->O, h->Wd);
   k_schur_dense<T><<<h->C * h->nseg, DENSE_THREADS, 0, s>>>(
       h->C, h->nseg, h->rowptr_cam, h->cm_pt, h->rowptr_pt, h->pm_cam, h->pm2cm, h->Wd, (const T*)h->Vinv, h->Spart);
-  count_launch();
   cudaMemsetAsync(h->bT, 0, h->bT_bytes, s);
-  cudaMemsetAsync(h->bflag, 0, sizeof(int) * h->bflag_count, s);
   k_schur_to_band<<<n, 256, 0, s>>>(h->C, h->nseg, h->Spart, h->U, lam_ptr, h->opt.diag_min, h->opt.diag_max,
                                     h->fixed, h->bwt, h->bT);
-  count_launch(2);
+  count_launch(3);
+  }
+  cudaMemsetAsync(h->bflag, 0, sizeof(int) * h->bflag_count, s);
   if (h->bnb * BAND_TB > n) {
     k_band_pad<<<1, BAND_TB, 0, s>>>(n, h->bnb, h->bwt, h->bT);
     count_launch();
@@ -359,7 +364,7 @@ void enqueue_solve(ba_problem* h, const double* lam_ptr, int maxiter, double tol
     Prof pr(h, BA_K_OTHER);
     k_cam_combine_schur<T, MF><<<h->ncb, CAM_THREADS, 0, s>>>(
         h->C, sptr, spart, h->U, h->gc, (const T*)h->camtab, lam_ptr, dmin, dmax, h->Minv, h->x,
-        h->r, h->z, h->p, (T*)h->pT, h->dot_rz + h->ncb, h->dot_bb, h->fixed, h->st, learned ? h->Sii : nullptr);
+        h->r, h->z, h->p, (T*)h->pT, h->dot_rz + h->ncb, h->dot_bb, h->fixed, h->st, learned || h->sx.pcg ? h->Sii : nullptr);
   }
   count_launch(3);
   if (learned) {
@@ -377,6 +382,13 @@ void enqueue_solve(ba_problem* h, const double* lam_ptr, int maxiter, double tol
   }
   if (h->opt.solver == BA_SOLVER_CHOLESKY) {
     enqueue_dense_solve<T, MF>(h, lam_ptr);
+  } else if (h->sx.pcg && !h->xch) {
+    {
+      Prof pr(h, BA_K_SCHUR_CAM);
+      schur_form(h);
+    }
+    Prof pr(h, BA_K_OTHER);
+    schur_pcg(h, maxiter, tol);
   } else {
     for (int k = 0; k < maxiter; ++k) {
       enqueue_pcg_iter<T, MF>(h, lam_ptr, k, tol);
@@ -792,12 +804,17 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
   CU(h->alloc(&h->dp, 3 * P * ts));
   CU(h->alloc(&h->part, (size_t)PART * std::max(h->npieces, 1) * 8));
   h->ncb = (int)nblk(C, CAM_THREADS);
+  {
+    const ba_status sb = schur_build(h, rq);
+    if (sb != BA_OK) return sb;
+  }
   if (h->opt.solver == BA_SOLVER_CHOLESKY) {
-    // the direct solve: W of every observation; partial copies of S, one
-    // CTA per camera and copy building them (as many copies as keep every
-    // CTA resident and fit in 96 MB, so in L2; at most 8, at least 1); the
-    // band tiles of the whole lower triangle; the factorisation's task list
-    // (ba_band_sched.h) for one block per SM
+    // the direct solve: the band tiles of the whole lower triangle; the
+    // factorisation's task list (ba_band_sched.h) for one block per SM; where
+    // S is not formed from sorted pairs (ba_schur.cu): W of every observation
+    // and partial copies of S, one CTA per camera and copy building them (as
+    // many copies as keep every CTA resident and fit in 96 MB, so in L2; at
+    // most 8, at least 1)
     const size_t n = 9 * (size_t)C;
     int dev = 0, nsm = 1, occ = 1;
     CU(cudaGetDevice(&dev));
@@ -806,8 +823,10 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
     const size_t by_slots = (size_t)std::max(1, occ) * (size_t)nsm / (size_t)std::max<long long>(1, C);
     const size_t by_bytes = (96ull << 20) / (n * n * 8);
     h->nseg = (int)std::max<size_t>(1, std::min<size_t>(8, std::min(by_slots, by_bytes)));
-    CU(h->alloc(&h->Wd, 27ull * 8 * (size_t)std::max<long long>(O, 1)));
-    CU(h->alloc(&h->Spart, (size_t)h->nseg * n * n * 8));
+    if (!h->sx.direct) {
+      CU(h->alloc(&h->Wd, 27ull * 8 * (size_t)std::max<long long>(O, 1)));
+      CU(h->alloc(&h->Spart, (size_t)h->nseg * n * n * 8));
+    }
     h->bnb = (int)((n + BAND_TB - 1) / BAND_TB);
     h->bwt = h->bnb - 1;
     const long long nupd = (long long)h->bnb * h->bwt * (h->bwt + 1) / 2;
@@ -965,13 +984,13 @@ void enqueue_slow_probes(ba_problem* h, const double* lam_ptr, int n, const int*
 }
 
 ba_status ensure_learn_buffers(ba_problem* h) {
-  if (h->Sii) return BA_OK;
-  CU(h->alloc(&h->mlp, (size_t)MLP_NPARAM * 4));
-  CU(h->alloc(&h->Sii, 45ull * h->C * 8));
+  if (h->mlp) return BA_OK;
+  if (!h->Sii) CU(h->alloc(&h->Sii, 45ull * h->C * 8));
   CU(h->alloc(&h->Xf, (size_t)MLP_FIN * h->C * 4));
   CU(h->alloc(&h->Ef, (size_t)MLP_FOUT * h->C * 4));
   CU(h->alloc(&h->Dsc, 9ull * h->C * 8));
   CU(h->alloc(&h->kap, (size_t)h->C * 8));
+  CU(h->alloc(&h->mlp, (size_t)MLP_NPARAM * 4));  // last: its presence means all are there
   CU(cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MLP_SMEM_FWD));
   return BA_OK;
 }
@@ -1067,6 +1086,53 @@ ba_status backward_via_f64(ba_problem* h, double lambda, int maxiter, double tol
   return st;
 }
 
+ba_status ba::problem_create(ba_problem** out, int C, int P, int O, const void* cams, const void* points,
+                             const int32_t* cam_idx, const int32_t* pt_idx, const void* pixels,
+                             const ba_options* opt, void* stream, bool batched) {
+  if (!out) return fail(BA_ERR_INVALID_ARG, "NULL output handle");
+  *out = nullptr;
+  if (C < 1 || P < 1 || O < 1) return fail(BA_ERR_INVALID_ARG, "C, P and O must be >= 1 (got %d, %d, %d)", C, P, O);
+  if (!cams || !points || !cam_idx || !pt_idx || !pixels) return fail(BA_ERR_INVALID_ARG, "NULL input array");
+  ba_options o;
+  if (opt) o = *opt;
+  else ba_options_default(&o);
+  ba_status st = check_options(&o);
+  if (st != BA_OK) return st;
+  if (o.solver == BA_SOLVER_CHOLESKY && 9LL * C > BA_DENSE_MAX_DIM)
+    return fail(BA_ERR_INVALID_ARG, "BA_SOLVER_CHOLESKY needs 9C <= %d (C = %d)", BA_DENSE_MAX_DIM, C);
+  ba_problem* h = new (std::nothrow) ba_problem();
+  if (!h) return fail(BA_ERR_OOM, "host allocation failed");
+  h->C = C;
+  h->P = P;
+  h->O = O;
+  h->prec = o.precision;
+  h->mf = o.jacobian_mode == BA_JAC_RECOMPUTE || (o.jacobian_mode == BA_JAC_AUTO && o.precision == BA_PREC_F32);
+  h->tsize = o.precision == BA_PREC_F32 ? 4 : 8;
+  h->opt = o;
+  h->batched = batched;
+  cudaError_t e = cudaStreamCreateWithFlags(&h->s, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_out, cudaEventDisableTiming);
+  if (e != cudaSuccess) {
+    delete h;
+    return fail(BA_ERR_CUDA, "stream/event creation failed: %s", cudaGetErrorString(e));
+  }
+  st = enter(h, stream);
+  if (st == BA_OK) {
+    st = h->prec == BA_PREC_F32 ? create_impl<float>(h, cams, points, cam_idx, pt_idx, pixels)
+                                : create_impl<double>(h, cams, points, cam_idx, pt_idx, pixels);
+  }
+  if (st != BA_OK) {
+    std::string msg = g_err;
+    cudaStreamSynchronize(h->s);
+    delete h;
+    g_err = msg;
+    return st;
+  }
+  *out = h;
+  return BA_OK;
+}
+
 extern "C" {
 
 ba_status ba_options_default(ba_options* o) {
@@ -1094,47 +1160,7 @@ ba_status ba_options_default(ba_options* o) {
 ba_status ba_problem_create(ba_problem** out, int C, int P, int O, const void* cams, const void* points,
                             const int32_t* cam_idx, const int32_t* pt_idx, const void* pixels,
                             const ba_options* opt, void* stream) {
-  if (!out) return fail(BA_ERR_INVALID_ARG, "NULL output handle");
-  *out = nullptr;
-  if (C < 1 || P < 1 || O < 1) return fail(BA_ERR_INVALID_ARG, "C, P and O must be >= 1 (got %d, %d, %d)", C, P, O);
-  if (!cams || !points || !cam_idx || !pt_idx || !pixels) return fail(BA_ERR_INVALID_ARG, "NULL input array");
-  ba_options o;
-  if (opt) o = *opt;
-  else ba_options_default(&o);
-  ba_status st = check_options(&o);
-  if (st != BA_OK) return st;
-  if (o.solver == BA_SOLVER_CHOLESKY && 9LL * C > BA_DENSE_MAX_DIM)
-    return fail(BA_ERR_INVALID_ARG, "BA_SOLVER_CHOLESKY needs 9C <= %d (C = %d)", BA_DENSE_MAX_DIM, C);
-  ba_problem* h = new (std::nothrow) ba_problem();
-  if (!h) return fail(BA_ERR_OOM, "host allocation failed");
-  h->C = C;
-  h->P = P;
-  h->O = O;
-  h->prec = o.precision;
-  h->mf = o.jacobian_mode == BA_JAC_RECOMPUTE || (o.jacobian_mode == BA_JAC_AUTO && o.precision == BA_PREC_F32);
-  h->tsize = o.precision == BA_PREC_F32 ? 4 : 8;
-  h->opt = o;
-  cudaError_t e = cudaStreamCreateWithFlags(&h->s, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_out, cudaEventDisableTiming);
-  if (e != cudaSuccess) {
-    delete h;
-    return fail(BA_ERR_CUDA, "stream/event creation failed: %s", cudaGetErrorString(e));
-  }
-  st = enter(h, stream);
-  if (st == BA_OK) {
-    st = h->prec == BA_PREC_F32 ? create_impl<float>(h, cams, points, cam_idx, pt_idx, pixels)
-                                : create_impl<double>(h, cams, points, cam_idx, pt_idx, pixels);
-  }
-  if (st != BA_OK) {
-    std::string msg = g_err;
-    cudaStreamSynchronize(h->s);
-    delete h;
-    g_err = msg;
-    return st;
-  }
-  *out = h;
-  return BA_OK;
+  return ba::problem_create(out, C, P, O, cams, points, cam_idx, pt_idx, pixels, opt, stream, false);
 }
 
 ba_status ba_problem_destroy(ba_problem* h) {

@@ -116,19 +116,22 @@ __device__ __forceinline__ void gx_warp_sums(double (&t)[NV]) {
   }
 }
 
-// Sums v over the block, then over the grid: every thread of every block
-// returns the totals in v.  Meanwhile the other warps run overlap(), which
+// Sums v over the block, then over the grid; the warp that has the totals
+// turns them into what the block goes on with, finish(totals), NV numbers that
+// every thread of every block returns in v.  (A division or a square root in
+// every warp of a block of 16 cost 5 us: 16 cycles for each of their FP64
+// instructions and warp.)  Meanwhile the other warps run overlap(), which
 // returns false if it gave up.  Returns false in every thread of the block if
 // a wait ran out.  set 0 or 1 alternates between calls, epoch is the call's
 // number in its set (1, 2, ...).  blockDim.x is a multiple of 32, at least 64
-// and at most NT.  The call begins and ends with a block barrier.
+// and at most NT; only the first nv threads (a multiple of 32) hold values.  The call begins and ends with a block barrier.
 //
 // One warp does the adding: an FP64 warp instruction takes 16 cycles of its
 // SM here, and a shuffle tree in every warp of every block was a quarter of a
 // PCG iteration.
-template <int NV, int NT, typename Overlap>
-__device__ __forceinline__ bool grid_exchange(const GridX& gx, int set, unsigned int epoch, double (&v)[NV],
-                                              Overlap overlap) {
+template <int NV, int NT, typename Finish, typename Overlap>
+__device__ __forceinline__ bool grid_exchange(const GridX& gx, int set, unsigned int epoch, double (&v)[NV], int nv,
+                                              Finish finish, Overlap overlap) {
   static_assert(2 * NV <= GX_WORDS, "a slot holds two doubles");
   __shared__ double s_v[NV][NT];
   __shared__ double s_tot[NV];
@@ -144,7 +147,7 @@ __device__ __forceinline__ bool grid_exchange(const GridX& gx, int set, unsigned
     double t[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) t[i] = s_v[i][lane];
-    for (int k = 32; k < (int)blockDim.x; k += 32)
+    for (int k = 32; k < nv; k += 32)
 #pragma unroll
       for (int i = 0; i < NV; ++i) t[i] += s_v[i][lane + k];
     gx_warp_sums(t);
@@ -185,6 +188,7 @@ __device__ __forceinline__ bool grid_exchange(const GridX& gx, int set, unsigned
           if (b0 + 32 * u + lane < G) t[i] += gx_value(w[u][2 * i], w[u][2 * i + 1]);
     }
     gx_warp_sums(t);
+    finish(t);
 #pragma unroll
     for (int i = 0; i < NV; ++i)
       if (lane == 0) s_tot[i] = t[i];
@@ -196,11 +200,6 @@ __device__ __forceinline__ bool grid_exchange(const GridX& gx, int set, unsigned
 #pragma unroll
   for (int i = 0; i < NV; ++i) v[i] = s_tot[i];
   return !(s_fail[0] | s_fail[1]);
-}
-
-template <int NV, int NT>
-__device__ __forceinline__ bool grid_exchange(const GridX& gx, int set, unsigned int epoch, double (&v)[NV]) {
-  return grid_exchange<NV, NT>(gx, set, epoch, v, [] { return true; });
 }
 
 }  // namespace ba

@@ -815,16 +815,17 @@ static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg_res(PcgAr
     gx_put(zx + 2 * o, 1, za);
     rz_part = za * ra;
   }
-  double rz;
+  // the polling warp keeps r . z and the last |r|^2
+  double rz, rr = 0.0;
   {
     double v[1] = {rz_part};
-    if (!grid_exchange<1, PGO_PCG_THREADS>(a.gx, 1, 1, v, [&] { return fetch_z(1); })) return;
+    if (!grid_exchange<1, PGO_PCG_THREADS>(a.gx, 1, 1, v, blockDim.x, [](double(&)[1]) {}, [&] { return fetch_z(1); })) return;
     rz = v[0];
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int wsl = lane / 6, wrow = lane % 6;  // five slots a warp, lanes 30 and 31 idle
+  const double stop = a.tol * bnorm;
   double beta = 0.0;
-  double rel = 1.0;
   int it = 0;
   while (it < a.maxiter) {
     // phase A: p = z + beta p; q = (H + D) p; p . q
@@ -877,14 +878,17 @@ static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg_res(PcgAr
       for (int sl = my_lo; sl < my_hi; ++sl) qa += su[6 * sl + row];
       qa += Da * pa;
     }
-    double pq;
+    // alpha = r . z / p . (H + D) p, or NaN to stop
+    double alpha;
     {
       double v[1] = {live ? pa * qa : 0.0};
-      if (!grid_exchange<1, PGO_PCG_THREADS>(a.gx, 0, it + 1, v)) return;
-      pq = v[0];
+      if (!grid_exchange<1, PGO_PCG_THREADS>(a.gx, 0, it + 1, v, blockDim.x,
+                                             [&](double(&t)[1]) { t[0] = t[0] > 0.0 ? rz / t[0] : nan(""); },
+                                             [] { return true; }))
+        return;
+      alpha = v[0];
     }
-    if (!(pq > 0.0)) break;
-    const double alpha = rz / pq;
+    if (isnan(alpha)) break;
     // phase B: x += alpha p, r -= alpha q, z = M r; r . r, r . z
     double rr_part = 0.0, rzp = 0.0;
     if (live) {
@@ -903,22 +907,28 @@ static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg_res(PcgAr
       rzp = za * ra;
     }
     ++it;
-    double rr, rz_new;
+    // beta and whether |r| <= tol |b|
     {
       double v[2] = {rr_part, rzp};
-      if (!grid_exchange<2, PGO_PCG_THREADS>(a.gx, 1, it + 1, v, [&] { return fetch_z(it + 1); })) return;
-      rr = v[0];
-      rz_new = v[1];
+      if (!grid_exchange<2, PGO_PCG_THREADS>(
+              a.gx, 1, it + 1, v, blockDim.x,
+              [&](double(&t)[2]) {
+                rr = t[0];
+                const double rz_new = t[1];
+                t[0] = sqrt(rr) <= stop ? 1.0 : 0.0;
+                t[1] = rz_new / rz;
+                rz = rz_new;
+              },
+              [&] { return fetch_z(it + 1); }))
+        return;
+      beta = v[1];
+      if (v[0] != 0.0) break;
     }
-    rel = sqrt(rr) / bnorm;
-    if (sqrt(rr) <= a.tol * bnorm) break;
-    beta = rz_new / rz;
-    rz = rz_new;
   }
   if (live) a.x[o] = xa;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     a.st->pcg_iters = it;
-    a.st->pcg_rel = it == 0 ? 1.0 : rel;
+    a.st->pcg_rel = it == 0 ? 1.0 : sqrt(rr) / bnorm;
     a.st->pcg_done = 1;
   }
 }

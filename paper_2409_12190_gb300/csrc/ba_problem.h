@@ -11,6 +11,23 @@
 #include "ba.h"
 #include "ba_kernels.cuh"
 
+struct ba_problem;
+
+namespace ba {
+// ba_problem_create; batched: the concatenated problems of a batch.
+ba_status problem_create(ba_problem** out, int C, int P, int O, const void* cams, const void* points,
+                         const int32_t* cam_idx, const int32_t* pt_idx, const void* pixels, const ba_options* opt,
+                         void* stream, bool batched);
+// The reduced system formed explicitly (ba_schur.cu).  schur_build chooses
+// between it and the implicit product and builds what it needs (rq: the row
+// pointers of the observations by point); h->sx.pcg / h->sx.direct say what
+// was chosen.  The others enqueue on h->s.
+ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq);
+void schur_form(ba_problem* h);                                 // the pairs' partial blocks
+void schur_to_band(ba_problem* h, const double* lam_ptr);       // into the band tiles
+void schur_pcg(ba_problem* h, int maxiter, double tol);         // panels, then the PCG (S_ii, M and r given)
+}  // namespace ba
+
 struct ba_problem {
   int C = 0, P = 0, O = 0, prec = 0;
   bool mf = false;  // recompute the Jacobian factors in every pass
@@ -87,6 +104,25 @@ struct ba_problem {
   int4* btask = nullptr;
   int bnb = 0, bwt = 0, bntask = 0, bncrit = 0, band_grid = 0, band_crit = 0;
   size_t bT_bytes = 0, bflag_count = 0;
+  // the reduced system formed block by block (ba_schur.cuh): pairs of
+  // observations sorted by camera pair, tasks, blocks; the PCG's row panels,
+  // camera lists and parts, and the words its blocks exchange through
+  struct {
+    bool direct = false;  // into the band tiles (else the row panels of the PCG)
+    bool pcg = false;     // ba_schur.cuh's PCG instead of the implicit product
+    int nblk = 0, ntask = 0, groups = 0, rpb = 0, nc_max = 0, parts_max = 0;
+    size_t words = 0;
+    int32_t *pk = nullptr, *pl = nullptr, *pj = nullptr;
+    int4* task = nullptr;
+    int2 *blk_cam = nullptr, *blk_pos = nullptr;
+    int* blk_task = nullptr;
+    void *part = nullptr, *val = nullptr;
+    int32_t *rowblk = nullptr, *cams = nullptr, *cam_ptr = nullptr, *part_ptr = nullptr, *row_part = nullptr;
+    uint16_t *colloc = nullptr, *ownloc = nullptr;
+    int4* parts = nullptr;
+    unsigned long long* gx = nullptr;
+  } sx;
+  bool batched = false;  // the concatenated problems of a batch: never solved as one
   ba::DevState* st = nullptr;
   ba_iter_stats* stats = nullptr;
   int cap = 0;

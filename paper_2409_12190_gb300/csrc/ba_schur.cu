@@ -1,0 +1,444 @@
+// Host side of the explicitly formed reduced camera system (ba_schur.cuh):
+// when it pays, its symbolic phase, and the launches.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <type_traits>
+#include <vector>
+
+#include "ba.h"
+#include "ba_internal.h"
+#include "ba_problem.h"
+#include "ba_schur.cuh"
+
+namespace ba {
+
+namespace {
+
+#define SCU(call)                                                                                       \
+  do {                                                                                                  \
+    cudaError_t e_ = (call);                                                                            \
+    if (e_ != cudaSuccess)                                                                              \
+      return set_error(e_ == cudaErrorMemoryAllocation ? BA_ERR_OOM : BA_ERR_CUDA, "%s failed: %s (%s:%d)", #call, \
+                       cudaGetErrorString(e_), __FILE__, __LINE__);                                     \
+  } while (0)
+
+inline unsigned nb_(long long n, int t) { return (unsigned)((n + t - 1) / t); }
+
+constexpr long long MAX_PAIRS = 1ll << 27;  // 12 bytes each kept, 36 more while they are sorted
+
+// FP32: formed only where the implicit iteration is mostly launches (20 us of
+// which 12 are launches at this size).  Beyond it the formed S would still be
+// 1.4 times as fast on 8.0M observations, but its rounding is another one than
+// the implicit product's, and on rings of thousands of cameras the points of
+// three neighbouring views amplify FP32 rounding (V* conditioned 1e4) beyond
+// what a result may move.
+constexpr long long F32_MAX_OBS = 1ll << 19;
+
+// The pairs of each point's observations (with the observation itself when
+// self): thread per observation q, rank a among its point's, writes pairs
+// (a, b), b > a (or >= a), the lower camera first.
+__global__ void k_pair_emit(int O, int self, const int32_t* __restrict__ rowptr_pt, const int32_t* __restrict__ poff,
+                            const int32_t* __restrict__ pm_pt, const int32_t* __restrict__ pm_cam,
+                            const int32_t* __restrict__ pm2cm, int32_t* __restrict__ ki, int32_t* __restrict__ kl,
+                            int32_t* __restrict__ sk, int32_t* __restrict__ sl) {
+  const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= O) return;
+  const int j = pm_pt[q], r0 = rowptr_pt[j], n = rowptr_pt[j + 1] - r0;
+  const long long a = q - r0;
+  // entries before rank a: sum of (n - 1 - a') (or n - a' with self)
+  long long w = poff[j] + (self ? a * n - a * (a - 1) / 2 : a * (n - 1) - a * (a - 1) / 2);
+  const int ca = pm_cam[q], s = pm2cm[q];
+  for (long long p = q + (self ? 0 : 1); p < r0 + n; ++p, ++w) {
+    const int cb = pm_cam[p], t = pm2cm[p];
+    const bool up = ca <= cb;
+    ki[w] = up ? ca : cb;
+    kl[w] = up ? cb : ca;
+    sk[w] = up ? s : t;
+    sl[w] = up ? t : s;
+  }
+}
+
+__global__ void k_pair_key(int n, const int32_t* __restrict__ perm, const int32_t* __restrict__ key,
+                           int32_t* __restrict__ out) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < n) out[e] = key[perm[e]];
+}
+
+// Entry e of the sorted order: its slots, point and cameras.
+__global__ void k_pair_gather(int n, const int32_t* __restrict__ perm_l, const int32_t* __restrict__ perm_i,
+                              const int32_t* __restrict__ ki, const int32_t* __restrict__ kl,
+                              const int32_t* __restrict__ sk, const int32_t* __restrict__ sl,
+                              const int32_t* __restrict__ cm_pt, int32_t* __restrict__ pk, int32_t* __restrict__ pl,
+                              int32_t* __restrict__ pj, int2* __restrict__ cams) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  const int p = perm_l[perm_i[e]];
+  const int s = sk[p];
+  pk[e] = s;
+  pl[e] = sl[p];
+  pj[e] = cm_pt[s];
+  cams[e] = make_int2(ki[p], kl[p]);
+}
+
+// 0 where a new camera pair begins, else 1 (a stable sort by it lists the heads).
+__global__ void k_pair_heads(int n, const int2* __restrict__ cams, int32_t* __restrict__ out) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  out[e] = e > 0 && cams[e].x == cams[e - 1].x && cams[e].y == cams[e - 1].y;
+}
+
+__global__ void k_pair_head_cams(int n, const int32_t* __restrict__ head, const int2* __restrict__ cams,
+                                 int2* __restrict__ out) {
+  const long long b = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (b < n) out[b] = cams[head[b]];
+}
+
+const void* form_kernel(bool direct, bool f32, bool mf) {
+  if (direct && f32)
+    return mf ? (const void*)k_schur_form<float, true, double> : (const void*)k_schur_form<float, false, double>;
+  if (f32) return mf ? (const void*)k_schur_form<float, true, float> : (const void*)k_schur_form<float, false, float>;
+  return mf ? (const void*)k_schur_form<double, true, double> : (const void*)k_schur_form<double, false, double>;
+}
+
+// Whether the PCG on the formed S takes less time than the implicit product
+// (us, one GB300; each constant beside what it was measured on).  An LM trial
+// at ordinary damping runs 30-80 iterations (rings of 64-4,000 cameras,
+// lambda 1e-4 to 2e-3, tol 1e-4), or maxiter: 32 are assumed.
+struct SchurCost {
+  bool f32;
+  int maxiter;
+  double iters() const { return std::min(maxiter, 32); }
+  // five launches and the passes over the observations (8.0M: 1,030 us FP64,
+  // 120 us FP32); an iteration past convergence still launches
+  double implicit_us(double O) const {
+    return iters() * (12.0 + O * (f32 ? 1.5e-5 : 1.28e-4)) + (maxiter - iters()) * 6.0;
+  }
+  // forming: FP64 pipe (13 ns per 32 pairs), FP32 arithmetic and gathers
+  double form_us(double pairs) const { return 25.0 + pairs * (f32 ? 3.0e-5 : 3.7e-4); }
+  // two exchanges, then 81 multiply-adds or 324 bytes a block
+  double iter_us(double blocks) const { return 8.0 + 162.0 * blocks * (f32 ? 0.8e-6 : 1.7e-6); }
+};
+
+}  // namespace
+
+ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
+  const bool direct = h->opt.solver == BA_SOLVER_CHOLESKY;
+  const bool f32 = h->prec == BA_PREC_F32;
+  if (h->batched) return BA_OK;
+  const int C = h->C, P = h->P, O = h->O;
+  const bool self = direct;
+  std::vector<int32_t> poff(P + 1);
+  long long np = 0;
+  for (int j = 0; j < P; ++j) {
+    const long long n = rq[j + 1] - rq[j];
+    poff[j] = (int32_t)std::min<long long>(np, INT32_MAX);
+    np += n * (n - 1) / 2 + (self ? n : 0);
+    if (np > MAX_PAIRS) return BA_OK;
+  }
+  poff[P] = (int32_t)np;
+  if (np == 0) return BA_OK;
+  const SchurCost cost{f32, h->opt.pcg_maxiter};
+  int dev = 0, nsm = 0, coop = 0;
+  SCU(cudaGetDevice(&dev));
+  SCU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  SCU(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+  int rpb = 1;
+  if (!direct) {
+    // FP64 that recomputes its Jacobians in every pass keeps the implicit
+    // product: a pair would recompute two observations in FP64
+    if (!coop || (!f32 && h->mf) || h->opt.pcg_maxiter < 1) return BA_OK;
+    if (cost.form_us((double)np) >= cost.implicit_us(O)) return BA_OK;
+    if (f32 && O > F32_MAX_OBS) return BA_OK;
+    rpb = (C + nsm - 1) / nsm;
+    if (rpb > SX_ROWS) return BA_OK;
+  }
+  cudaStream_t s = h->s;
+  const int n = (int)np;
+  std::vector<void*> tmp;  // freed on return, but for what keep() hands to the problem
+  struct Free {
+    std::vector<void*>& v;
+    ~Free() {
+      for (void* p : v) cudaFree(p);
+    }
+  } free_tmp{tmp};
+  auto grab = [&](auto** p, size_t bytes) {
+    void* v = nullptr;
+    const cudaError_t e = cudaMalloc(&v, std::max<size_t>(bytes, 16));
+    if (e == cudaSuccess) {
+      tmp.push_back(v);
+      *p = static_cast<std::remove_reference_t<decltype(**p)>*>(v);
+    }
+    return e;
+  };
+  int32_t *d_poff = nullptr, *ki = nullptr, *kl = nullptr, *sk = nullptr, *sl = nullptr, *perm_l = nullptr,
+          *perm_i = nullptr, *key = nullptr, *rows = nullptr;
+  int2* cams = nullptr;
+  void* scratch = nullptr;
+  cudaError_t e = grab(&d_poff, 4ull * (P + 1));
+  for (int32_t** p : {&ki, &kl, &sk, &sl, &perm_l, &perm_i, &key})
+    if (e == cudaSuccess) e = grab(p, 4ull * n);
+  if (e == cudaSuccess) e = grab(&rows, 4ull * (std::max(C, 2) + 1));
+  if (e == cudaSuccess) e = grab(&cams, 8ull * n);
+  if (e == cudaSuccess) e = grab((char**)&scratch, csr_scratch_bytes(n));
+  auto& x = h->sx;
+  int32_t *pk = nullptr, *pl = nullptr, *pj = nullptr;  // kept if S is formed
+  for (int32_t** p : {&pk, &pl, &pj})
+    if (e == cudaSuccess) e = grab(p, 4ull * n);
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // no room: the implicit product (or the dense build) as before
+    return BA_OK;
+  }
+  int* derr = &h->st->err;
+  SCU(cudaMemcpyAsync(d_poff, poff.data(), 4ull * (P + 1), cudaMemcpyHostToDevice, s));
+  k_pair_emit<<<nb_(O, 256), 256, 0, s>>>(O, self ? 1 : 0, h->rowptr_pt, d_poff, h->pm_pt, h->pm_cam, h->pm2cm, ki, kl,
+                                          sk, sl);
+  SCU(csr_build_async(kl, n, C, perm_l, rows, scratch, derr, s));
+  k_pair_key<<<nb_(n, 256), 256, 0, s>>>(n, perm_l, ki, key);
+  SCU(csr_build_async(key, n, C, perm_i, rows, scratch, derr, s));
+  k_pair_gather<<<nb_(n, 256), 256, 0, s>>>(n, perm_l, perm_i, ki, kl, sk, sl, h->cm_pt, pk, pl, pj, cams);
+  k_pair_heads<<<nb_(n, 256), 256, 0, s>>>(n, cams, key);
+  SCU(csr_build_async(key, n, 2, perm_l, rows, scratch, derr, s));
+  count_launch(4);
+  int32_t hrow[3];
+  SCU(cudaMemcpyAsync(hrow, rows, 12, cudaMemcpyDeviceToHost, s));
+  SCU(cudaStreamSynchronize(s));
+  const int nhead = hrow[1];
+  const size_t vs = direct || !f32 ? 8 : 4;
+  if (!direct && (cost.form_us((double)np) + cost.iters() * cost.iter_us(nhead) >= cost.implicit_us(O) ||
+                  2ull * nhead * SX_PART * vs > (16ull << 30)))
+    return BA_OK;
+  int2* d_hcam = nullptr;
+  if (grab(&d_hcam, 8ull * nhead) != cudaSuccess) {
+    cudaGetLastError();
+    return BA_OK;
+  }
+  k_pair_head_cams<<<nb_(nhead, 256), 256, 0, s>>>(nhead, perm_l, cams, d_hcam);
+  count_launch();
+  std::vector<int32_t> head(nhead);
+  std::vector<int2> hcam(nhead);
+  SCU(cudaMemcpyAsync(head.data(), perm_l, 4ull * nhead, cudaMemcpyDeviceToHost, s));
+  SCU(cudaMemcpyAsync(hcam.data(), d_hcam, 8ull * nhead, cudaMemcpyDeviceToHost, s));
+  SCU(cudaStreamSynchronize(s));
+
+  // tasks: about eight warps an SM a round and at least four rounds of lanes
+  // where there are that many pairs (a task ends with 81 x 32 additions)
+  const int seg = (int)std::min<long long>(512, std::max<long long>(32, (np / (8LL * nsm) + 31) / 32 * 32));
+  std::vector<int4> task;
+  std::vector<int2> bcam;
+  std::vector<int> btask;
+  auto block = [&](int2 c, int b0, int b1) {
+    btask.push_back((int)task.size());
+    for (int q = b0; q < b1; q += seg) task.push_back(make_int4((int)bcam.size(), q, std::min(b1, q + seg), 0));
+    bcam.push_back(c);
+  };
+  int next = 0;  // direct: every camera has a diagonal block, observed or not
+  for (int b = 0; b < nhead; ++b) {
+    if (direct)
+      for (; next <= hcam[b].x; ++next)
+        if (next < hcam[b].x || hcam[b].y != hcam[b].x) block(make_int2(next, next), 0, 0);
+    block(hcam[b], head[b], b + 1 < nhead ? head[b + 1] : n);
+  }
+  if (direct)
+    for (; next < C; ++next) block(make_int2(next, next), 0, 0);
+  btask.push_back((int)task.size());
+  const int nblk = x.nblk = (int)bcam.size();
+  x.ntask = (int)task.size();
+  auto up = [&](auto** p, const auto& v) {
+    cudaError_t r = h->alloc(p, v.size() * sizeof(v[0]));
+    if (r == cudaSuccess) r = cudaMemcpy(*p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
+    return r;
+  };
+  auto keep = [&](int32_t** dst, int32_t* p) {
+    tmp.erase(std::find(tmp.begin(), tmp.end(), (void*)p));
+    h->allocs.push_back(p);
+    *dst = p;
+  };
+  auto kernel_attr = [&](const void* k, int bytes) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  kernel_attr(form_kernel(direct, f32, h->mf), direct || !f32 ? sf_smem<double>() : sf_smem<float>());
+  if (e == cudaSuccess) e = up(&x.task, task);
+  if (e == cudaSuccess) e = up(&x.blk_cam, bcam);
+  if (e == cudaSuccess) e = up(&x.blk_task, btask);
+  if (e == cudaSuccess) e = h->alloc(&x.part, (size_t)x.ntask * SX_PART * vs);
+  if (direct) {
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return BA_OK;
+    }
+    keep(&x.pk, pk);
+    keep(&x.pl, pl);
+    keep(&x.pj, pj);
+    x.direct = true;
+    return BA_OK;
+  }
+
+  // row panels: neighbours in camera order (blocks come sorted by their lower
+  // camera, so every row meets its lower neighbours in order)
+  std::vector<int32_t> rowblk(C + 1, 0), lower(C, 0), fill(C, 0);
+  for (const int2& c : bcam) {
+    ++rowblk[c.x + 1];
+    if (c.x != c.y) {
+      ++rowblk[c.y + 1];
+      ++lower[c.y];
+    }
+  }
+  for (int i = 0; i < C; ++i) rowblk[i + 1] += rowblk[i];
+  std::vector<int32_t> col(rowblk[C]), upper(C, 0);
+  std::vector<int2> pos(nblk);
+  for (int b = 0; b < nblk; ++b) {
+    const int i = bcam[b].x, l = bcam[b].y;
+    pos[b].x = lower[i] + upper[i]++;
+    col[rowblk[i] + pos[b].x] = l;
+    pos[b].y = pos[b].x;
+    if (i != l) {
+      pos[b].y = fill[l]++;
+      col[rowblk[l] + pos[b].y] = i;
+    }
+  }
+  const int groups = (C + rpb - 1) / rpb;
+  std::vector<int32_t> list, lptr{0}, mark(C, -1), rpart{0}, pptr{0};
+  std::vector<uint16_t> colloc(col.size()), ownloc(C);
+  std::vector<int4> parts;
+  long long wmax = 1;
+  for (int g = 0; g < groups; ++g)
+    wmax = std::max<long long>(wmax, 9LL * (rowblk[std::min(C, (g + 1) * rpb)] - rowblk[g * rpb]));
+  // a warp's share: FP64 adds the lanes of a share at 17 instructions of 16
+  // cycles, so few shares, but enough loads in flight (three rows of 900
+  // columns: 27.8k cycles a product with 3 shares, 17.9k with 12, of which
+  // 14.4k are the multiply-adds); FP32 takes a share for every warp
+  const int shares = f32 ? SX_THREADS / 32 : 8;
+  const int pcol = (int)std::max<long long>(32, (wmax / shares + 31) / 32 * 32);
+  bool fits = true;
+  for (int g = 0; g < groups && fits; ++g) {
+    const int i0 = g * rpb, i1 = std::min(C, i0 + rpb);
+    const size_t l0 = list.size();
+    auto local = [&](int c) {
+      if (mark[c] < (int)l0 || mark[c] >= (int)list.size() || list[mark[c]] != c) {
+        mark[c] = (int)list.size();
+        list.push_back(c);
+      }
+      return mark[c] - (int)l0;
+    };
+    for (int i = i0; i < i1; ++i) ownloc[i] = (uint16_t)local(i);
+    for (int i = i0; i < i1; ++i) {
+      for (int q = rowblk[i]; q < rowblk[i + 1]; ++q) colloc[q] = (uint16_t)local(col[q]);
+      const int w = 9 * (rowblk[i + 1] - rowblk[i]);
+      for (int c = 0; c < w; c += pcol) parts.push_back(make_int4(i - i0, c, std::min(w, c + pcol), 0));
+      rpart.push_back((int32_t)parts.size());
+    }
+    x.nc_max = std::max(x.nc_max, (int)(list.size() - l0));
+    x.parts_max = std::max(x.parts_max, (int)parts.size() - pptr.back());
+    lptr.push_back((int32_t)list.size());
+    pptr.push_back((int32_t)parts.size());
+    fits = x.nc_max < 65536 && sx_smem(x.nc_max, x.parts_max) <= 200u * 1024u;
+  }
+  if (!fits) return BA_OK;
+  if (parts.empty()) parts.push_back(make_int4(0, 0, 0, 0));
+  const size_t smem = sx_smem(x.nc_max, x.parts_max);
+  const void* kern = f32 ? (const void*)k_schur_pcg<float> : (const void*)k_schur_pcg<double>;
+  int occ = 0;
+  SCU(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+  SCU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, SX_THREADS, smem));
+  if ((long long)occ * nsm < groups) return BA_OK;
+  x.words = sx_words(groups, C) + 1;  // and the error flag
+  if (e == cudaSuccess) e = up(&x.blk_pos, pos);
+  if (e == cudaSuccess) e = up(&x.rowblk, rowblk);
+  if (e == cudaSuccess) e = up(&x.cams, list);
+  if (e == cudaSuccess) e = up(&x.cam_ptr, lptr);
+  if (e == cudaSuccess) e = up(&x.part_ptr, pptr);
+  if (e == cudaSuccess) e = up(&x.row_part, rpart);
+  if (e == cudaSuccess) e = up(&x.colloc, colloc);
+  if (e == cudaSuccess) e = up(&x.ownloc, ownloc);
+  if (e == cudaSuccess) e = up(&x.parts, parts);
+  if (e == cudaSuccess) e = h->alloc(&x.val, (size_t)rowblk[C] * SX_PART * vs);
+  if (e == cudaSuccess) e = h->alloc(&x.gx, 8 * x.words);
+  if (e == cudaSuccess && !h->Sii) e = h->alloc(&h->Sii, 45ull * C * 8);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return BA_OK;
+  }
+  keep(&x.pk, pk);
+  keep(&x.pl, pl);
+  keep(&x.pj, pj);
+  x.groups = groups;
+  x.rpb = rpb;
+  x.pcg = true;
+  return BA_OK;
+}
+
+namespace {
+
+template <typename T, bool MF, typename ACC>
+void form(ba_problem* h) {
+  auto& x = h->sx;
+  static_assert(sizeof(ACC) >= sizeof(T), "the sums hold what the Jacobians hold");
+  k_schur_form<T, MF, ACC><<<nb_(x.ntask, SF_WARPS), 32 * SF_WARPS, sf_smem<ACC>(), h->s>>>(
+      x.ntask, x.task, x.blk_cam, x.pk, x.pl, x.pj, (const T*)h->Jcm, h->O, (const T*)h->camtab, (const T*)h->ptab,
+      (const T*)h->cm_sw, (const T*)h->Vinv, (ACC*)x.part);
+  count_launch();
+}
+
+template <typename VT>
+void pcg(ba_problem* h, int maxiter, double tol) {
+  auto& x = h->sx;
+  cudaStream_t s = h->s;
+  k_schur_combine<VT, VT><<<x.nblk, 96, 0, s>>>(x.blk_cam, x.blk_pos, x.blk_task, x.rowblk, (const VT*)x.part,
+                                                (VT*)x.val);
+  cudaMemsetAsync(x.gx, 0, 8 * x.words, s);
+  SchurPcg<VT> a;
+  a.C = h->C;
+  a.rpb = x.rpb;
+  a.rowblk = x.rowblk;
+  a.val = (const VT*)x.val;
+  a.colloc = x.colloc;
+  a.cams = x.cams;
+  a.cam_ptr = x.cam_ptr;
+  a.parts = x.parts;
+  a.part_ptr = x.part_ptr;
+  a.row_part = x.row_part;
+  a.ownloc = x.ownloc;
+  a.nc_max = x.nc_max;
+  a.Sii = h->Sii;
+  a.Minv = h->Minv;
+  a.b = h->r;
+  a.fixed = h->fixed;
+  a.x = h->x;
+  a.maxiter = maxiter;
+  a.tol = tol;
+  a.gx = GridX{x.gx, reinterpret_cast<int*>(x.gx + x.words - 1)};
+  a.st = h->st;
+  void* args[] = {&a};
+  cudaLaunchCooperativeKernel((const void*)k_schur_pcg<VT>, dim3(x.groups), dim3(SX_THREADS), args,
+                              sx_smem(x.nc_max, x.parts_max), s);
+  count_launch(2);
+}
+
+}  // namespace
+
+void schur_form(ba_problem* h) {
+  const bool f32 = h->prec == BA_PREC_F32;
+  if (h->sx.direct) {
+    if (f32) h->mf ? form<float, true, double>(h) : form<float, false, double>(h);
+    else h->mf ? form<double, true, double>(h) : form<double, false, double>(h);
+  } else if (f32) {
+    h->mf ? form<float, true, float>(h) : form<float, false, float>(h);
+  } else {
+    form<double, false, double>(h);
+  }
+}
+
+void schur_to_band(ba_problem* h, const double* lam_ptr) {
+  auto& x = h->sx;
+  k_schur_band<<<x.nblk, 96, 0, h->s>>>(x.blk_cam, x.blk_task, (const double*)x.part, h->U, lam_ptr, h->opt.diag_min,
+                                        h->opt.diag_max, h->fixed, h->bwt, h->bT);
+  count_launch();
+}
+
+void schur_pcg(ba_problem* h, int maxiter, double tol) {
+  if (h->prec == BA_PREC_F32) pcg<float>(h, maxiter, tol);
+  else pcg<double>(h, maxiter, tol);
+}
+
+}  // namespace ba
