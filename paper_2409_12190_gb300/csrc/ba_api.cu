@@ -146,7 +146,7 @@ void enqueue_lin(ba_problem* h, int gate) {
   }
   {
     Prof pr(h, BA_K_OTHER, -2);
-    k_cam_combine_lin<<<nblk(h->C, 128), 128, 0, s>>>(h->C, h->cam_piece_ptr, h->part, h->st, gate,
+    k_cam_combine_lin<<<nblk(54LL * h->C, 128), 128, 0, s>>>(h->C, h->cam_piece_ptr, h->part, h->st, gate,
                                                       h->xch ? h->U_loc : h->U, h->xch ? h->gc_loc : h->gc);
   }
   if (h->xch) {
@@ -342,7 +342,7 @@ void enqueue_solve(ba_problem* h, const double* lam_ptr, int maxiter, double tol
   {
     Prof pr(h, BA_K_OTHER);
     k_pt_damp<T><<<nblk(h->P, PT_THREADS), PT_THREADS, 0, s>>>(h->P, h->V, h->gp, lam_ptr, dmin, dmax,
-                                                              (T*)h->Vinv, (T*)h->y0);
+                                                              (T*)h->Vinv, (T*)h->y0, h->st);
   }
   {
     Prof pr(h, BA_K_SCHUR_CAM);
@@ -360,11 +360,17 @@ void enqueue_solve(ba_problem* h, const double* lam_ptr, int maxiter, double tol
     sptr = h->ident_ptr;
     spart = h->camsum;
   }
-  {
+  if (h->sx.pcg && !h->xch && !learned && h->C <= CAM_WARP_MAX) {
     Prof pr(h, BA_K_OTHER);
-    k_cam_combine_schur<T, MF><<<h->ncb, CAM_THREADS, 0, s>>>(
-        h->C, sptr, spart, h->U, h->gc, (const T*)h->camtab, lam_ptr, dmin, dmax, h->Minv, h->x,
-        h->r, h->z, h->p, (T*)h->pT, h->dot_rz + h->ncb, h->dot_bb, h->fixed, h->st, learned || h->sx.pcg ? h->Sii : nullptr);
+    k_cam_schur_warp<<<h->C, 32, 0, s>>>(h->C, sptr, spart, h->U, h->gc, lam_ptr, dmin, dmax, h->fixed, h->Minv, h->x,
+                                         h->r, h->Sii, h->st);
+  } else {
+  {
+      Prof pr(h, BA_K_OTHER);
+      k_cam_combine_schur<T, MF><<<h->ncb, CAM_THREADS, 0, s>>>(
+          h->C, sptr, spart, h->U, h->gc, (const T*)h->camtab, lam_ptr, dmin, dmax, h->Minv, h->x,
+          h->r, h->z, h->p, (T*)h->pT, h->dot_rz + h->ncb, h->dot_bb, h->fixed, h->st, learned || h->sx.pcg ? h->Sii : nullptr);
+    }
   }
   count_launch(3);
   if (learned) {
@@ -538,7 +544,7 @@ void enqueue_matvec(ba_problem* h, const double* lam_ptr) {
   cudaStream_t s = h->s;
   const double dmin = h->opt.diag_min, dmax = h->opt.diag_max;
   k_pt_damp<T><<<nblk(h->P, PT_THREADS), PT_THREADS, 0, s>>>(h->P, h->V, h->gp, lam_ptr, dmin, dmax, (T*)h->Vinv,
-                                                            (T*)h->y0);
+                                                            (T*)h->y0, h->st);
   k_pass_vec<T, MF><<<nblk(h->C, 128), 128, 0, s>>>(h->C, h->p, (const T*)h->camtab, (T*)h->pT);
   enqueue_schur_product<T, MF>(h, (const T*)h->pT, -1, 0);
   k_pcg_q<T, MF><<<h->ncb, VT, 0, s>>>(h->C, h->cam_piece_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr,
@@ -654,31 +660,6 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
     CU(e);
   }
 
-  // pieces: each camera's slots cut into runs of at most PIECE
-  std::vector<int32_t> rp(C + 1);
-  CU(cudaMemcpy(rp.data(), h->rowptr_cam, (C + 1) * 4, cudaMemcpyDeviceToHost));
-  std::vector<int32_t> pc, pb, pe, cpp(C + 1);
-  for (long long c = 0; c < C; ++c) {
-    cpp[c] = (int32_t)pc.size();
-    const int n = rp[c + 1] - rp[c];
-    const int k = (n + PIECE - 1) / PIECE;
-    for (int i = 0; i < k; ++i) {
-      pc.push_back((int32_t)c);
-      pb.push_back(rp[c] + (int)((long long)n * i / k));
-      pe.push_back(rp[c] + (int)((long long)n * (i + 1) / k));
-    }
-  }
-  cpp[C] = (int32_t)pc.size();
-  h->npieces = (int)pc.size();
-  CU(h->alloc(&h->piece_cam, pc.size() * 4));
-  CU(h->alloc(&h->piece_beg, pc.size() * 4));
-  CU(h->alloc(&h->piece_end, pc.size() * 4));
-  CU(h->alloc(&h->cam_piece_ptr, (C + 1) * 4));
-  CU(cudaMemcpy(h->piece_cam, pc.data(), pc.size() * 4, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(h->piece_beg, pb.data(), pb.size() * 4, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(h->piece_end, pe.data(), pe.size() * 4, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(h->cam_piece_ptr, cpp.data(), (C + 1) * 4, cudaMemcpyHostToDevice));
-
   // point chunks: runs of whole points with at most CHUNK_SLOTS observations
   // and CHUNK_PTS points (a point with more observations is a chunk alone)
   std::vector<int32_t> rq(P + 1), pch;
@@ -770,6 +751,50 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
     }
   }
 
+  {
+    const ba_status sb = schur_build(h, rq);
+    if (sb != BA_OK) return sb;
+  }
+
+  // pieces: each camera's slots cut into runs of at most piece_max.  The
+  // camera passes of one linearisation are then all a trial runs over the
+  // pieces when S is formed, one block of 64 threads each: about six blocks
+  // an SM keep the FP64 pipes busy (16 cameras: 16 pieces of 500 slots took
+  // 100 us a pass, 250 cameras: 250 pieces 375 us, twice what its arithmetic
+  // takes).  The implicit product runs over them in every iteration and adds a
+  // reduction for each: as long as they may be.
+  int piece_max = PIECE;
+  if (h->sx.pcg || h->sx.direct) {
+    int dev = 0, nsm = 1;
+    CU(cudaGetDevice(&dev));
+    CU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+    const long long per = O / (6LL * nsm);
+    piece_max = (int)std::min<long long>(PIECE, std::max<long long>(LIN_THREADS, (per + LIN_THREADS - 1) / LIN_THREADS * LIN_THREADS));
+  }
+  std::vector<int32_t> rp(C + 1);
+  CU(cudaMemcpy(rp.data(), h->rowptr_cam, (C + 1) * 4, cudaMemcpyDeviceToHost));
+  std::vector<int32_t> pc, pb, pe, cpp(C + 1);
+  for (long long c = 0; c < C; ++c) {
+    cpp[c] = (int32_t)pc.size();
+    const int n = rp[c + 1] - rp[c];
+    const int k = (n + piece_max - 1) / piece_max;
+    for (int i = 0; i < k; ++i) {
+      pc.push_back((int32_t)c);
+      pb.push_back(rp[c] + (int)((long long)n * i / k));
+      pe.push_back(rp[c] + (int)((long long)n * (i + 1) / k));
+    }
+  }
+  cpp[C] = (int32_t)pc.size();
+  h->npieces = (int)pc.size();
+  CU(h->alloc(&h->piece_cam, pc.size() * 4));
+  CU(h->alloc(&h->piece_beg, pc.size() * 4));
+  CU(h->alloc(&h->piece_end, pc.size() * 4));
+  CU(h->alloc(&h->cam_piece_ptr, (C + 1) * 4));
+  CU(cudaMemcpy(h->piece_cam, pc.data(), pc.size() * 4, cudaMemcpyHostToDevice));
+  CU(cudaMemcpy(h->piece_beg, pb.data(), pb.size() * 4, cudaMemcpyHostToDevice));
+  CU(cudaMemcpy(h->piece_end, pe.data(), pe.size() * 4, cudaMemcpyHostToDevice));
+  CU(cudaMemcpy(h->cam_piece_ptr, cpp.data(), (C + 1) * 4, cudaMemcpyHostToDevice));
+
   // linearisation and solver buffers
   CU(h->alloc(&h->camtab, CT * C * ts));
   CU(h->alloc(&h->ptab, 8 * P * ts));
@@ -804,10 +829,6 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
   CU(h->alloc(&h->dp, 3 * P * ts));
   CU(h->alloc(&h->part, (size_t)PART * std::max(h->npieces, 1) * 8));
   h->ncb = (int)nblk(C, CAM_THREADS);
-  {
-    const ba_status sb = schur_build(h, rq);
-    if (sb != BA_OK) return sb;
-  }
   if (h->opt.solver == BA_SOLVER_CHOLESKY) {
     // the direct solve: the band tiles of the whole lower triangle; the
     // factorisation's task list (ba_band_sched.h) for one block per SM; where
@@ -943,7 +964,7 @@ void enqueue_collect(ba_problem* h, const double* lam_ptr, int K, const float* z
   const double dmin = h->opt.diag_min, dmax = h->opt.diag_max;
   enqueue_lin<T, MF>(h, 1);
   k_pt_damp<T><<<nblk(h->P, PT_THREADS), PT_THREADS, 0, s>>>(h->P, h->V, h->gp, lam_ptr, dmin, dmax, (T*)h->Vinv,
-                                                            (T*)h->y0);
+                                                            (T*)h->y0, h->st);
   k_schur_cam<T, MF><<<h->npieces, LIN_THREADS, 0, s>>>(
       h->piece_cam, h->piece_beg, h->piece_end, h->cm_pt, (const T*)h->Jcm, (const T*)h->camtab, (const T*)h->pts,
       (const T*)h->cm_sw, h->st, h->P, (const T*)h->Vinv, (const T*)h->y0, h->O, h->part);

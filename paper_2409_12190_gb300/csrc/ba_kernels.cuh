@@ -229,6 +229,19 @@ __device__ __forceinline__ void warp_rs64_ff(const float (&v)[64], float& h0, fl
   l1 = l[1];
 }
 
+// A step of the reduce-scatter of doubles: lanes with bit OFF keep the upper
+// N of 2 N values.
+template <int N, int OFF>
+__device__ __forceinline__ void rs_d_step(double (&h)[32], int lane) {
+  const bool up = (lane & OFF) != 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const double k = up ? h[N + i] : h[i];
+    const double g = up ? h[i] : h[N + i];
+    h[i] = k + __shfl_xor_sync(0xffffffffu, g, OFF);
+  }
+}
+
 // Sum NV per-thread values over the block and write them to out (NV
 // doubles), warps then the warps in order.  Doubles are reduced in double.
 // blockDim.x <= 1024.
@@ -242,10 +255,28 @@ __device__ __forceinline__ void block_sum_store(double (&v)[NV], double* __restr
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int nw = (blockDim.x + 31) >> 5;
+  if constexpr (NV > 32 && NV <= 64) {
+    // the same sums (warp_sum's tree) by a reduce-scatter: 62 additions a
+    // lane instead of 5 NV (FP64 takes 16 cycles a warp instruction)
+    double h[32];
+    const bool up = (lane & 16) != 0;
 #pragma unroll
-  for (int i = 0; i < NV; ++i) {
-    const double s = warp_sum(v[i]);
-    if (lane == 0) red[warp][i] = s;
+    for (int i = 0; i < 32; ++i) {
+      const double lo = v[i], hi = 32 + i < NV ? v[32 + i < NV ? 32 + i : 0] : 0.0;
+      h[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, 16);
+    }
+    rs_d_step<16, 8>(h, lane);
+    rs_d_step<8, 4>(h, lane);
+    rs_d_step<4, 2>(h, lane);
+    rs_d_step<2, 1>(h, lane);
+    if (2 * lane < NV) red[warp][2 * lane] = h[0];
+    if (2 * lane + 1 < NV) red[warp][2 * lane + 1] = h[1];
+  } else {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const double s = warp_sum(v[i]);
+      if (lane == 0) red[warp][i] = s;
+    }
   }
   __syncthreads();
   for (int i = threadIdx.x; i < NV; i += blockDim.x) {
@@ -933,14 +964,21 @@ __device__ __forceinline__ void cam_combine_lin_one(int p0, int p1, const double
   }
 }
 
-// Add the pieces of each camera in order: U [C][45], gc [C][9].
+// Add the pieces of each camera in order: U [C][45], gc [C][9]; a thread per
+// value (a thread per camera took 16 us whatever C: 54 sums one after the
+// other).
 static __global__ void k_cam_combine_lin(int C, const int32_t* __restrict__ cam_piece_ptr,
                                   const double* __restrict__ part, const DevState* __restrict__ st,
                                   int gate, double* __restrict__ U, double* __restrict__ gc) {
   if (gate && !st->need_lin) return;
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= C) return;
-  cam_combine_lin_one(cam_piece_ptr[c], cam_piece_ptr[c + 1], part, U + 45LL * c, gc + 9LL * c);
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= 54LL * C) return;
+  const int c = (int)(t / 54), i = (int)(t % 54);
+  double s = 0.0;
+  const int p1 = cam_piece_ptr[c + 1];
+  for (int p = cam_piece_ptr[c]; p < p1; ++p) s += part[(long long)PART * p + i];
+  if (i < 45) U[45LL * c + i] = s;
+  else gc[9LL * c + i - 45] = s;
 }
 
 // Point-major pass over one chunk of points: V (6) and gp (3) per point,
@@ -1107,8 +1145,9 @@ __device__ __forceinline__ void pt_damp_one(int j, const double* __restrict__ V,
 template <typename T>
 static __global__ void k_pt_damp(int P, const double* __restrict__ V, const double* __restrict__ gp,
                           const double* __restrict__ lam_ptr, double dmin, double dmax,
-                          T* __restrict__ Vinv, T* __restrict__ y0) {
+                          T* __restrict__ Vinv, T* __restrict__ y0, DevState* __restrict__ st) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j == 0) st->fallbacks = 0;  // counted by the camera kernels of this solve
   if (j >= P) return;
   pt_damp_one<T>(j, V, gp, *lam_ptr, dmin, dmax, Vinv, y0);
 }
@@ -1430,7 +1469,6 @@ k_cam_combine_schur(int C, const int32_t* __restrict__ cam_piece_ptr, const doub
     st->pcg_done = 0;
     st->pcg_iters = 0;
     st->pcg_rel = 1.0;
-    st->fallbacks = 0;
   }
   if (c < C) {
     int fb;
@@ -1446,6 +1484,109 @@ k_cam_combine_schur(int C, const int32_t* __restrict__ cam_piece_ptr, const doub
   if (threadIdx.x == 0) {
     dot_rz1[blockIdx.x] = v[0];
     dot_bb[blockIdx.x] = v[1];
+  }
+}
+
+// The same for the PCG on the formed S, one warp per camera: the pieces summed
+// a value a lane, the 9 x 9 factorisation and inverse over the lanes.  Writes
+// S_ii, M_i, x = 0 and r = b.  A thread per camera (above) runs its 2,000
+// serial FP64 instructions in 35 us at any C up to some thousands; a warp per
+// camera takes 7 us a camera of an SM, so it is used up to CAM_WARP_MAX.
+constexpr int CAM_WARP_MAX = 608;
+static __global__ void __launch_bounds__(32)
+k_cam_schur_warp(int C, const int32_t* __restrict__ cam_piece_ptr, const double* __restrict__ part,
+                 const double* __restrict__ U, const double* __restrict__ gc, const double* __restrict__ lam_ptr,
+                 double dmin, double dmax, const uint8_t* __restrict__ fixed, double* __restrict__ Minv,
+                 double* __restrict__ x, double* __restrict__ r, double* __restrict__ Sii, DevState* st) {
+  __shared__ double A[9][10], Li[9][10], bv[9], inv[9];
+  const int c = blockIdx.x, lane = threadIdx.x;
+  const double lam = *lam_ptr;
+  const double* Uc = U + 45LL * c;
+  if (c == 0 && lane == 0) {
+    st->pcg_done = 0;
+    st->pcg_iters = 0;
+    st->pcg_rel = 1.0;
+  }
+  // this lane's entries (i, j), j >= i, of the packed upper triangle
+  int ei[2], ej[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    int e = lane + 32 * u, i = 0;
+    while (i < 8 && e >= 9 - i) e -= 9 - i++;
+    ei[u] = i;
+    ej[u] = i + e;
+  }
+  const int p0 = cam_piece_ptr[c], p1 = cam_piece_ptr[c + 1];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int e = lane + 32 * u;
+    if (e >= 54) continue;
+    double v;
+    if (e < 45) {
+      v = Uc[e];
+      if (ei[u] == ej[u]) v += damp(v, lam, dmin, dmax);
+      for (int q = p0; q < p1; ++q) v -= part[(long long)PART * q + e];
+      if (fixed && (fixed[9LL * c + ei[u]] || fixed[9LL * c + ej[u]])) v = ei[u] == ej[u] ? 1.0 : 0.0;
+      Sii[45LL * c + e] = v;
+      A[ej[u]][ei[u]] = v;  // lower triangle
+    } else {
+      v = -gc[9LL * c + e - 45];
+      for (int q = p0; q < p1; ++q) v += part[(long long)PART * q + e];
+      if (fixed && fixed[9LL * c + e - 45]) v = 0.0;
+      bv[e - 45] = v;
+    }
+  }
+  __syncwarp();
+  bool spd = true;
+#pragma unroll 1
+  for (int j = 0; j < 9; ++j) {
+    const double d = A[j][j];
+    if (!(d > 0.0) || !isfinite(d)) {
+      spd = false;
+      break;
+    }
+    const double ljj = sqrt(d), il = 1.0 / ljj;
+    __syncwarp();
+    if (lane == j) A[j][j] = ljj;
+    if (lane > j && lane < 9) A[lane][j] *= il;
+    __syncwarp();
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+      if (lane + 32 * u < 45 && ei[u] > j) A[ej[u]][ei[u]] -= A[ej[u]][j] * A[ei[u]][j];
+    __syncwarp();
+  }
+  if (spd) {
+    if (lane < 9) inv[lane] = 1.0 / A[lane][lane];
+    __syncwarp();
+    if (lane < 9) {  // column `lane` of L^{-1}
+      for (int i = 0; i < lane; ++i) Li[i][lane] = 0.0;
+      Li[lane][lane] = inv[lane];
+      for (int i = lane + 1; i < 9; ++i) {
+        double s = 0.0;
+        for (int k = lane; k < i; ++k) s += A[i][k] * Li[k][lane];
+        Li[i][lane] = -s * inv[i];
+      }
+    }
+    __syncwarp();
+  } else if (lane == 0) {
+    atomicAdd(&st->fallbacks, 1);
+  }
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int e = lane + 32 * u;
+    if (e >= 45) continue;
+    double m = 0.0;
+    if (spd) {
+      for (int k = ej[u]; k < 9; ++k) m += Li[k][ei[u]] * Li[k][ej[u]];
+    } else if (ei[u] == ej[u]) {
+      // not SPD in this precision: the inverse diagonal of U*
+      m = 1.0 / (Uc[e] + damp(Uc[e], lam, dmin, dmax));
+    }
+    Minv[45LL * c + e] = m;
+  }
+  if (lane < 9) {
+    x[9LL * c + lane] = 0.0;
+    r[9LL * c + lane] = bv[lane];
   }
 }
 

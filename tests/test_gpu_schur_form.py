@@ -103,3 +103,36 @@ def test_unobserved_camera_in_the_direct_solve():
     with problem(sc, pix, "f64", solver="cholesky") as prob:
         dc = np64(prob.damped_solve(1e-2, 0, 0.0)[0])
     assert np.all(dc[5] == 0.0) and rel_err(dc, dc_ref) < 1e-9
+
+
+def test_solves_on_two_streams_at_once():
+    """Two problems solved at the same time, each on a stream and thread of its
+    own, give the bits that they give alone."""
+    import threading
+
+    scs = [_ragged(160, 2000, seed=5), _ragged(60, 3000, seed=6)]
+    pix = [orc.pixels_from_scene(sc) for sc in scs]
+    alone = []
+    for sc, px in zip(scs, pix):
+        with problem(sc, px, "f64", pcg_maxiter=40) as prob:
+            prob.solve(6)
+            alone.append(prob.params())
+    probs = [problem(sc, px, "f64", pcg_maxiter=40) for sc, px in zip(scs, pix)]
+    torch.cuda.synchronize()
+
+    def work(prob):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(6):
+                prob.solve(1)
+
+    threads = [threading.Thread(target=work, args=(p,)) for p in probs]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    for prob, want in zip(probs, alone):
+        got = prob.params()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+        prob.close()
