@@ -132,7 +132,8 @@ void enqueue_lin(ba_problem* h, int gate) {
   const T delta = (T)(h->opt.huber_delta > 0 ? h->opt.huber_delta : 0.0);
   {
     Prof pr(h, BA_K_OTHER, -2);
-    k_cam_prep<T><<<nblk(h->C, 128), 128, 0, s>>>(h->C, (const T*)h->cams, h->st, gate, (T*)h->camtab);
+    k_cam_prep<T><<<nblk(h->C, 128), 128, 0, s>>>(h->C, (const T*)h->cams, h->st, gate, (T*)h->camtab,
+                                                  h->sx.lean_marked);
   }
   {
     Prof pr(h, BA_K_OTHER, -2);
@@ -140,9 +141,13 @@ void enqueue_lin(ba_problem* h, int gate) {
   }
   {
     Prof pr(h, BA_K_LIN_CAM, -2);
-    k_lin_cam<T, !MF><<<h->npieces, LIN_THREADS, 0, s>>>(
+    auto lin = k_lin_cam<T, !MF>;
+    if constexpr (!MF && std::is_same<T, double>::value)
+      if (h->sx.lean) lin = k_lin_cam<T, true, true>;
+    lin<<<h->npieces, LIN_THREADS, 0, s>>>(
         h->piece_cam, h->piece_beg, h->piece_end, h->cm_pt, (const T*)h->cm_px, (const T*)h->pts,
-        (const T*)h->camtab, h->st, gate, delta, h->O, h->P, (T*)h->Jcm, (T*)h->cm_sw, h->part);
+        (const T*)h->camtab, h->st, gate, delta, h->O, h->P, (T*)h->Jcm, (T*)h->cm_sw, h->part,
+        (T*)h->sx.lean_w, h->sx.lean_marked);
   }
   {
     Prof pr(h, BA_K_OTHER, -2);
@@ -346,9 +351,13 @@ void enqueue_solve(ba_problem* h, const double* lam_ptr, int maxiter, double tol
   }
   {
     Prof pr(h, BA_K_SCHUR_CAM);
-    k_schur_cam<T, MF><<<h->npieces, LIN_THREADS, 0, s>>>(
+    auto sc = k_schur_cam<T, MF>;
+    if constexpr (!MF && std::is_same<T, double>::value)
+      if (h->sx.lean) sc = k_schur_cam<T, false, true>;
+    sc<<<h->npieces, LIN_THREADS, 0, s>>>(
         h->piece_cam, h->piece_beg, h->piece_end, h->cm_pt, (const T*)h->Jcm, (const T*)h->camtab,
-        (const T*)h->pts, (const T*)h->cm_sw, h->st, h->P, (const T*)h->Vinv, (const T*)h->y0, h->O, h->part);
+        (const T*)h->pts, (const T*)h->cm_sw, h->st, h->P, (const T*)h->Vinv, (const T*)h->y0, h->O, h->part,
+        (T*)h->sx.lean_t);
   }
   const int32_t* sptr = h->cam_piece_ptr;
   const double* spart = h->part;
@@ -802,8 +811,10 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
   if (!h->mf) {
     CU(h->alloc(&h->Jcm, (size_t)NPLANE * O * ts));
     if (h->fa) {
-      // the planes in point-major order for the fused stored pass A
-      CU(h->alloc(&h->Jpm, (size_t)NPLANE * O * ts));
+      // the planes in point-major order for the fused stored pass A; where S
+      // is formed its few implicit products take passes A1 and A2 instead (a
+      // copy of the planes costs each linearisation what one product saves)
+      if (!h->sx.pcg && !h->sx.direct) CU(h->alloc(&h->Jpm, (size_t)NPLANE * O * ts));
       if (fs_smem<T>(FA_CAMS) > 48 * 1024)
         CU(cudaFuncSetAttribute(k_pass_fs<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, fs_smem<T>(FA_CAMS)));
     }
@@ -967,7 +978,7 @@ void enqueue_collect(ba_problem* h, const double* lam_ptr, int K, const float* z
                                                             (T*)h->y0, h->st);
   k_schur_cam<T, MF><<<h->npieces, LIN_THREADS, 0, s>>>(
       h->piece_cam, h->piece_beg, h->piece_end, h->cm_pt, (const T*)h->Jcm, (const T*)h->camtab, (const T*)h->pts,
-      (const T*)h->cm_sw, h->st, h->P, (const T*)h->Vinv, (const T*)h->y0, h->O, h->part);
+      (const T*)h->cm_sw, h->st, h->P, (const T*)h->Vinv, (const T*)h->y0, h->O, h->part, nullptr);
   k_cam_combine_schur<T, MF><<<h->ncb, CAM_THREADS, 0, s>>>(
       h->C, h->cam_piece_ptr, h->part, h->U, h->gc, (const T*)h->camtab, lam_ptr, dmin, dmax, h->Minv, h->x, h->r,
       h->z, h->p, (T*)h->pT, h->dot_rz + h->ncb, h->dot_bb, h->fixed, h->st, h->Sii);
@@ -1645,6 +1656,8 @@ ba_status ba_set_exchange(ba_problem* h, ba_exchange_fn fn, void* ctx, double* x
     CU(h->alloc(&h->gc_loc, 9ull * h->C * 8));
     CU(h->alloc(&h->xscal, 8 * 8));
   }
+  // a part's PCG runs the implicit product: its fused pass A
+  if (fn && !h->mf && h->fa && !h->Jpm) CU(h->alloc(&h->Jpm, (size_t)NPLANE * h->O * h->tsize));
   CU(cudaStreamSynchronize(h->s));
   h->xch = fn;
   h->xctx = ctx;

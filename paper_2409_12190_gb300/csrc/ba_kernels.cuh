@@ -796,9 +796,10 @@ static __global__ void k_project(int O, const T* __restrict__ cams, const T* __r
 
 template <typename T>
 static __global__ void k_cam_prep(int C, const T* __restrict__ cams_buf, const DevState* __restrict__ st,
-                           int gate, T* __restrict__ camtab) {
+                           int gate, T* __restrict__ camtab, int* __restrict__ lean_marked) {
   if (gate && !st->need_lin) return;
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c == 0 && lean_marked) *lean_marked = 0;
   if (c >= C) return;
   camera_table(cams_buf + (long long)st->cur * 9 * C + 9LL * c, camtab + (long long)CT * c);
 }
@@ -891,14 +892,50 @@ static __global__ void k_compose_perm(int O, const int32_t* __restrict__ perm_a,
   if (s < O) out[s] = inv_b[perm_a[s]];
 }
 
+// The lean form of an observation's block W = Jc^T Jp, for forming S.  With
+// M = [A_0 A_1; A_1 A_4] (d pi / d p with the depth and weight), A = M [I | p]
+// and d p along p an eigenvector, M p = mu p, so
+//   Jc = M [ [I | p] (-[RX]_x) J_l | [I | p] | p q'^T ],  q' = q / mu,
+//   W  = Jc'^T (M^T Jp),
+// Jc' without M: eight numbers (RX, p, q') and the six of M^T Jp.  It needs mu
+// away from 0 (where the distortion folds the image plane; the tangential
+// eigenvalue is A_0 + A_4 - mu): below an eighth of the other the observation
+// is marked, q'_0 = NaN, and takes the planes instead.
+// Planes in pairs: (RX0, RX1) (RX2, p0) (p1, q'0) (q'1, q'2), then M^T Jp (3).
+constexpr int NLEAN = 14;
+template <typename T>
+__device__ __forceinline__ bool lean_obs(const Fac<T>& o, const T (&pl)[NPLANE], T (&v)[NLEAN]) {
+  const T r2 = o.px * o.px + o.py * o.py;
+  const T m = o.A[2] * o.px + o.A[5] * o.py;  // mu r2
+  const T im = r2 > T(0) ? r2 / m : T(0);     // 1 / mu (p = 0: p q' = 0 whatever q')
+  const T mu = r2 > T(0) ? m / r2 : o.A[0];
+  const bool ok = fabs(mu) >= T(0.125) * fabs(o.A[0] + o.A[4] - mu);
+  v[0] = o.RX0;
+  v[1] = o.RX1;
+  v[2] = o.RX2;
+  v[3] = o.px;
+  v[4] = o.py;
+  v[5] = ok ? o.q0 * im : T(nan(""));
+  v[6] = o.q1 * im;
+  v[7] = o.q2 * im;
+  const T* Jp = pl + NPLANE_JC;
+#pragma unroll
+  for (int j = 0; j < 3; ++j) {
+    v[8 + j] = o.A[0] * Jp[j] + o.A[1] * Jp[3 + j];
+    v[11 + j] = o.A[1] * Jp[j] + o.A[4] * Jp[3 + j];
+  }
+  return ok;
+}
+
 // Camera-major slots [beg, end) of one camera, NT threads striding: residuals,
 // weights and the per-thread partial U (45) and gc (9); in the stored mode
 // also the planes, in any mode sqrt(w) when sw_out is given.
-template <typename T, bool STORE, int NT>
+template <typename T, bool STORE, int NT, bool LEAN = false>
 __device__ __forceinline__ void lin_cam_range(int beg, int end, const int32_t* __restrict__ cm_pt,
                                               const T* __restrict__ cm_px, const T* __restrict__ pts,
                                               const T* __restrict__ sct, T delta, int O, T* __restrict__ Jcm,
-                                              T* __restrict__ sw_out, T (&acc)[54]) {
+                                              T* __restrict__ sw_out, T (&acc)[54], T* __restrict__ lean = nullptr,
+                                              int* __restrict__ lean_marked = nullptr) {
   for (int s = beg + threadIdx.x; s < end; s += NT) {
     const int j = cm_pt[s];
     Fac<T> o;
@@ -918,6 +955,18 @@ __device__ __forceinline__ void lin_cam_range(int beg, int end, const int32_t* _
         reinterpret_cast<V2*>(Jcm)[(long long)q * O + s] = v;
       }
     }
+    if constexpr (LEAN) {
+      using V2 = typename Vec2<T>::type;
+      T v[NLEAN];
+      if (!lean_obs(o, pl, v)) *lean_marked = 1;
+#pragma unroll
+      for (int q = 0; q < NLEAN / 2; ++q) {
+        V2 w;
+        w.x = v[2 * q];
+        w.y = v[2 * q + 1];
+        reinterpret_cast<V2*>(lean)[(long long)q * O + s] = w;
+      }
+    }
     T j0[9], j1[9];
     jc_rows(pl, j0, j1);
 #pragma unroll
@@ -931,13 +980,13 @@ __device__ __forceinline__ void lin_cam_range(int beg, int end, const int32_t* _
 
 // Camera-major pass: residuals, weights, U (45) and gc (9) per piece; in the
 // stored mode also the planes, in any mode sqrt(w) when sw_out is given.
-template <typename T, bool STORE>
+template <typename T, bool STORE, bool LEAN = false>
 static __global__ void __launch_bounds__(LIN_THREADS)
 k_lin_cam(const int32_t* __restrict__ piece_cam, const int32_t* __restrict__ piece_beg,
           const int32_t* __restrict__ piece_end, const int32_t* __restrict__ cm_pt,
           const T* __restrict__ cm_px, const T* __restrict__ pts_buf, const T* __restrict__ camtab,
           const DevState* __restrict__ st, int gate, T delta, int O, int P, T* __restrict__ Jcm,
-          T* __restrict__ sw_out, double* __restrict__ part) {
+          T* __restrict__ sw_out, double* __restrict__ part, T* __restrict__ lean, int* __restrict__ lean_marked) {
   if (gate && !st->need_lin) return;
   __shared__ T sct[CT];
   const int b = blockIdx.x;
@@ -948,8 +997,8 @@ k_lin_cam(const int32_t* __restrict__ piece_cam, const int32_t* __restrict__ pie
   T acc[54];
 #pragma unroll
   for (int i = 0; i < 54; ++i) acc[i] = T(0);
-  lin_cam_range<T, STORE, LIN_THREADS>(piece_beg[b], piece_end[b], cm_pt, cm_px, pts, sct, delta, O, Jcm, sw_out,
-                                         acc);
+  lin_cam_range<T, STORE, LIN_THREADS, LEAN>(piece_beg[b], piece_end[b], cm_pt, cm_px, pts, sct, delta, O, Jcm, sw_out,
+                                             acc, lean, lean_marked);
   block_sum_store<54>(acc, part + (long long)PART * b);
 }
 
@@ -1168,12 +1217,12 @@ __device__ __forceinline__ void cm_planes(const T* __restrict__ Jcm, long long O
 
 // Camera-major slots [beg, end), NT threads striding: per-thread partial
 // sum_k Jc^T (Jp V*^{-1} Jp^T) Jc (45) and sum_k Jc^T Jp y0 (9).
-template <typename T, bool MF, int NT>
+template <typename T, bool MF, int NT, bool LEAN = false>
 __device__ __forceinline__ void schur_cam_range(int beg, int end, const int32_t* __restrict__ cm_pt,
                                                 const T* __restrict__ Jcm, const T* __restrict__ sct,
                                                 const T* __restrict__ pts, const T* __restrict__ cm_sw,
                                                 const T* __restrict__ Vinv, const T* __restrict__ y0, int O,
-                                                T (&acc)[54]) {
+                                                T (&acc)[54], T* __restrict__ lean_t = nullptr) {
   for (int s = beg + threadIdx.x; s < end; s += NT) {
     const int j = cm_pt[s];
     T pl[NPLANE];
@@ -1187,6 +1236,23 @@ __device__ __forceinline__ void schur_cam_range(int beg, int end, const int32_t*
       t[3 * a] = Jp[3 * a] * v00 + Jp[3 * a + 1] * v01 + Jp[3 * a + 2] * v02;
       t[3 * a + 1] = Jp[3 * a] * v01 + Jp[3 * a + 1] * v11 + Jp[3 * a + 2] * v12;
       t[3 * a + 2] = Jp[3 * a] * v02 + Jp[3 * a + 1] * v12 + Jp[3 * a + 2] * v22;
+    }
+    if constexpr (LEAN) {
+      // M^T Jp V*^{-1} of the lean form (M = [A_0 A_1; A_1 A_4])
+      using V2 = typename Vec2<T>::type;
+      T w[6];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        w[c] = pl[0] * t[c] + pl[1] * t[3 + c];
+        w[3 + c] = pl[1] * t[c] + pl[4] * t[3 + c];
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        V2 v;
+        v.x = w[2 * q];
+        v.y = w[2 * q + 1];
+        reinterpret_cast<V2*>(lean_t)[(long long)q * O + s] = v;
+      }
     }
     const T m00 = t[0] * Jp[0] + t[1] * Jp[1] + t[2] * Jp[2];
     const T m01 = t[0] * Jp[3] + t[1] * Jp[4] + t[2] * Jp[5];
@@ -1210,13 +1276,13 @@ __device__ __forceinline__ void schur_cam_range(int beg, int end, const int32_t*
 
 // Camera-major pass: per piece, sum_k Jc^T (Jp V*^{-1} Jp^T) Jc (45) and
 // sum_k Jc^T Jp y0 (9).
-template <typename T, bool MF>
+template <typename T, bool MF, bool LEAN = false>
 static __global__ void __launch_bounds__(LIN_THREADS)
 k_schur_cam(const int32_t* __restrict__ piece_cam, const int32_t* __restrict__ piece_beg,
             const int32_t* __restrict__ piece_end, const int32_t* __restrict__ cm_pt,
             const T* __restrict__ Jcm, const T* __restrict__ camtab, const T* __restrict__ pts_buf,
             const T* __restrict__ cm_sw, const DevState* __restrict__ st, int P, const T* __restrict__ Vinv,
-            const T* __restrict__ y0, int O, double* __restrict__ part) {
+            const T* __restrict__ y0, int O, double* __restrict__ part, T* __restrict__ lean_t) {
   __shared__ T sct[CT];
   const int b = blockIdx.x;
   const int c = piece_cam[b];
@@ -1226,7 +1292,8 @@ k_schur_cam(const int32_t* __restrict__ piece_cam, const int32_t* __restrict__ p
   T acc[54];
 #pragma unroll
   for (int i = 0; i < 54; ++i) acc[i] = T(0);
-  schur_cam_range<T, MF, LIN_THREADS>(piece_beg[b], piece_end[b], cm_pt, Jcm, sct, pts, cm_sw, Vinv, y0, O, acc);
+  schur_cam_range<T, MF, LIN_THREADS, LEAN>(piece_beg[b], piece_end[b], cm_pt, Jcm, sct, pts, cm_sw, Vinv, y0, O, acc,
+                                            lean_t);
   block_sum_store<54>(acc, part + (long long)PART * b);
 }
 

@@ -98,7 +98,7 @@ const void* form_kernel(bool direct, bool f32, bool mf) {
   if (direct && f32)
     return mf ? (const void*)k_schur_form<float, true, double> : (const void*)k_schur_form<float, false, double>;
   if (f32) return mf ? (const void*)k_schur_form<float, true, float> : (const void*)k_schur_form<float, false, float>;
-  return mf ? (const void*)k_schur_form<double, true, double> : (const void*)k_schur_form<double, false, double>;
+  return mf ? (const void*)k_schur_form<double, true, double> : (const void*)k_schur_form_lean;
 }
 
 // Whether the PCG on the formed S takes less time than the implicit product
@@ -115,7 +115,7 @@ struct SchurCost {
     return iters() * (12.0 + O * (f32 ? 1.5e-5 : 1.28e-4)) + (maxiter - iters()) * 6.0;
   }
   // forming: FP64 pipe (13 ns per 32 pairs), FP32 arithmetic and gathers
-  double form_us(double pairs) const { return 25.0 + pairs * (f32 ? 3.0e-5 : 3.7e-4); }
+  double form_us(double pairs) const { return 25.0 + pairs * (f32 ? 5.0e-5 : 3.1e-4); }
   // two exchanges, then 81 multiply-adds or 324 bytes a block
   double iter_us(double blocks) const { return 8.0 + 162.0 * blocks * (f32 ? 0.8e-6 : 1.7e-6); }
 };
@@ -258,6 +258,14 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   };
   kernel_attr(form_kernel(direct, f32, h->mf), direct || !f32 ? sf_smem<double>() : sf_smem<float>());
+  const bool lean = !f32 && !h->mf;
+  if (lean) {
+    kernel_attr((const void*)k_schur_form_marked, sf_smem<double>());
+    if (e == cudaSuccess) e = h->alloc(&x.lean_w, 8ull * NLEAN * O);
+    if (e == cudaSuccess) e = h->alloc(&x.lean_t, 8ull * 6 * O);
+    if (e == cudaSuccess) e = h->alloc(&x.lean_marked, sizeof(int));
+    if (e == cudaSuccess) e = cudaMemsetAsync(x.lean_marked, 0, sizeof(int), s);
+  }
   if (e == cudaSuccess) e = up(&x.task, task);
   if (e == cudaSuccess) e = up(&x.blk_cam, bcam);
   if (e == cudaSuccess) e = up(&x.blk_task, btask);
@@ -271,6 +279,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
     keep(&x.pl, pl);
     keep(&x.pj, pj);
     x.direct = true;
+    x.lean = lean;
     return BA_OK;
   }
 
@@ -365,6 +374,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   x.groups = groups;
   x.rpb = rpb;
   x.pcg = true;
+  x.lean = lean;
   return BA_OK;
 }
 
@@ -385,7 +395,7 @@ void pcg(ba_problem* h, int maxiter, double tol) {
   auto& x = h->sx;
   cudaStream_t s = h->s;
   k_schur_combine<VT, VT><<<x.nblk, 96, 0, s>>>(x.blk_cam, x.blk_pos, x.blk_task, x.rowblk, (const VT*)x.part,
-                                                (VT*)x.val);
+                                                (VT*)x.val, x.lean ? (const double*)h->camtab : nullptr);
   cudaMemsetAsync(x.gx, 0, 8 * x.words, s);
   SchurPcg<VT> a;
   a.C = h->C;
@@ -419,20 +429,29 @@ void pcg(ba_problem* h, int maxiter, double tol) {
 
 void schur_form(ba_problem* h) {
   const bool f32 = h->prec == BA_PREC_F32;
+  if (h->sx.lean) {
+    auto& x = h->sx;
+    const unsigned g = nb_(x.ntask, SF_WARPS);
+    k_schur_form_lean<<<g, 32 * SF_WARPS, sf_smem<double>(), h->s>>>(
+        x.ntask, x.task, x.pk, x.pl, (const double2*)x.lean_w, (const double2*)x.lean_t, h->O, (double*)x.part);
+    k_schur_form_marked<<<std::min(g, 304u), 32 * SF_WARPS, sf_smem<double>(), h->s>>>(
+        x.ntask, x.task, x.pk, x.pl, x.pj, (const double2*)x.lean_w, (const double*)h->Jcm, h->O,
+        (const double*)h->Vinv, x.lean_marked, (double*)x.part);
+    count_launch(2);
+    return;
+  }
   if (h->sx.direct) {
     if (f32) h->mf ? form<float, true, double>(h) : form<float, false, double>(h);
-    else h->mf ? form<double, true, double>(h) : form<double, false, double>(h);
-  } else if (f32) {
-    h->mf ? form<float, true, float>(h) : form<float, false, float>(h);
+    else form<double, true, double>(h);
   } else {
-    form<double, false, double>(h);
+    h->mf ? form<float, true, float>(h) : form<float, false, float>(h);
   }
 }
 
 void schur_to_band(ba_problem* h, const double* lam_ptr) {
   auto& x = h->sx;
   k_schur_band<<<x.nblk, 96, 0, h->s>>>(x.blk_cam, x.blk_task, (const double*)x.part, h->U, lam_ptr, h->opt.diag_min,
-                                        h->opt.diag_max, h->fixed, h->bwt, h->bT);
+                                        h->opt.diag_max, h->fixed, h->bwt, h->bT, h->sx.lean ? (const double*)h->camtab : nullptr);
   count_launch();
 }
 

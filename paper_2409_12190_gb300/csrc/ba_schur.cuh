@@ -23,9 +23,9 @@
 //   k_schur_band     per block: into the band tiles of the direct solver
 //   k_schur_pcg      the whole PCG
 //
-// Bound: the FP64 pipe for double (210 + 18 multiply-adds a pair; a warp
-// instruction takes 16 cycles of its SM), FP32 arithmetic and the gathers of
-// the points for float.
+// Bound: the FP64 pipe for double (157 multiply-adds a pair in the lean form,
+// 228 from the planes; a warp instruction takes 16 cycles of its SM), FP32
+// arithmetic and the gathers of the points for float.
 #pragma once
 
 #include "ba_band.cuh"
@@ -43,6 +43,25 @@ constexpr int SX_PART = 81;                  // numbers of a task's partial bloc
 template <typename ACC>
 constexpr int sf_smem() {
   return SF_WARPS * 32 * SX_PART * (int)sizeof(ACC);
+}
+
+// The lanes' 81 sums, four runs of eight lanes, to out (or added to it); nl
+// lanes had an entry; red holds 32 x 81.
+template <typename ACC, bool ADD>
+__device__ __forceinline__ void sf_reduce(const ACC (&acc)[SX_PART], ACC* red, int nl, ACC* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int i = 0; i < SX_PART; ++i) red[lane * SX_PART + i] = acc[i];
+  __syncwarp();
+  for (int i = lane; i < SX_PART; i += 32) {
+    ACC s[4] = {ACC(0), ACC(0), ACC(0), ACC(0)};
+    for (int q = 0; q < nl; q += 4)
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (q + u < nl) s[u] += red[(q + u) * SX_PART + i];
+    const ACC v = (s[0] + s[1]) + (s[2] + s[3]);
+    out[i] = ADD ? out[i] + v : v;
+  }
 }
 
 // One observation's planes: all of them from the factored form (recompute
@@ -159,40 +178,191 @@ k_schur_form(int ntask, const int4* __restrict__ task, const int2* __restrict__ 
       }
     }
   }
-  // the lanes' sums, four runs of eight lanes
-  ACC* red = reinterpret_cast<ACC*>(sf_raw) + warp * 32 * SX_PART;
+  sf_reduce<ACC, false>(acc, reinterpret_cast<ACC*>(sf_raw) + warp * 32 * SX_PART, min(32, tk.z - tk.y),
+                        part + (long long)SX_PART * t);
+}
+
+// The same sums from the lean form (lean_obs), FP64: Jc' = [I | p] E with
+// E = [-[RX]_x | I | e_3 q'^T], so a pair's block is E_k^T N E_l with the 3 x 3
+// N = [I | p_k]^T K [I | p_l], K = (M^T Jp V*^{-1})_k (M^T Jp)_l^T: 157
+// multiply-adds instead of 228 with the planes, 14 loads of 16 bytes instead
+// of 27.  In the cameras' factored coordinates: J_l comes in with the block
+// (sf_finish).  Pairs with a marked observation are left to k_schur_form_marked.
+// FP64 pipe bound: 39M pairs of a 4,000-camera ring 17.9 -> 13.4 ms (lower bound
+// at the measured FMA rate 11.6 ms), 2.9M pairs of 250 cameras 1.46 -> 1.1 ms.
+static __global__ void __launch_bounds__(32 * SF_WARPS, 2)
+k_schur_form_lean(int ntask, const int4* __restrict__ task, const int32_t* __restrict__ pk,
+                  const int32_t* __restrict__ pl_, const double2* __restrict__ W, const double2* __restrict__ TV, int O,
+                  double* __restrict__ part) {
+  extern __shared__ __align__(16) unsigned char sf_raw[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t = blockIdx.x * SF_WARPS + warp;
+  if (t >= ntask) return;
+  const int4 tk = task[t];
+  const long long o = O;
+  double acc[SX_PART];
 #pragma unroll
-  for (int i = 0; i < SX_PART; ++i) red[lane * SX_PART + i] = acc[i];
-  __syncwarp();
-  const int nl = min(32, tk.z - tk.y);  // lanes that had an entry
-  for (int i = lane; i < SX_PART; i += 32) {
-    ACC s[4] = {ACC(0), ACC(0), ACC(0), ACC(0)};
-    for (int q = 0; q < nl; q += 4)
+  for (int i = 0; i < SX_PART; ++i) acc[i] = 0.0;
+  for (int e = tk.y + lane; e < tk.z; e += 32) {
+    const int k = pk[e], l = pl_[e];
+    const double2 k2 = W[2 * o + k], l2 = W[2 * o + l];  // (p1, q'0)
+    if (isnan(k2.y) || isnan(l2.y)) continue;
+    double N[9];
+    {
+      const double half = k == l ? 0.5 : 1.0;
+      const double2 t0 = TV[k], t1 = TV[o + k], t2 = TV[2 * o + k];
+      const double2 j0 = W[4 * o + l], j1 = W[5 * o + l], j2 = W[6 * o + l];
+      const double a0 = half * t0.x, a1 = half * t0.y, a2 = half * t1.x;
+      const double b0 = half * t1.y, b1 = half * t2.x, b2 = half * t2.y;
+      N[0] = a0 * j0.x + a1 * j0.y + a2 * j1.x;
+      N[1] = a0 * j1.y + a1 * j2.x + a2 * j2.y;
+      N[3] = b0 * j0.x + b1 * j0.y + b2 * j1.x;
+      N[4] = b0 * j1.y + b1 * j2.x + b2 * j2.y;
+    }
+    const double2 k0 = W[k], k1 = W[o + k], k3 = W[3 * o + k];  // (RX0, RX1) (RX2, p0) .. (q'1, q'2)
+    const double2 l0 = W[l], l1 = W[o + l], l3 = W[3 * o + l];
+    N[2] = N[0] * l1.y + N[1] * l2.x;
+    N[5] = N[3] * l1.y + N[4] * l2.x;
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (q + u < nl) s[u] += red[(q + u) * SX_PART + i];
-    part[(long long)SX_PART * t + i] = (s[0] + s[1]) + (s[2] + s[3]);
+    for (int c = 0; c < 3; ++c) N[6 + c] = k1.y * N[c] + k2.x * N[3 + c];
+    const double R0 = k0.x, R1 = k0.y, R2 = k1.x;
+    // one column of E_l at a time
+#pragma unroll
+    for (int c = 0; c < 9; ++c) {
+      double F[3];
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        const double* n = N + 3 * r;
+        F[r] = c == 0 ? n[2] * l0.y - n[1] * l1.x
+             : c == 1 ? n[0] * l1.x - n[2] * l0.x
+             : c == 2 ? n[1] * l0.x - n[0] * l0.y
+             : c < 6 ? n[c - 3]
+             : n[2] * (c == 6 ? l2.y : c == 7 ? l3.x : l3.y);
+      }
+      acc[c] = fma(R1, F[2], fma(-R2, F[1], acc[c]));
+      acc[9 + c] = fma(R2, F[0], fma(-R0, F[2], acc[9 + c]));
+      acc[18 + c] = fma(R0, F[1], fma(-R1, F[0], acc[18 + c]));
+      acc[27 + c] += F[0];
+      acc[36 + c] += F[1];
+      acc[45 + c] += F[2];
+      acc[54 + c] = fma(k2.y, F[2], acc[54 + c]);
+      acc[63 + c] = fma(k3.x, F[2], acc[63 + c]);
+      acc[72 + c] = fma(k3.y, F[2], acc[72 + c]);
+    }
   }
+  sf_reduce<double, false>(acc, reinterpret_cast<double*>(sf_raw) + warp * 32 * SX_PART, min(32, tk.z - tk.y),
+                           part + (long long)SX_PART * t);
+}
+
+// The pairs that k_schur_form_lean left out, from the planes, in the same
+// coordinates, added to its sums (a grid of a few blocks an SM strides over the tasks: it
+// returns at once when no observation is marked).
+static __global__ void __launch_bounds__(32 * SF_WARPS)
+k_schur_form_marked(int ntask, const int4* __restrict__ task, const int32_t* __restrict__ pk,
+                    const int32_t* __restrict__ pl_, const int32_t* __restrict__ pj, const double2* __restrict__ W,
+                    const double* __restrict__ Jcm, int O, const double* __restrict__ Vinv,
+                    const int* __restrict__ marked, double* __restrict__ part) {
+  if (!*marked) return;
+  extern __shared__ __align__(16) unsigned char sf_raw[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long long o = O;
+  auto rows = [&](int s, double(&j0)[9], double(&j1)[9], double(&jp)[6]) {
+    double pl[NPLANE];
+    load_planes(Jcm, o, s, pl);
+    jc_rows(pl, j0, j1);
+    const double2 r01 = W[s];
+    const double R0 = r01.x, R1 = r01.y, R2 = W[o + s].x;
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const double* A = pl + 3 * a;
+      double* j = a == 0 ? j0 : j1;
+      j[0] = R1 * A[2] - R2 * A[1];
+      j[1] = R2 * A[0] - R0 * A[2];
+      j[2] = R0 * A[1] - R1 * A[0];
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) jp[i] = pl[NPLANE_JC + i];
+  };
+  for (int t = blockIdx.x * SF_WARPS + warp; t < ntask; t += gridDim.x * SF_WARPS) {
+    const int4 tk = task[t];
+    double acc[SX_PART];
+#pragma unroll
+    for (int i = 0; i < SX_PART; ++i) acc[i] = 0.0;
+    bool any = false;
+    for (int e = tk.y + lane; e < tk.z; e += 32) {
+      const int k = pk[e], l = pl_[e];
+      if (!isnan(W[2 * o + k].y) && !isnan(W[2 * o + l].y)) continue;
+      any = true;
+      const double* vi = Vinv + 6LL * pj[e];
+      double k0[9], k1[9], l0[9], l1[9], jk[6], jl[6], K[4];
+      rows(k, k0, k1, jk);
+      rows(l, l0, l1, jl);
+      const double half = k == l ? 0.5 : 1.0;
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const double* p = jk + 3 * r;
+        const double t0 = p[0] * vi[0] + p[1] * vi[1] + p[2] * vi[2];
+        const double t1 = p[0] * vi[1] + p[1] * vi[3] + p[2] * vi[4];
+        const double t2 = p[0] * vi[2] + p[1] * vi[4] + p[2] * vi[5];
+#pragma unroll
+        for (int c = 0; c < 2; ++c) K[2 * r + c] = half * (t0 * jl[3 * c] + t1 * jl[3 * c + 1] + t2 * jl[3 * c + 2]);
+      }
+#pragma unroll
+      for (int c = 0; c < 9; ++c) {
+        const double g0 = K[0] * l0[c] + K[1] * l1[c], g1 = K[2] * l0[c] + K[3] * l1[c];
+#pragma unroll
+        for (int r = 0; r < 9; ++r) acc[9 * r + c] += k0[r] * g0 + k1[r] * g1;
+      }
+    }
+    if (__any_sync(0xffffffffu, any))
+      sf_reduce<double, true>(acc, reinterpret_cast<double*>(sf_raw) + warp * 32 * SX_PART, min(32, tk.z - tk.y),
+                              part + (long long)SX_PART * t);
+    __syncwarp();
+  }
+}
+
+// A block's 81 sums (in sv, row of its first camera, column of its second)
+// from factored to plain coordinates: rows 0-2 by J_l^T of the first camera,
+// columns 0-2 by J_l of the second.  96 threads, all of them.
+__device__ __forceinline__ void sf_finish(double* sv, int e, const double* __restrict__ ct_i,
+                                          const double* __restrict__ ct_l) {
+  const int r = e / 9, q = e % 9;
+  double v = 0.0;
+  if (e < 27)
+    for (int m = 0; m < 3; ++m) v += ct_i[CT_JL + 3 * m + r] * sv[9 * m + q];
+  __syncthreads();
+  if (e < 27) sv[e] = v;
+  __syncthreads();
+  const int r2 = e / 3, q2 = e % 3;
+  v = 0.0;
+  if (e < 27)
+    for (int m = 0; m < 3; ++m) v += sv[9 * r2 + m] * ct_l[CT_JL + 3 * m + q2];
+  __syncthreads();
+  if (e < 27) sv[9 * r2 + q2] = v;
+  __syncthreads();
 }
 
 // Block b of S from its tasks' partial sums, negated, into the row panels of
 // both of its cameras.  blk_pos: its position in row i and in row l; a block
 // of a camera with itself (a point observed twice by it) is added with its
-// transpose.
+// transpose.  camtab: the sums are in factored coordinates (the lean form).
 template <typename ACC, typename VT>
 static __global__ void __launch_bounds__(96)
 k_schur_combine(const int2* __restrict__ blk_cam, const int2* __restrict__ blk_pos, const int* __restrict__ blk_task,
-                const int32_t* __restrict__ rowblk, const ACC* __restrict__ part, VT* __restrict__ val) {
+                const int32_t* __restrict__ rowblk, const ACC* __restrict__ part, VT* __restrict__ val,
+                const double* __restrict__ camtab) {
   __shared__ double sv[SX_PART];
   const int b = blockIdx.x, e = threadIdx.x;
   const int2 c = blk_cam[b], pos = blk_pos[b];
-  double v = 0.0;
   if (e < SX_PART) {
-    for (int t = blk_task[b]; t < blk_task[b + 1]; ++t) v += (double)part[(long long)SX_PART * t + e];
-    sv[e] = v;
+    double s = 0.0;
+    for (int t = blk_task[b]; t < blk_task[b + 1]; ++t) s += (double)part[(long long)SX_PART * t + e];
+    sv[e] = s;
   }
   __syncthreads();
+  if (camtab) sf_finish(sv, e, camtab + (long long)CT * c.x, camtab + (long long)CT * c.y);
   if (e >= SX_PART) return;
+  const double v = sv[e];
   const int r = e / 9, q = e % 9;
   const long long bi = rowblk[c.x], bl = rowblk[c.y];
   const int wi = 9 * (rowblk[c.x + 1] - (int)bi), wl = 9 * (rowblk[c.y + 1] - (int)bl);
@@ -211,7 +381,7 @@ k_schur_combine(const int2* __restrict__ blk_cam, const int2* __restrict__ blk_p
 static __global__ void __launch_bounds__(96)
 k_schur_band(const int2* __restrict__ blk_cam, const int* __restrict__ blk_task, const double* __restrict__ part,
              const double* __restrict__ U, const double* __restrict__ lam_ptr, double dmin, double dmax,
-             const uint8_t* __restrict__ fixed, int bwt, double* __restrict__ T) {
+             const uint8_t* __restrict__ fixed, int bwt, double* __restrict__ T, const double* __restrict__ camtab) {
   __shared__ double sv[SX_PART];
   const int b = blockIdx.x, e = threadIdx.x;
   const int2 c = blk_cam[b];
@@ -221,6 +391,7 @@ k_schur_band(const int2* __restrict__ blk_cam, const int* __restrict__ blk_task,
     sv[e] = v;
   }
   __syncthreads();
+  if (camtab) sf_finish(sv, e, camtab + (long long)CT * c.x, camtab + (long long)CT * c.y);
   if (e >= SX_PART) return;
   const int r = e / 9, q = e % 9;  // row of camera c.y, column of camera c.x
   const int R = 9 * c.y + r, C = 9 * c.x + q;

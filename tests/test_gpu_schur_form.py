@@ -136,3 +136,28 @@ def test_solves_on_two_streams_at_once():
         torch.cuda.synchronize()
         assert all(torch.equal(a, b) for a, b in zip(got, want))
         prob.close()
+
+
+@pytest.mark.parametrize("solver", ["pcg", "cholesky"])
+@pytest.mark.parametrize("k1", [-3.0, -8.0])
+def test_observations_near_the_fold_of_the_distortion(solver, k1):
+    """Where 1 + 3 k1 r^2 + 5 k2 r^4 passes through 0 the lean form of an
+    observation does not exist: those take their planes.  Two cameras with such
+    a distortion, the image radius of their points spread over the fold."""
+    sc = _ragged(8, 400, seed=11, lo=3, hi=6)
+    cams = sc.cams_init.copy()
+    cams[[2, 5], 7] = k1
+    pix = orc.pixels_from_scene(sc)
+    X = orc.rodrigues(cams[sc.cam_idx, :3]) @ sc.points_init[sc.pt_idx][:, :, None]
+    X = X[:, :, 0] + cams[sc.cam_idx, 3:6]
+    r2 = ((X[:, :2] / X[:, 2:]) ** 2).sum(1)
+    mu, nu = (1 + n * cams[sc.cam_idx, 7] * r2 + m * cams[sc.cam_idx, 8] * r2 * r2 for n, m in ((3, 5), (1, 1)))
+    assert np.sum(np.abs(mu) < 0.125 * np.abs(nu)) >= 3
+    sc = scenegen.Scene(sc.cams_gt, sc.points_gt, sc.cam_idx, sc.pt_idx, sc.noise, cams, sc.points_init)
+    blk = orc.assemble(sc.cams_init, sc.points_init, sc.cam_idx, sc.pt_idx, pix)
+    its = 8
+    dc_ref, dp_ref, _, _ = orc.solve_damped(blk, sc.cam_idx, sc.pt_idx, 1e-1,
+                                            orc.LMOptions(solver=solver, pcg_maxiter=its, pcg_tol=0.0))
+    with problem(sc, pix, "f64", solver=solver) as prob:
+        dc, dp, _, _ = prob.damped_solve(1e-1, its, 0.0)
+    assert rel_err(np64(dc), dc_ref) < 1e-9 and rel_err(np64(dp), dp_ref) < 1e-9
