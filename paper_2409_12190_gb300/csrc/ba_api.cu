@@ -449,19 +449,19 @@ void enqueue_solve(ba_problem* h, const double* lam_ptr, int maxiter, double tol
 template <typename T, bool MF>
 void enqueue_cost(ba_problem* h, bool gated = false) {
   const T delta = (T)(h->opt.huber_delta > 0 ? h->opt.huber_delta : 0.0);
-  k_cost_cam<T, false, MF><<<h->npieces, PIECE_THREADS, 0, h->s>>>(
-      h->piece_cam, h->piece_beg, h->piece_end, h->cm_pt, (const T*)h->cm_px, (const T*)h->cams,
+  k_cost_cam<T, false, MF><<<h->ncost, PIECE_THREADS, 0, h->s>>>(
+      h->cost_cam, h->cost_beg, h->cost_end, h->cm_pt, (const T*)h->cm_px, (const T*)h->cams,
       (const T*)h->pts, h->st, gated ? 2 : 0, delta, h->C, h->P, h->O, nullptr, nullptr, nullptr, nullptr, nullptr,
       h->part);
   if (h->xch) {
     // the cost over every part (0 from each part when F is not stale)
-    k_part_cost_sum<<<1, 256, 0, h->s>>>(h->npieces, h->part, h->st, gated ? 1 : 0, h->xscal + 4);
+    k_part_cost_sum<<<1, 256, 0, h->s>>>(h->ncost, h->part, h->st, gated ? 1 : 0, h->xscal + 4);
     xchg(h, h->xscal + 4, 1);
     k_cost_set<<<1, 1, 0, h->s>>>(h->st, gated ? 1 : 0, h->xscal + 4);
     count_launch(3);
     return;
   }
-  k_cost_finalize<<<1, 256, 0, h->s>>>(h->npieces, h->part, h->st, gated ? 1 : 0);
+  k_cost_finalize<<<1, 256, 0, h->s>>>(h->ncost, h->part, h->st, gated ? 1 : 0);
   count_launch(2);
 }
 
@@ -780,28 +780,48 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
     const long long per = O / (6LL * nsm);
     piece_max = (int)std::min<long long>(PIECE, std::max<long long>(LIN_THREADS, (per + LIN_THREADS - 1) / LIN_THREADS * LIN_THREADS));
   }
+  // F itself keeps the pieces of PIECE slots: a batch of problems adds it in
+  // the same order.
   std::vector<int32_t> rp(C + 1);
   CU(cudaMemcpy(rp.data(), h->rowptr_cam, (C + 1) * 4, cudaMemcpyDeviceToHost));
-  std::vector<int32_t> pc, pb, pe, cpp(C + 1);
-  for (long long c = 0; c < C; ++c) {
-    cpp[c] = (int32_t)pc.size();
-    const int n = rp[c + 1] - rp[c];
-    const int k = (n + piece_max - 1) / piece_max;
-    for (int i = 0; i < k; ++i) {
-      pc.push_back((int32_t)c);
-      pb.push_back(rp[c] + (int)((long long)n * i / k));
-      pe.push_back(rp[c] + (int)((long long)n * (i + 1) / k));
+  std::vector<int32_t> cpp(C + 1);
+  auto cut = [&](int most, int* count, int32_t** d_cam, int32_t** d_beg, int32_t** d_end) -> ba_status {
+    std::vector<int32_t> pc, pb, pe;
+    for (long long c = 0; c < C; ++c) {
+      cpp[c] = (int32_t)pc.size();
+      const int n = rp[c + 1] - rp[c];
+      const int k = (n + most - 1) / most;
+      for (int i = 0; i < k; ++i) {
+        pc.push_back((int32_t)c);
+        pb.push_back(rp[c] + (int)((long long)n * i / k));
+        pe.push_back(rp[c] + (int)((long long)n * (i + 1) / k));
+      }
     }
+    cpp[C] = (int32_t)pc.size();
+    *count = (int)pc.size();
+    CU(h->alloc(d_cam, pc.size() * 4));
+    CU(h->alloc(d_beg, pc.size() * 4));
+    CU(h->alloc(d_end, pc.size() * 4));
+    CU(cudaMemcpy(*d_cam, pc.data(), pc.size() * 4, cudaMemcpyHostToDevice));
+    CU(cudaMemcpy(*d_beg, pb.data(), pb.size() * 4, cudaMemcpyHostToDevice));
+    CU(cudaMemcpy(*d_end, pe.data(), pe.size() * 4, cudaMemcpyHostToDevice));
+    return BA_OK;
+  };
+  if (piece_max != PIECE) {
+    const ba_status cs = cut(PIECE, &h->ncost, &h->cost_cam, &h->cost_beg, &h->cost_end);
+    if (cs != BA_OK) return cs;
   }
-  cpp[C] = (int32_t)pc.size();
-  h->npieces = (int)pc.size();
-  CU(h->alloc(&h->piece_cam, pc.size() * 4));
-  CU(h->alloc(&h->piece_beg, pc.size() * 4));
-  CU(h->alloc(&h->piece_end, pc.size() * 4));
+  {
+    const ba_status cs = cut(piece_max, &h->npieces, &h->piece_cam, &h->piece_beg, &h->piece_end);
+    if (cs != BA_OK) return cs;
+  }
+  if (piece_max == PIECE) {
+    h->ncost = h->npieces;
+    h->cost_cam = h->piece_cam;
+    h->cost_beg = h->piece_beg;
+    h->cost_end = h->piece_end;
+  }
   CU(h->alloc(&h->cam_piece_ptr, (C + 1) * 4));
-  CU(cudaMemcpy(h->piece_cam, pc.data(), pc.size() * 4, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(h->piece_beg, pb.data(), pb.size() * 4, cudaMemcpyHostToDevice));
-  CU(cudaMemcpy(h->piece_end, pe.data(), pe.size() * 4, cudaMemcpyHostToDevice));
   CU(cudaMemcpy(h->cam_piece_ptr, cpp.data(), (C + 1) * 4, cudaMemcpyHostToDevice));
 
   // linearisation and solver buffers

@@ -94,8 +94,8 @@ struct BShared {
   double U[BMAXC * 45];
   double M[BMAXC * 45];
   double gc[BMAXC * 9];
-  double x[BMAXC * 9], r[BMAXC * 9], z[BMAXC * 9], p[BMAXC * 9], q[BMAXC * 9], ss[BMAXC * 9];
-  double red[8 * 54];  // reduction scratch (float2 or double per slot)
+  double x[BMAXC * 9], r[BMAXC * 9], z[BMAXC * 9], p[BMAXC * 9], ss[BMAXC * 9];
+  double red[2 * BT];  // reduction scratch (float2 or double per slot)
   double tot[9];
   T ct[BMAXC][CT];  // camera tables of the linearisation
   T pT[BMAXC][PV];  // PCG direction in the passes' form
@@ -210,6 +210,32 @@ __device__ __forceinline__ void bred_all(BShared<T>& S, double (&v)[NV]) {
 #pragma unroll
   for (int i = 0; i < NV; ++i) v[i] = S.tot[i];
   __syncthreads();
+}
+
+// Sums of NV values of the first n threads (S.red[i * BT + t]) by warp 0,
+// which returns them in t; the other warps return at once.  For the PCG's
+// scalars: an FP64 warp instruction takes 16 cycles of the SM, so a shuffle
+// tree, a division or a square root in each of eight warps was a third of an
+// iteration.
+template <int NV, typename T>
+__device__ __forceinline__ bool bred_warp0(BShared<T>& S, int n, double (&t)[NV]) {
+  __syncthreads();
+  if (threadIdx.x >= 32) return false;
+  const int lane = threadIdx.x;
+#pragma unroll
+  for (int i = 0; i < NV; ++i) t[i] = lane < n ? S.red[i * BT + lane] : 0.0;
+  for (int k = lane + 32; k < n; k += 32)
+#pragma unroll
+    for (int i = 0; i < NV; ++i) t[i] += S.red[i * BT + k];
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    double u[NV];
+#pragma unroll
+    for (int i = 0; i < NV; ++i) u[i] = __shfl_xor_sync(0xffffffffu, t[i], off);
+#pragma unroll
+    for (int i = 0; i < NV; ++i) t[i] += u[i];
+  }
+  return true;
 }
 
 // = block_sum_array
@@ -548,7 +574,7 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
       S.ss[o] = sum;
     }
     __syncthreads();
-    double pq = 0.0;
+    double qv = 0.0;
     if (ok) {
       if (MF && ci < 3) {
         const T* Jl = S.ct[lc] + CT_JL;
@@ -559,28 +585,28 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
       double y = damp(Uc[sym9(ci, ci)], lam, a.dmin, a.dmax) * S.p[o];
 #pragma unroll
       for (int j = 0; j < 9; ++j) y += Uc[sym9_rt(ci, j)] * S.p[9 * lc + j];
-      y -= sum;
-      S.q[o] = y;
-      pq = pv * y;
+      qv = y - sum;
+      S.red[tid] = pv * qv;
     }
     {
-      double v[1] = {pq};
-      bred_all<1>(S, v);
-      pq = v[0];
+      // alpha, or NaN for no positive curvature (b = 0 or breakdown): keep x, stop
+      double t[1];
+      if (bred_warp0<1>(S, 9 * R.nc, t) && tid == 0)
+        S.tot[0] = t[0] > 0.0 && isfinite(t[0]) ? S.rz_old / t[0] : nan("");
     }
-    if (!(pq > 0.0) || !isfinite(pq)) {
-      // no positive curvature (b = 0 or breakdown): keep x, stop
+    __syncthreads();
+    const double alpha = S.tot[0];
+    if (isnan(alpha)) {
       if (tid == 0) {
         S.pcg_iters = k;
         if (k == 0) S.pcg_rel = 0.0;
       }
       break;
     }
-    const double alpha = S.rz_old / pq;
     double rv = 0.0;
     if (ok) {
       S.x[o] += alpha * S.p[o];
-      rv = S.r[o] - alpha * S.q[o];
+      rv = S.r[o] - alpha * qv;
       S.r[o] = rv;
     }
     __syncthreads();
@@ -589,21 +615,25 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
       const double* Mc = S.M + 45 * lc;
 #pragma unroll
       for (int j = 0; j < 9; ++j) zz += Mc[sym9_rt(ci, j)] * S.r[9 * lc + j];
-      S.z[o] = zz;
+      S.red[tid] = rv * zz;
+      S.red[BT + tid] = rv * rv;
     }
-    double v2[2] = {rv * zz, rv * rv};
-    bred_all<2>(S, v2);
-    const double rz_new = v2[0], rr = v2[1], rz_old = S.rz_old, bb = S.bb;
-    const bool conv = sqrt(rr) <= a.tol * sqrt(bb);
-    if (tid == 0) {
-      S.pcg_iters = k + 1;
-      S.pcg_rel = bb > 0.0 ? sqrt(rr / bb) : 0.0;
+    {
+      double t[2];
+      if (bred_warp0<2>(S, 9 * R.nc, t) && tid == 0) {
+        const double bb = S.bb;
+        S.tot[0] = t[0] / S.rz_old;
+        S.tot[1] = sqrt(t[1]) <= a.tol * sqrt(bb) ? 1.0 : 0.0;
+        S.rz_old = t[0];
+        S.pcg_iters = k + 1;
+        S.pcg_rel = bb > 0.0 ? sqrt(t[1] / bb) : 0.0;
+      }
     }
-    if (conv) break;
-    const double beta = rz_new / rz_old;
+    __syncthreads();
+    const double beta = S.tot[0];
+    if (S.tot[1] != 0.0) break;
     if (ok) {
-      const double pn = S.z[o] + beta * S.p[o];
-      S.p[o] = pn;
+      S.p[o] = zz + beta * S.p[o];
     }
     __syncthreads();
     if (ok) {
@@ -616,7 +646,6 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
         S.pT[lc][ci] = (T)S.p[o];
       }
     }
-    if (tid == 0) S.rz_old = rz_new;
     __syncthreads();
   }
   __syncthreads();

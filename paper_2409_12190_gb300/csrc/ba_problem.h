@@ -66,6 +66,8 @@ struct ba_problem {
   void *cm_px = nullptr, *pm_px = nullptr, *px_in = nullptr;
   int npieces = 0;
   int32_t *piece_cam = nullptr, *piece_beg = nullptr, *piece_end = nullptr, *cam_piece_ptr = nullptr;
+  int ncost = 0;  // pieces of F
+  int32_t *cost_cam = nullptr, *cost_beg = nullptr, *cost_end = nullptr;
   // parameters, double-buffered (current / trial)
   void *cams = nullptr, *pts = nullptr;
   // linearisation
