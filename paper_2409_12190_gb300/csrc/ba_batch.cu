@@ -36,6 +36,12 @@ struct ba_batch {
   int* work = nullptr;
   void *cams0 = nullptr, *pts0 = nullptr;  // parameters at creation (internal order)
   // launch configuration
+  // formed reduced systems (form_setup), or NULL
+  int32_t* sx_off = nullptr;
+  int4* sx_blk = nullptr;
+  int32_t *sx_pk = nullptr, *sx_pl = nullptr, *sx_pj = nullptr;
+  long long* sx_val_off = nullptr;
+  void* sx_val = nullptr;
   int ctas_per_sm = 1, variant = 0, order = 0;
   // segment sizes: camera-major pieces of at most piece_max slots, point
   // chunks of at most chunk_slots slots and chunk_pts points
@@ -152,6 +158,13 @@ BatchArgs<T> make_args(ba_batch* b, int iters) {
   a.state = b->state;
   a.stats = b->stats;
   a.cap = b->cap;
+  a.sx_off = b->sx_off;
+  a.sx_blk = b->sx_blk;
+  a.sx_pk = b->sx_pk;
+  a.sx_pl = b->sx_pl;
+  a.sx_pj = b->sx_pj;
+  a.sx_val_off = b->sx_val_off;
+  a.sx_val = (T*)b->sx_val;
   a.work = b->work;
   a.iters = iters;
   a.delta = (T)(o.huber_delta > 0 ? o.huber_delta : 0.0);
@@ -178,6 +191,52 @@ const void* kernel_of(const ba_batch* b, int variant) {
   const ba_problem* h = b->h;
   if (h->prec == BA_PREC_F32) return h->mf ? kernel_for<float, true>(variant) : kernel_for<float, false>(variant);
   return h->mf ? kernel_for<double, true>(variant) : kernel_for<double, false>(variant);
+}
+
+// The reduced systems formed explicitly in FP32 recompute mode: a pair of
+// observations costs about 2 ns of a CTA, an observation of an implicit
+// iteration 5 (latency: 512 windows, 8 warps a CTA), so with 12 iterations
+// (or maxiter, if less) up to 2.5 pairs an observation and iteration are worth
+// forming.  (28 cameras have at most 13.5 pairs an observation.)
+ba_status form_setup(ba_batch* b, const std::vector<int32_t>& rq) {
+  ba_problem* h = b->h;
+  SchurPairs pr;
+  ba_status st = schur_pairs(h, rq, false, (long long)(2.5 * std::min(h->opt.pcg_maxiter, 12) * h->O), pr);
+  if (st != BA_OK || pr.n == 0) return st;
+  std::vector<int4> blk;
+  std::vector<int32_t> off(1, 0);
+  std::vector<long long> voff;
+  long long vals = 0;
+  size_t q = 0;
+  for (int i = 0; i < b->nprob; ++i) {
+    const int c0 = b->cam_off[i], c1 = b->cam_off[i + 1];
+    for (; q < pr.head.size() && pr.cam[q].x < c1; ++q)
+      blk.push_back(make_int4(pr.cam[q].x - c0, pr.cam[q].y - c0, pr.head[q],
+                              q + 1 < pr.head.size() ? pr.head[q + 1] : pr.n));
+    off.push_back((int32_t)blk.size());
+    voff.push_back(vals);
+    vals += ((long long)9 * (c1 - c0) * sx_ld(c1 - c0) + 3) / 4 * 4;
+  }
+  cudaError_t e = b->alloc(&b->sx_off, off.size() * 4);
+  if (e == cudaSuccess) e = b->alloc(&b->sx_blk, blk.size() * sizeof(int4));
+  if (e == cudaSuccess) e = b->alloc(&b->sx_val_off, voff.size() * 8);
+  if (e == cudaSuccess) e = cudaMemcpy(b->sx_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(b->sx_blk, blk.data(), blk.size() * sizeof(int4), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaMemcpy(b->sx_val_off, voff.data(), voff.size() * 8, cudaMemcpyHostToDevice);
+  void* val = nullptr;
+  if (e == cudaSuccess) e = b->alloc(&val, vals * 4);
+  // blocks of cameras without a common point stay zero
+  if (e == cudaSuccess) e = cudaMemset(val, 0, vals * 4);
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // no room: the implicit product
+    return BA_OK;
+  }
+  b->sx_pk = pr.pk;
+  b->sx_pl = pr.pl;
+  b->sx_pj = pr.pj;
+  pr.keep(b->allocs);
+  b->sx_val = val;
+  return BA_OK;
 }
 
 int grid_of(const ba_batch* b) { return std::max(1, std::min(b->nprob, b->ctas_per_sm * b->nsm)); }
@@ -405,6 +464,13 @@ ba_status ba_batch_create(ba_batch** out, int nprob, const int32_t* cam_counts, 
   }
   if (e != cudaSuccess)
     return fail_out(e == cudaErrorMemoryAllocation ? BA_ERR_OOM : BA_ERR_CUDA, "batch allocation failed");
+  if (h->prec == BA_PREC_F32 && h->mf) {
+    st = form_setup(b, rq);
+    if (st != BA_OK) {
+      delete b;
+      return st;
+    }
+  }
   b->smem = h->prec == BA_PREC_F32 ? sizeof(BShared<float>) : sizeof(BShared<double>);
   if (h->prec == BA_PREC_F32) e = h->mf ? set_smem_attr<float, true>(b->smem) : set_smem_attr<float, false>(b->smem);
   else e = h->mf ? set_smem_attr<double, true>(b->smem) : set_smem_attr<double, false>(b->smem);
@@ -412,10 +478,11 @@ ba_status ba_batch_create(ba_batch** out, int nprob, const int32_t* cam_counts, 
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return fail_out(BA_ERR_CUDA, "kernel attribute set-up failed");
-  // two CTAs an SM where there are problems for both (512 sliding windows:
-  // 8.9 ms with one CTA an SM, 6.9 ms with two); with fewer problems than SMs
-  // the one CTA with all of the registers (8.9 against 9.8 ms alone on an SM)
-  b->variant = b->nprob > b->nsm && occupancy(b, 1) >= 2 ? 1 : 0;
+  // With the systems formed one CTA an SM with all of the registers (512
+  // windows 5.4 ms, two with half of them 6.0: the 81 sums of a block spill).
+  // Otherwise two CTAs an SM where there are problems for both (8.9 against
+  // 6.9 ms); with fewer problems than SMs one (8.9 against 9.8 ms).
+  b->variant = !b->sx_val && b->nprob > b->nsm && occupancy(b, 1) >= 2 ? 1 : 0;
   b->ctas_per_sm = occupancy(b, b->variant);
   b->order = 0;
   st = upload_order(b);

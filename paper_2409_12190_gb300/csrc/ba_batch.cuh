@@ -25,11 +25,13 @@
 #include <stddef.h>
 
 #include "ba_kernels.cuh"
+#include "ba_schur.cuh"
 
 namespace ba {
 
 constexpr int BT = PIECE_THREADS;  // threads per problem
 constexpr int BMAXC = 28;          // cameras per problem: 9 * BMAXC <= BT
+constexpr int CT_TAB64 = 15;       // R, t, f, k1, k2: what a cost reads of a camera table
 static_assert(9 * BMAXC <= BT, "the per-camera vector phase runs one thread per component");
 static_assert(CHUNK_THREADS == BT, "point chunks are reduced with the block's threads");
 
@@ -81,6 +83,15 @@ struct BatchArgs {
   BState* state;
   ba_iter_stats* stats;  // [nprob][cap]
   int cap;
+  // the reduced system of each problem formed explicitly (FP32 recompute
+  // mode), or NULL: the camera-pair blocks (local cameras, entries e0 .. e1 of
+  // the sorted pairs) of each problem, and its dense matrix without the
+  // diagonal blocks, rows of sx_ld(nc)
+  const int32_t* sx_off;  // [nprob + 1]
+  const int4* sx_blk;
+  const int32_t *sx_pk, *sx_pl, *sx_pj;
+  const long long* sx_val_off;  // [nprob]
+  T* sx_val;
   int* work;
   int iters;
   T delta;
@@ -100,17 +111,22 @@ struct BShared {
   T ct[BMAXC][CT];  // camera tables of the linearisation
   T pT[BMAXC][PV];  // PCG direction in the passes' form
   T xT[BMAXC][PV];  // camera step in the passes' form
-  double sce64[CT]; // camera table of the evaluated parameters (cost, in double)
-  FFCam sceff;      // the same split into float-float pairs (FP32 cost)
+  double sce64[BMAXC][CT_TAB64];  // camera tables of the evaluated parameters (cost, in double)
+  static constexpr bool F32 = sizeof(T) == 4;
+  FFCam sceff[F32 ? BMAXC : 1];   // the same split into float-float pairs (FP32 cost)
   // recompute mode: padded copies of the camera tables and of the vector a
   // point-major pass reads (neighbouring slots use different cameras), and
   // the per-observation products of one point chunk
   T fct[BMAXC][17];
   T fxv[BMAXC][13];
   alignas(16) T sz[CHUNK_SLOTS * 4];  // read and written as 4-vectors
+  // formed system: diagonal blocks, and the PCG direction in T
+  double Sii[F32 ? BMAXC * 45 : 1];
+  alignas(16) T pf[F32 ? BT : 4];
   double lam, F, rz_old, bb, pcg_rel, dot_gc;
   long long trials;
-  int cur, need_lin, pcg_iters, fallbacks, widx;
+  double stop, rr;  // PCG: the bound of |r|, the last |r|^2
+  int cur, need_lin, pcg_iters, fallbacks, widx, next_blk;
 };
 
 static_assert(offsetof(BShared<float>, sz) % 16 == 0 && offsetof(BShared<double>, sz) % 16 == 0,
@@ -390,6 +406,151 @@ __device__ __forceinline__ void batch_stage_fxv(BShared<T>& S, const BRange<T>& 
   __syncthreads();
 }
 
+// Row stride of a formed system of nc cameras.
+__host__ __device__ constexpr int sx_ld(int nc) { return (9 * nc + 3) / 4 * 4; }
+
+// Warp reduce-scatter of 81 floats (padded to 96): lane l returns the totals
+// of values 3 l .. 3 l + 2.
+template <int N, int OFF>
+__device__ __forceinline__ void sx_rs96_step(float (&h)[48], int lane) {
+  const bool up = (lane & OFF) != 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const float k = up ? h[N + i] : h[i];
+    const float g = up ? h[i] : h[N + i];
+    h[i] = k + __shfl_xor_sync(0xffffffffu, g, OFF);
+  }
+}
+
+// The off-diagonal blocks of S of problem b, -sum W_k V*^{-1} W_l^T over the
+// common points of each camera pair, both triangles: one warp a block, one
+// pair a lane (the arithmetic of k_schur_form).  The largest of 512 windows
+// (20 cameras, 20,900 observations) alone in its CTA took 1.8 ms a trial of ten
+// implicit iterations; a pair costs about what one observation of one
+// iteration does, and an iteration on the formed S reads 130 KB from L2.  The
+// warps take the blocks from a counter.
+template <typename T>
+__device__ __noinline__ void batch_form(const BatchArgs<T>& a, const BRange<T>& R, BShared<T>& S, int b) {
+  const int lane = threadIdx.x & 31;
+  const int ld = sx_ld(R.nc);
+  T* val = a.sx_val + a.sx_val_off[b];
+  for (;;) {
+    // the next block of the problem (each is summed by one warp whichever it is)
+    int q = 0;
+    if (lane == 0) q = atomicAdd(&S.next_blk, 1);
+    q = __shfl_sync(0xffffffffu, q, 0);
+    if (q >= a.sx_off[b + 1]) break;
+    const int4 blk = a.sx_blk[q];
+    T acc[SX_PART];
+#pragma unroll
+    for (int i = 0; i < SX_PART; ++i) acc[i] = T(0);
+    for (int e = blk.z + lane; e < blk.w; e += 32) {
+      const int j = a.sx_pj[e];
+      const int k = a.cm_sw ? a.sx_pk[e] : 0, l = a.cm_sw ? a.sx_pl[e] : 0;
+      T X0, X1, X2, pad;
+      load4(a.ptab + 8LL * j, X0, X1, X2, pad);
+      const T* vi = a.Vinv + 6LL * j;
+      const T v00 = vi[0], v01 = vi[1], v02 = vi[2], v11 = vi[3], v12 = vi[4], v22 = vi[5];
+      SfObs<T, true> u, w;
+      u.open(nullptr, 0, k, S.ct[blk.x], X0, X1, X2, a.cm_sw);
+      w.open(nullptr, 0, l, S.ct[blk.y], X0, X1, X2, a.cm_sw);
+      T K[4];
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const T* p = u.pl + NPLANE_JC + 3 * r;
+        const T t0 = p[0] * v00 + p[1] * v01 + p[2] * v02;
+        const T t1 = p[0] * v01 + p[1] * v11 + p[2] * v12;
+        const T t2 = p[0] * v02 + p[1] * v12 + p[2] * v22;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const T* z = w.pl + NPLANE_JC + 3 * c;
+          K[2 * r + c] = t0 * z[0] + t1 * z[1] + t2 * z[2];
+        }
+      }
+      T k0[9], k1[9], l0[9], l1[9];
+      jc_rows(u.pl, k0, k1);
+      jc_rows(w.pl, l0, l1);
+#pragma unroll
+      for (int c = 0; c < 9; ++c) {
+        const T g0 = K[0] * l0[c] + K[1] * l1[c], g1 = K[2] * l0[c] + K[3] * l1[c];
+#pragma unroll
+        for (int r = 0; r < 9; ++r) acc[9 * r + c] += k0[r] * g0 + k1[r] * g1;
+      }
+    }
+    float h[48];
+    {
+      const bool up = (lane & 16) != 0;
+#pragma unroll
+      for (int i = 0; i < 48; ++i) {
+        const float lo = acc[i], hi = 48 + i < SX_PART ? acc[48 + i < SX_PART ? 48 + i : 0] : 0.f;
+        h[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, 16);
+      }
+    }
+    sx_rs96_step<24, 8>(h, lane);
+    sx_rs96_step<12, 4>(h, lane);
+    sx_rs96_step<6, 2>(h, lane);
+    sx_rs96_step<3, 1>(h, lane);
+    if (blk.x == blk.y) {
+      // a camera that observes a point twice: with the transpose
+#pragma unroll
+      for (int u = 0; u < 3; ++u) {
+        const int v = 3 * lane + u, t = 9 * (v % 9) + v / 9, src = min(t / 3, 31);
+        const float t0 = __shfl_sync(0xffffffffu, h[0], src), t1 = __shfl_sync(0xffffffffu, h[1], src),
+                    t2 = __shfl_sync(0xffffffffu, h[2], src);
+        h[3 + u] = h[u] + (t % 3 == 0 ? t0 : t % 3 == 1 ? t1 : t2);
+      }
+#pragma unroll
+      for (int u = 0; u < 3; ++u) h[u] = h[3 + u];
+    }
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      const int v = 3 * lane + u, r = 9 * blk.x + v / 9, c = 9 * blk.y + v % 9;
+      if (v >= SX_PART) continue;
+      val[r * ld + c] = -h[u];
+      if (blk.x != blk.y) val[c * ld + r] = -h[u];
+    }
+  }
+}
+
+// S.ss = (S without its diagonal blocks) pf: a warp takes eight rows at a time,
+// a lane four columns.
+template <typename T>
+__device__ __forceinline__ void batch_formed_product(const BatchArgs<T>& a, const BRange<T>& R, BShared<T>& S, int b) {
+  constexpr int RB = 8;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int n = 9 * R.nc, l4 = sx_ld(R.nc) / 4;
+  const float4* val = reinterpret_cast<const float4*>(a.sx_val + a.sx_val_off[b]);
+  const float4* pf = reinterpret_cast<const float4*>(S.pf);
+  for (int r0 = RB * warp; r0 < n; r0 += RB * (BT / 32)) {
+    float acc[RB];
+#pragma unroll
+    for (int r = 0; r < RB; ++r) acc[r] = 0.f;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int c = lane + 32 * u;
+      if (c >= l4) continue;
+      float4 v[RB];
+#pragma unroll
+      for (int r = 0; r < RB; ++r) v[r] = val[min(r0 + r, n - 1) * l4 + c];
+      const float4 p = pf[c];
+#pragma unroll
+      for (int r = 0; r < RB; ++r) acc[r] += (v[r].x * p.x + v[r].y * p.y) + (v[r].z * p.z + v[r].w * p.w);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      float t[RB];
+#pragma unroll
+      for (int r = 0; r < RB; ++r) t[r] = __shfl_xor_sync(0xffffffffu, acc[r], off);
+#pragma unroll
+      for (int r = 0; r < RB; ++r) acc[r] += t[r];
+    }
+#pragma unroll
+    for (int r = 0; r < RB; ++r)
+      if (lane == r && r0 + r < n) S.ss[r0 + r] = (double)acc[r];
+  }
+}
+static_assert(sx_ld(BMAXC) <= 256, "a row of the formed system is two rounds of a warp's four-vectors");
+
 // The linearisation (a1 + a2) at the current parameters.
 template <typename T, bool MF>
 __device__ void batch_linearise(const BatchArgs<T>& a, const BRange<T>& R, BShared<T>& S, int cur) {
@@ -473,17 +634,20 @@ template <typename T, bool MODEL, bool MF>
 __device__ void batch_cost(const BatchArgs<T>& a, const BRange<T>& R, BShared<T>& S, int buf, int cur) {
   const T* pts = a.pts + (long long)buf * 3 * a.P;
   const T* pts_old = a.pts + (long long)cur * 3 * a.P;
+  // the camera tables, a thread each (one thread for one camera before every
+  // piece took 8 us a piece)
+  if (threadIdx.x < R.nc) {
+    double ct[CT];
+    camera_table_f64(a.cams + (long long)buf * 9 * a.C + 9LL * (R.c0 + threadIdx.x), ct);
+    for (int i = 0; i < CT_TAB64; ++i) S.sce64[threadIdx.x][i] = ct[i];
+    if (S.F32) ffcam_from(ct, S.sceff[S.F32 ? threadIdx.x : 0]);
+  }
+  __syncthreads();
   for (int q = R.q0; q < R.q1; ++q) {
-    const int cg = a.piece_cam[q];
-    const int c = cg - R.c0;
-    if (threadIdx.x == 0) {
-      camera_table_f64(a.cams + (long long)buf * 9 * a.C + 9LL * cg, S.sce64);
-      ffcam_from(S.sce64, S.sceff);
-    }
-    __syncthreads();
+    const int c = a.piece_cam[q] - R.c0;
     double cost = 0.0, quad = 0.0;
-    cost_cam_range<T, MODEL, MF, BT>(a.piece_beg[q], a.piece_end[q], a.cm_pt, a.cm_px, pts, pts_old, &S.sceff,
-                                     S.sce64, S.ct[c], S.xT[c], a.delta, a.O, a.Jcm, a.cm_sw, a.dp, cost, quad);
+    cost_cam_range<T, MODEL, MF, BT>(a.piece_beg[q], a.piece_end[q], a.cm_pt, a.cm_px, pts, pts_old, &S.sceff[S.F32 ? c : 0],
+                                     S.sce64[c], S.ct[c], S.xT[c], a.delta, a.O, a.Jcm, a.cm_sw, a.dp, cost, quad);
     double v[2] = {cost, quad};
     bred_store<2, true>(v, S.red, a.part + (long long)PART * q);
   }
@@ -514,6 +678,12 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
       bred_store<54, true>(acc, S.red, a.part + (long long)PART * q);
     }
   }
+  bool formed = false;
+  if constexpr (MF && sizeof(T) == 4) formed = a.sx_val != nullptr;
+  if (formed) {
+    if (tid == 0) S.next_blk = a.sx_off[b];
+    __syncthreads();
+  }
   if (tid < 32) {
     double rz = 0.0, bb = 0.0;
     int fb = 0;
@@ -521,7 +691,7 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
       const int cg = R.c0 + tid;
       cam_schur_one<T, MF, true>(a.cam_piece_ptr[cg], a.cam_piece_ptr[cg + 1], a.part, S.U + 45 * tid, S.gc + 9 * tid,
                            S.ct[tid], lam, a.dmin, a.dmax, nullptr, S.M + 45 * tid, S.x + 9 * tid, S.r + 9 * tid,
-                           S.z + 9 * tid, S.p + 9 * tid, S.pT[tid], rz, bb, fb);
+                           S.z + 9 * tid, S.p + 9 * tid, S.pT[tid], rz, bb, fb, S.F32 ? S.Sii + 45 * tid : nullptr);
     }
     const int nfb = __popc(__ballot_sync(0xffffffffu, fb != 0));
     rz = warp_total(rz);
@@ -529,11 +699,17 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
     if (tid == 0) {
       S.rz_old = rz;
       S.bb = bb;
+      S.stop = a.tol * sqrt(bb);
+      S.rr = 0.0;
       S.fallbacks = nfb;
       S.pcg_iters = 0;
       S.pcg_rel = 1.0;
     }
   }
+  // S formed by the other warps meanwhile (the first joins them when the
+  // cameras' blocks are factored)
+  if constexpr (MF && sizeof(T) == 4)
+    if (formed) batch_form<T>(a, R, S, b);
   __syncthreads();
 
   // a4: block-Jacobi PCG on S dc = b (thread lc*9 + i owns component i of
@@ -541,8 +717,14 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
   const int lc = tid / 9, ci = tid % 9;
   const bool ok = lc < R.nc;
   const int o = 9 * lc + ci;
+  if (formed) {
+    if (tid < sx_ld(R.nc)) S.pf[tid] = ok ? (T)S.p[o] : T(0);
+    __syncthreads();
+  }
   for (int k = 0; k < a.maxiter; ++k) {
-    if (MF) {
+    if (formed) {
+      if constexpr (MF && sizeof(T) == 4) batch_formed_product<T>(a, R, S, b);
+    } else if (MF) {
       batch_stage_fxv(S, R, S.pT);
       batch_pass_fa<T, 0>(a, R, S, cur);
     } else {
@@ -551,7 +733,7 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
       batch_pass_a2<T, 0>(a, R, S, cur);
     }
     __syncthreads();
-    for (int q = R.q0; q < R.q1; ++q) {
+    for (int q = formed ? R.q1 : R.q0; q < R.q1; ++q) {
       const int c = a.piece_cam[q] - R.c0;
       T ctl[15];
 #pragma unroll
@@ -568,14 +750,22 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
     double pv = 0.0, sum = 0.0;
     if (ok) {
       pv = S.p[o];
-      const int cg = R.c0 + lc;
-      const int p1 = a.cam_piece_ptr[cg + 1];
-      for (int kq = a.cam_piece_ptr[cg]; kq < p1; ++kq) sum += a.part[(long long)PART * kq + ci];
-      S.ss[o] = sum;
+      if (!formed) {
+        const int cg = R.c0 + lc;
+        const int p1 = a.cam_piece_ptr[cg + 1];
+        for (int kq = a.cam_piece_ptr[cg]; kq < p1; ++kq) sum += a.part[(long long)PART * kq + ci];
+        S.ss[o] = sum;
+      }
     }
-    __syncthreads();
+    if (!formed) __syncthreads();
     double qv = 0.0;
-    if (ok) {
+    if (ok && formed) {
+      const double* Sc = S.Sii + 45 * lc;
+      qv = S.ss[o];
+#pragma unroll
+      for (int j = 0; j < 9; ++j) qv += Sc[sym9_rt(ci, j)] * S.p[9 * lc + j];
+      S.red[tid] = pv * qv;
+    } else if (ok) {
       if (MF && ci < 3) {
         const T* Jl = S.ct[lc] + CT_JL;
         sum = (double)Jl[ci] * S.ss[9 * lc] + (double)Jl[3 + ci] * S.ss[9 * lc + 1] +
@@ -597,10 +787,7 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
     __syncthreads();
     const double alpha = S.tot[0];
     if (isnan(alpha)) {
-      if (tid == 0) {
-        S.pcg_iters = k;
-        if (k == 0) S.pcg_rel = 0.0;
-      }
+      if (tid == 0 && k == 0) S.pcg_rel = 0.0;
       break;
     }
     double rv = 0.0;
@@ -621,12 +808,11 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
     {
       double t[2];
       if (bred_warp0<2>(S, 9 * R.nc, t) && tid == 0) {
-        const double bb = S.bb;
         S.tot[0] = t[0] / S.rz_old;
-        S.tot[1] = sqrt(t[1]) <= a.tol * sqrt(bb) ? 1.0 : 0.0;
+        S.tot[1] = sqrt(t[1]) <= S.stop ? 1.0 : 0.0;
         S.rz_old = t[0];
+        S.rr = t[1];
         S.pcg_iters = k + 1;
-        S.pcg_rel = bb > 0.0 ? sqrt(t[1] / bb) : 0.0;
       }
     }
     __syncthreads();
@@ -636,7 +822,9 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
       S.p[o] = zz + beta * S.p[o];
     }
     __syncthreads();
-    if (ok) {
+    if (formed) {
+      if (ok) S.pf[o] = (T)S.p[o];
+    } else if (ok) {
       if (MF && ci < 3) {
         const T* Jl = S.ct[lc] + CT_JL;
         S.pT[lc][ci] = (T)((double)Jl[3 * ci] * S.p[9 * lc] + (double)Jl[3 * ci + 1] * S.p[9 * lc + 1] +
@@ -651,6 +839,7 @@ __device__ void batch_trial(const BatchArgs<T>& a, const BRange<T>& R, BShared<T
   __syncthreads();
 
   // a5: trial cameras, back-substitution and trial points
+  if (tid == 0 && S.pcg_iters > 0) S.pcg_rel = S.bb > 0.0 ? sqrt(S.rr / S.bb) : 0.0;
   if (tid < 32) {
     double gd = 0.0;
     if (tid < R.nc) {

@@ -18,6 +18,19 @@ namespace ba {
 ba_status problem_create(ba_problem** out, int C, int P, int O, const void* cams, const void* points,
                          const int32_t* cam_idx, const int32_t* pt_idx, const void* pixels, const ba_options* opt,
                          void* stream, bool batched);
+// The pairs of observations of each point, sorted by camera pair (device, n
+// each: camera-major slots of both, the point; freed with the object unless
+// kept), and where each camera pair begins.  n stays 0 above `most` pairs or
+// when there is no room.
+struct SchurPairs {
+  int n = 0;
+  int32_t *pk = nullptr, *pl = nullptr, *pj = nullptr;
+  std::vector<int32_t> head;
+  std::vector<int2> cam;
+  ~SchurPairs();
+  void keep(std::vector<void*>& allocs);
+};
+ba_status schur_pairs(ba_problem* h, const std::vector<int32_t>& rq, bool self, long long most, SchurPairs& out);
 // The reduced system formed explicitly (ba_schur.cu).  schur_build chooses
 // between it and the implicit product and builds what it needs (rq: the row
 // pointers of the observations by point); h->sx.pcg / h->sx.direct say what

@@ -116,79 +116,68 @@ struct SchurCost {
   }
   // forming: FP64 pipe (13 ns per 32 pairs), FP32 arithmetic and gathers
   double form_us(double pairs) const { return 25.0 + pairs * (f32 ? 5.0e-5 : 3.1e-4); }
+  // more pairs than this and forming alone takes longer
+  long long most_pairs(double O) const { return (long long)(std::max(0.0, implicit_us(O) - 25.0) / (f32 ? 5.0e-5 : 3.1e-4)); }
   // two exchanges, then 81 multiply-adds or 324 bytes a block
   double iter_us(double blocks) const { return 8.0 + 162.0 * blocks * (f32 ? 0.8e-6 : 1.7e-6); }
 };
 
 }  // namespace
 
-ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
-  const bool direct = h->opt.solver == BA_SOLVER_CHOLESKY;
-  const bool f32 = h->prec == BA_PREC_F32;
-  if (h->batched) return BA_OK;
+SchurPairs::~SchurPairs() {
+  for (int32_t* p : {pk, pl, pj}) cudaFree(p);
+}
+
+void SchurPairs::keep(std::vector<void*>& allocs) {
+  for (int32_t** p : {&pk, &pl, &pj}) {
+    allocs.push_back(*p);
+    *p = nullptr;
+  }
+}
+
+ba_status schur_pairs(ba_problem* h, const std::vector<int32_t>& rq, bool self, long long most, SchurPairs& out) {
   const int C = h->C, P = h->P, O = h->O;
-  const bool self = direct;
   std::vector<int32_t> poff(P + 1);
   long long np = 0;
   for (int j = 0; j < P; ++j) {
     const long long n = rq[j + 1] - rq[j];
     poff[j] = (int32_t)std::min<long long>(np, INT32_MAX);
     np += n * (n - 1) / 2 + (self ? n : 0);
-    if (np > MAX_PAIRS) return BA_OK;
+    if (np > std::min(most, MAX_PAIRS)) return BA_OK;
   }
   poff[P] = (int32_t)np;
   if (np == 0) return BA_OK;
-  const SchurCost cost{f32, h->opt.pcg_maxiter};
-  int dev = 0, nsm = 0, coop = 0;
-  SCU(cudaGetDevice(&dev));
-  SCU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  SCU(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-  int rpb = 1;
-  if (!direct) {
-    // FP64 that recomputes its Jacobians in every pass keeps the implicit
-    // product: a pair would recompute two observations in FP64
-    if (!coop || (!f32 && h->mf) || h->opt.pcg_maxiter < 1) return BA_OK;
-    if (cost.form_us((double)np) >= cost.implicit_us(O)) return BA_OK;
-    if (f32 && O > F32_MAX_OBS) return BA_OK;
-    rpb = (C + nsm - 1) / nsm;
-    if (rpb > SX_ROWS) return BA_OK;
-  }
   cudaStream_t s = h->s;
   const int n = (int)np;
-  std::vector<void*> tmp;  // freed on return, but for what keep() hands to the problem
+  // one allocation for everything that is not kept
+  const size_t scratch_bytes = csr_scratch_bytes(n);
+  auto al = [](size_t b) { return (b + 255) / 256 * 256; };
+  const size_t need = al(4ull * (P + 1)) + 7 * al(4ull * n) + al(4ull * (std::max(C, 2) + 1)) + al(8ull * n) +
+                      al(scratch_bytes);
+  char* base = nullptr;
+  cudaError_t e = cudaMalloc(&base, need);
+  for (int32_t** p : {&out.pk, &out.pl, &out.pj})
+    if (e == cudaSuccess) e = cudaMalloc(p, 4ull * n);
   struct Free {
-    std::vector<void*>& v;
-    ~Free() {
-      for (void* p : v) cudaFree(p);
-    }
-  } free_tmp{tmp};
-  auto grab = [&](auto** p, size_t bytes) {
-    void* v = nullptr;
-    const cudaError_t e = cudaMalloc(&v, std::max<size_t>(bytes, 16));
-    if (e == cudaSuccess) {
-      tmp.push_back(v);
-      *p = static_cast<std::remove_reference_t<decltype(**p)>*>(v);
-    }
-    return e;
-  };
-  int32_t *d_poff = nullptr, *ki = nullptr, *kl = nullptr, *sk = nullptr, *sl = nullptr, *perm_l = nullptr,
-          *perm_i = nullptr, *key = nullptr, *rows = nullptr;
-  int2* cams = nullptr;
-  void* scratch = nullptr;
-  cudaError_t e = grab(&d_poff, 4ull * (P + 1));
-  for (int32_t** p : {&ki, &kl, &sk, &sl, &perm_l, &perm_i, &key})
-    if (e == cudaSuccess) e = grab(p, 4ull * n);
-  if (e == cudaSuccess) e = grab(&rows, 4ull * (std::max(C, 2) + 1));
-  if (e == cudaSuccess) e = grab(&cams, 8ull * n);
-  if (e == cudaSuccess) e = grab((char**)&scratch, csr_scratch_bytes(n));
-  auto& x = h->sx;
-  int32_t *pk = nullptr, *pl = nullptr, *pj = nullptr;  // kept if S is formed
-  for (int32_t** p : {&pk, &pl, &pj})
-    if (e == cudaSuccess) e = grab(p, 4ull * n);
+    char* p;
+    ~Free() { cudaFree(p); }
+  } free_base{base};
   if (e != cudaSuccess) {
     cudaGetLastError();  // no room: the implicit product (or the dense build) as before
     return BA_OK;
   }
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    char* p = base + off;
+    off += al(bytes);
+    return p;
+  };
+  int32_t* d_poff = (int32_t*)take(4ull * (P + 1));
+  int32_t *ki = (int32_t*)take(4ull * n), *kl = (int32_t*)take(4ull * n), *sk = (int32_t*)take(4ull * n),
+          *sl = (int32_t*)take(4ull * n), *perm_l = (int32_t*)take(4ull * n), *perm_i = (int32_t*)take(4ull * n),
+          *key = (int32_t*)take(4ull * n), *rows = (int32_t*)take(4ull * (std::max(C, 2) + 1));
+  int2* cams = (int2*)take(8ull * n);
+  void* scratch = take(scratch_bytes);
   int* derr = &h->st->err;
   SCU(cudaMemcpyAsync(d_poff, poff.data(), 4ull * (P + 1), cudaMemcpyHostToDevice, s));
   k_pair_emit<<<nb_(O, 256), 256, 0, s>>>(O, self ? 1 : 0, h->rowptr_pt, d_poff, h->pm_pt, h->pm_cam, h->pm2cm, ki, kl,
@@ -196,7 +185,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   SCU(csr_build_async(kl, n, C, perm_l, rows, scratch, derr, s));
   k_pair_key<<<nb_(n, 256), 256, 0, s>>>(n, perm_l, ki, key);
   SCU(csr_build_async(key, n, C, perm_i, rows, scratch, derr, s));
-  k_pair_gather<<<nb_(n, 256), 256, 0, s>>>(n, perm_l, perm_i, ki, kl, sk, sl, h->cm_pt, pk, pl, pj, cams);
+  k_pair_gather<<<nb_(n, 256), 256, 0, s>>>(n, perm_l, perm_i, ki, kl, sk, sl, h->cm_pt, out.pk, out.pl, out.pj, cams);
   k_pair_heads<<<nb_(n, 256), 256, 0, s>>>(n, cams, key);
   SCU(csr_build_async(key, n, 2, perm_l, rows, scratch, derr, s));
   count_launch(4);
@@ -204,22 +193,54 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   SCU(cudaMemcpyAsync(hrow, rows, 12, cudaMemcpyDeviceToHost, s));
   SCU(cudaStreamSynchronize(s));
   const int nhead = hrow[1];
+  // the heads' cameras over ki and kl, which are adjacent and done with
+  int2* d_hcam = (int2*)ki;
+  k_pair_head_cams<<<nb_(nhead, 256), 256, 0, s>>>(nhead, perm_l, cams, d_hcam);
+  count_launch();
+  out.head.resize(nhead);
+  out.cam.resize(nhead);
+  SCU(cudaMemcpyAsync(out.head.data(), perm_l, 4ull * nhead, cudaMemcpyDeviceToHost, s));
+  SCU(cudaMemcpyAsync(out.cam.data(), d_hcam, 8ull * nhead, cudaMemcpyDeviceToHost, s));
+  SCU(cudaStreamSynchronize(s));
+  out.n = n;
+  return BA_OK;
+}
+
+ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
+  const bool direct = h->opt.solver == BA_SOLVER_CHOLESKY;
+  const bool f32 = h->prec == BA_PREC_F32;
+  if (h->batched) return BA_OK;
+  const int C = h->C, O = h->O;
+  const SchurCost cost{f32, h->opt.pcg_maxiter};
+  int dev = 0, nsm = 0, coop = 0;
+  SCU(cudaGetDevice(&dev));
+  SCU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  SCU(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+  int rpb = 1;
+  long long most = MAX_PAIRS;
+  if (!direct) {
+    // FP64 that recomputes its Jacobians in every pass keeps the implicit
+    // product: a pair would recompute two observations in FP64
+    if (!coop || (!f32 && h->mf) || h->opt.pcg_maxiter < 1) return BA_OK;
+    if (f32 && O > F32_MAX_OBS) return BA_OK;
+    rpb = (C + nsm - 1) / nsm;
+    if (rpb > SX_ROWS) return BA_OK;
+    most = cost.most_pairs(O);
+  }
+  SchurPairs pr;
+  const ba_status ps = schur_pairs(h, rq, direct, most, pr);
+  if (ps != BA_OK || pr.n == 0) return ps;
+  const int n = pr.n, nhead = (int)pr.head.size();
+  const long long np = n;
+  const std::vector<int32_t>& head = pr.head;
+  const std::vector<int2>& hcam = pr.cam;
+  auto& x = h->sx;
+  cudaStream_t s = h->s;
+  cudaError_t e = cudaSuccess;
   const size_t vs = direct || !f32 ? 8 : 4;
   if (!direct && (cost.form_us((double)np) + cost.iters() * cost.iter_us(nhead) >= cost.implicit_us(O) ||
                   2ull * nhead * SX_PART * vs > (16ull << 30)))
     return BA_OK;
-  int2* d_hcam = nullptr;
-  if (grab(&d_hcam, 8ull * nhead) != cudaSuccess) {
-    cudaGetLastError();
-    return BA_OK;
-  }
-  k_pair_head_cams<<<nb_(nhead, 256), 256, 0, s>>>(nhead, perm_l, cams, d_hcam);
-  count_launch();
-  std::vector<int32_t> head(nhead);
-  std::vector<int2> hcam(nhead);
-  SCU(cudaMemcpyAsync(head.data(), perm_l, 4ull * nhead, cudaMemcpyDeviceToHost, s));
-  SCU(cudaMemcpyAsync(hcam.data(), d_hcam, 8ull * nhead, cudaMemcpyDeviceToHost, s));
-  SCU(cudaStreamSynchronize(s));
 
   // tasks: about eight warps an SM a round and at least four rounds of lanes
   // where there are that many pairs (a task ends with 81 x 32 additions)
@@ -249,10 +270,11 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
     if (r == cudaSuccess) r = cudaMemcpy(*p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
     return r;
   };
-  auto keep = [&](int32_t** dst, int32_t* p) {
-    tmp.erase(std::find(tmp.begin(), tmp.end(), (void*)p));
-    h->allocs.push_back(p);
-    *dst = p;
+  auto keep = [&] {
+    x.pk = pr.pk;
+    x.pl = pr.pl;
+    x.pj = pr.pj;
+    pr.keep(h->allocs);
   };
   auto kernel_attr = [&](const void* k, int bytes) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -275,9 +297,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
       cudaGetLastError();
       return BA_OK;
     }
-    keep(&x.pk, pk);
-    keep(&x.pl, pl);
-    keep(&x.pj, pj);
+    keep();
     x.direct = true;
     x.lean = lean;
     return BA_OK;
@@ -368,9 +388,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
     cudaGetLastError();
     return BA_OK;
   }
-  keep(&x.pk, pk);
-  keep(&x.pl, pl);
-  keep(&x.pj, pj);
+  keep();
   x.groups = groups;
   x.rpb = rpb;
   x.pcg = true;
