@@ -102,6 +102,25 @@ __device__ __forceinline__ bool gx_gather(const GridX& gx, const unsigned long l
   return true;
 }
 
+// 1 / d: for a normal d well inside the range a third-order step
+// y (1 + r + r^2), r = 1 - m y, on the FP32 reciprocal of d's significand (error
+// 2^-23 -> below 2^-60, so the result is within an ulp), scaled and checked on
+// the integer side; else the division.  A warp issues an FP64 instruction in
+// some 70 cycles; the division's were on the PCG's critical path twice an
+// iteration (with 1 / rz taken while the sums travel and no square root in the
+// stopping test: sphere of 2,500 poses 2,514 -> 2,371 us, ring of 97 cameras
+// in FP32 757 -> 727 us).
+__device__ __forceinline__ double gx_rcp(double d) {
+  const int hi = __double2hiint(d), ex = hi >> 20;
+  if (ex < 23 || ex > 2023) return 1.0 / d;
+  const int up = (ex - 1023) * (1 << 20);
+  const double m = __hiloint2double(hi - up, __double2loint(d));
+  const double y = (double)(1.0f / (float)m);
+  const double r = fma(-m, y, 1.0);
+  const double z = fma(y, fma(r, r, r), y);  // in (1/2, 1]
+  return __hiloint2double(__double2hiint(z) - up, __double2loint(z));
+}
+
 // warp_sum of NV values, the trees interleaved (the shuffles of one keep their
 // program order: one tree after the other took twice the latency).
 template <int NV>
@@ -120,18 +139,19 @@ __device__ __forceinline__ void gx_warp_sums(double (&t)[NV]) {
 // turns them into what the block goes on with, finish(totals), NV numbers that
 // every thread of every block returns in v.  (A division or a square root in
 // every warp of a block of 16 cost 5 us: 16 cycles for each of their FP64
-// instructions and warp.)  Meanwhile the other warps run overlap(), which
-// returns false if it gave up.  Returns false in every thread of the block if
+// instructions and warp.)  It runs prepare() while its sums travel; meanwhile
+// the other warps run overlap(), which returns false if it gave up.  Returns false in every thread of the block if
 // a wait ran out.  set 0 or 1 alternates between calls, epoch is the call's
 // number in its set (1, 2, ...).  blockDim.x is a multiple of 32, at least 64
-// and at most NT; only the first nv threads (a multiple of 32) hold values.  The call begins and ends with a block barrier.
+// and at most NT; only the first nv threads (a multiple of 32) hold values.
+// The call begins and ends with a block barrier.
 //
 // One warp does the adding: an FP64 warp instruction takes 16 cycles of its
 // SM here, and a shuffle tree in every warp of every block was a quarter of a
 // PCG iteration.
-template <int NV, int NT, typename Finish, typename Overlap>
+template <int NV, int NT, typename Prepare, typename Finish, typename Overlap>
 __device__ __forceinline__ bool grid_exchange(const GridX& gx, int set, unsigned int epoch, double (&v)[NV], int nv,
-                                              Finish finish, Overlap overlap) {
+                                              Prepare prepare, Finish finish, Overlap overlap) {
   static_assert(2 * NV <= GX_WORDS, "a slot holds two doubles");
   __shared__ double s_v[NV][NT];
   __shared__ double s_tot[NV];
@@ -156,6 +176,7 @@ __device__ __forceinline__ bool grid_exchange(const GridX& gx, int set, unsigned
       for (int i = 0; i < NV; ++i)
         gx_put(base + ((size_t)lane * G + blockIdx.x) * GX_WORDS + 2 * i, epoch, t[i]);
     }
+    prepare();
     constexpr int U = 5;  // slots of a lane in flight: 160 blocks a round
     const unsigned long long* mine = base + (size_t)(blockIdx.x % GX_COPIES) * G * GX_WORDS;
     bool ok = true;

@@ -819,12 +819,13 @@ static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg_res(PcgAr
   double rz, rr = 0.0;
   {
     double v[1] = {rz_part};
-    if (!grid_exchange<1, PGO_PCG_THREADS>(a.gx, 1, 1, v, blockDim.x, [](double(&)[1]) {}, [&] { return fetch_z(1); })) return;
+    if (!grid_exchange<1, PGO_PCG_THREADS>(a.gx, 1, 1, v, blockDim.x, [] {}, [](double(&)[1]) {}, [&] { return fetch_z(1); })) return;
     rz = v[0];
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   const int wsl = lane / 6, wrow = lane % 6;  // five slots a warp, lanes 30 and 31 idle
-  const double stop = a.tol * bnorm;
+  const double stop = (a.tol * bnorm) * (a.tol * bnorm);
+  double inv_rz = 0.0;
   double beta = 0.0;
   int it = 0;
   while (it < a.maxiter) {
@@ -882,9 +883,9 @@ static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg_res(PcgAr
     double alpha;
     {
       double v[1] = {live ? pa * qa : 0.0};
-      if (!grid_exchange<1, PGO_PCG_THREADS>(a.gx, 0, it + 1, v, blockDim.x,
-                                             [&](double(&t)[1]) { t[0] = t[0] > 0.0 ? rz / t[0] : nan(""); },
-                                             [] { return true; }))
+      if (!grid_exchange<1, PGO_PCG_THREADS>(
+              a.gx, 0, it + 1, v, blockDim.x, [&] { inv_rz = gx_rcp(rz); },
+              [&](double(&t)[1]) { t[0] = t[0] > 0.0 ? rz * gx_rcp(t[0]) : nan(""); }, [] { return true; }))
         return;
       alpha = v[0];
     }
@@ -911,13 +912,12 @@ static __global__ void __launch_bounds__(PGO_PCG_THREADS, 1) k_pgo_pcg_res(PcgAr
     {
       double v[2] = {rr_part, rzp};
       if (!grid_exchange<2, PGO_PCG_THREADS>(
-              a.gx, 1, it + 1, v, blockDim.x,
+              a.gx, 1, it + 1, v, blockDim.x, [] {},
               [&](double(&t)[2]) {
                 rr = t[0];
-                const double rz_new = t[1];
-                t[0] = sqrt(rr) <= stop ? 1.0 : 0.0;
-                t[1] = rz_new / rz;
-                rz = rz_new;
+                rz = t[1];
+                t[0] = rr <= stop ? 1.0 : 0.0;
+                t[1] = rz * inv_rz;
               },
               [&] { return fetch_z(it + 1); }))
         return;

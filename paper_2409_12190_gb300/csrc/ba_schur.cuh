@@ -529,14 +529,15 @@ static __global__ void __launch_bounds__(SX_THREADS, 1) k_schur_pcg(SchurPcg<VT>
     v2[0] = za * ra;
     v2[1] = ra * ra;
   }
-  if (!grid_exchange<2, SX_THREADS>(a.gx, 1, 1, v2, nv, [](double(&)[2]) {}, [&] { return fetch_z(1); })) return;
-  // the polling warp keeps r . z and the last |r|^2; |b|^2 and the bound of |r|
+  bool lost = !grid_exchange<2, SX_THREADS>(a.gx, 1, 1, v2, nv, [] {}, [](double(&)[2]) {}, [&] { return fetch_z(1); });
+  // the polling warp keeps r . z and the last |r|^2; |b|^2 and the bound of |r|^2
   double rz = v2[0], rr = 0.0;
   const double bb = v2[1];
-  const double stop = warp == 0 ? a.tol * sqrt(bb) : 0.0;
+  const double stop = warp == 0 ? a.tol * a.tol * bb : 0.0;
+  double inv_rz = 0.0;
   double beta = 0.0;
   int it = 0, done = 0;
-  while (it < a.maxiter) {
+  while (!lost && it < a.maxiter) {
     for (int e = tid; e < 9 * nc; e += blockDim.x) sp[e] = sz[e] + beta * sp[e];
     pa = za + beta * pa;
     __syncthreads();
@@ -568,9 +569,12 @@ static __global__ void __launch_bounds__(SX_THREADS, 1) k_schur_pcg(SchurPcg<VT>
     // alpha = r . z / p . S p, or NaN to stop: no positive curvature (b = 0 or
     // breakdown) keeps x
     if (!grid_exchange<1, SX_THREADS>(
-            a.gx, 0, it + 1, v1, nv,
-            [&](double(&t)[1]) { t[0] = t[0] > 0.0 && isfinite(t[0]) ? rz / t[0] : nan(""); }, [] { return true; }))
-      return;
+            a.gx, 0, it + 1, v1, nv, [&] { inv_rz = gx_rcp(rz); },
+            [&](double(&t)[1]) { t[0] = t[0] > 0.0 && isfinite(t[0]) ? rz * gx_rcp(t[0]) : nan(""); },
+            [] { return true; })) {
+      lost = true;
+      break;
+    }
     const double alpha = v1[0];
     if (isnan(alpha)) {
       done = 1;
@@ -592,27 +596,30 @@ static __global__ void __launch_bounds__(SX_THREADS, 1) k_schur_pcg(SchurPcg<VT>
     ++it;
     // beta and whether |r| <= tol |b|
     if (!grid_exchange<2, SX_THREADS>(
-            a.gx, 1, it + 1, v2, nv,
+            a.gx, 1, it + 1, v2, nv, [] {},
             [&](double(&t)[2]) {
-              const double rz_new = t[0];
+              rz = t[0];
               rr = t[1];
-              t[0] = rz_new / rz;
-              t[1] = sqrt(rr) <= stop ? 1.0 : 0.0;
-              rz = rz_new;
+              t[0] = rz * inv_rz;
+              t[1] = rr <= stop ? 1.0 : 0.0;
             },
-            [&] { return fetch_z(it + 1); }))
-      return;
+            [&] { return fetch_z(it + 1); })) {
+      lost = true;
+      break;
+    }
     beta = v2[0];
     if (v2[1] != 0.0) {
       done = 1;
       break;
     }
   }
-  if (live) a.x[o] = xa;
+  // a wait that ran out: no step, counted (as the direct solver does)
+  if (live) a.x[o] = lost ? 0.0 : xa;
   if (g == 0 && tid == 0) {
+    if (lost) a.st->fallbacks += 1;
     a.st->pcg_iters = it;
-    a.st->pcg_rel = it > 0 ? (bb > 0.0 ? sqrt(rr / bb) : 0.0) : done ? 0.0 : 1.0;
-    a.st->pcg_done = done;
+    a.st->pcg_rel = lost ? 1.0 : it > 0 ? (bb > 0.0 ? sqrt(rr / bb) : 0.0) : done ? 0.0 : 1.0;
+    a.st->pcg_done = done | lost;
   }
 }
 
