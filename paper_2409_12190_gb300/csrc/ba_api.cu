@@ -320,17 +320,13 @@ void enqueue_dense_solve(ba_problem* h, const double* lam_ptr) {
   count_launch(3);
   }
   cudaMemsetAsync(h->bflag, 0, sizeof(int) * h->bflag_count, s);
+  const BandShape sh{h->bnb, h->bwt, h->bnb, h->bnb};  // the whole triangle: from the top
   if (h->bnb * BAND_TB > n) {
-    k_band_pad<<<1, BAND_TB, 0, s>>>(n, h->bnb, h->bwt, h->bT);
+    k_band_pad<<<1, BAND_TB, 0, s>>>(n, sh, h->bT);
     count_launch();
   }
-  const size_t ntile = (size_t)h->bnb * (h->bwt + 1);
-  int* ctr = h->bflag + 2 * ntile;
-  BandArgs ba_{h->bnb, h->bwt, n, h->bntask, h->bncrit, h->band_crit, h->btask, h->bT, h->brs, h->bUi, h->r,
-               h->dy, h->x, h->bflag, h->bflag + ntile, ctr, ctr + 5, ctr + 6};
-  void* args[] = {&ba_};
-  cudaLaunchCooperativeKernel((const void*)k_band_chol, dim3(h->band_grid), dim3(BAND_THREADS), args, 0, s);
-  k_band_finish<<<nblk(n, 256), 256, 0, s>>>(n, ctr + 5, ctr, h->x, h->st);
+  band_chol(sh, n, h->bntask, h->bncrit, h->band_crit, h->btask, h->bT, h->brs, h->bUi, h->r, h->dy, h->x, h->bflag,
+            h->band_grid, h->st, s);
   count_launch(2);
 }
 
@@ -890,7 +886,7 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
     if (h->bncrit == 0) h->band_crit = 0;
     h->bntask = (int)tasks.size();
     h->bT_bytes = (size_t)h->bnb * (h->bwt + 1) * (BAND_TB * BAND_TB) * sizeof(double);
-    h->bflag_count = 2 * (size_t)h->bnb * (h->bwt + 1) + 6 + h->bnb;
+    h->bflag_count = band_flags(BandShape{h->bnb, h->bwt, h->bnb, h->bnb});
     CU(h->alloc(&h->bT, h->bT_bytes));
     CU(h->alloc(&h->brs, 8ull * h->bnb * BAND_TB));
     CU(h->alloc(&h->bUi, 8ull * h->bnb * BAND_TB * BAND_TB));

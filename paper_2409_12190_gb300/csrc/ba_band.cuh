@@ -7,14 +7,15 @@
 //
 // Storage.  In the factored order (for the pose graphs, reverse
 // Cuthill-McKee when narrower) the matrix has half-bandwidth bw unknowns, so
-// its lower triangle lies in the TB x TB tiles (I, J) with
-// 0 <= I - J <= bwt = ceil(bw / TB).  Only those
-// tiles are stored: tile (I, J) at T + (J (bwt + 1) + I - J) TB^2, row-major.
-// The order is padded to nb TB unknowns with identity rows.  Cholesky keeps
-// the fill inside the band, so L takes the same tiles.
+// its lower triangle lies in the TB x TB tiles of block rows at most
+// bwt = ceil(bw / TB) apart.  Only those tiles are stored.  The block rows
+// are eliminated in the order of BandShape (ba_band_sched.h): from the top,
+// or from both ends towards the middle; I and J are positions in that order,
+// tile (I, J) lies at T + (J (bwt + 1) + slot(I, J)) TB^2, row-major.  The
+// matrix is padded to nb TB unknowns with identity rows.  Cholesky keeps the
+// fill inside the band, so L takes the same tiles.
 //
-// Tasks (a dependency graph; K0(I) = max(0, I - bwt) is the first column
-// that reaches row I):
+// Tasks (a dependency graph):
 //   D_J     the diagonal chain: L_{J,J-1} = A_{J,J-1} L_{J-1,J-1}^{-T}, then
 //           A_JJ -= L_{J,J-1} L_{J,J-1}^T and L_JJ = chol(A_JJ);
 //   U       A_IJ -= L_IK L_JK^T for K in [Ka, Ka + cnt): the updates of a
@@ -24,7 +25,8 @@
 //           triangular solves below are products, not serial substitutions;
 //   F_J     y_J = U_J^T (b_J - sum_K L_JK y_K);
 //   B_I     x_I = U_I (y_I - sum_K L_KI^T x_K).
-// The chain D_0, D_1, ... is the critical path; one D_J is a triangular
+// A chain D_0, D_1, ... is the critical path (33 us a step; from both ends
+// two run at once, and the middle's follows them); one D_J is a triangular
 // solve, a symmetric update and a factorisation of single tiles, while the U
 // and T tasks of later columns run beside it.  The host orders the tasks by
 // a list-scheduling simulation (a topological order) and splits them into two
@@ -35,7 +37,7 @@
 // predecessor done; if no block holds it, every block of its pool holds an
 // earlier task of the same pool, which is impossible.  So the schedule cannot
 // deadlock; every wait is bounded all the same (2^25 polls, about a second or
-// more), and one that runs out sets ctr[3], after which every block stops.
+// more), and one that runs out sets BAND_LOST, after which every block stops.
 //
 // Each entry of L is a fixed-order sum (K ascending, then the tile's own
 // columns), so the result does not depend on the schedule.
@@ -56,9 +58,9 @@ constexpr int BAND_TRI = BAND_TB * (BAND_TB + 1) / 2;  // entries of a tile's lo
 
 // The launch's arguments; the tasks are ba_band_sched.h's BandTask records,
 // read as int4.
+template <typename Shape>  // BandShape or BandTop
 struct BandArgs {
-  int nb;             // block rows of the padded order (nb * TB >= n)
-  int bwt;            // half-bandwidth in tiles
+  Shape sh;       // block rows (nb * TB >= n), half-bandwidth and elimination order
   int n;              // unknowns
   int ntask;          // tasks
   int ncrit;          // the near-diagonal pool's tasks (the first ncrit of the list)
@@ -68,32 +70,43 @@ struct BandArgs {
   double* rsd;        // [nb TB] 1 / L_cc of every diagonal entry
   double* Ui;         // [nb TB TB] U_J = L_JJ^{-T}, row-major (upper triangular)
   const double* rhs;  // [n] b
-  double* y;          // [nb TB] y, then x
+  double* y;          // [nb TB] y, then x, in elimination order
   double* sol;        // [n] x
   int* tflag;         // [nb (bwt + 1)] tile final (L)
   int* tprog;         // [nb (bwt + 1)] updates applied to the tile
-  int* ctr;           // [0] bulk ticket, [1] forward blocks done, [2] backward blocks done, [3] a wait ran out,
-                      // [4] near-diagonal ticket
-  int* fail;          // a pivot not positive or not finite
+  int* ctr;           // BAND_CTRS counters
   int* iflag;         // [nb] U_J final
 };
 
-__device__ __forceinline__ long long band_index(const BandArgs& a, int I, int J) {
-  return (long long)J * (a.bwt + 1) + (I - J);
+// The counters, before iflag.
+enum {
+  BAND_BULK = 0,   // the bulk pool's ticket
+  BAND_FWD = 1,    // forward blocks done of each chain, in its order (3)
+  BAND_BWD = 4,    // backward blocks done of each chain (3)
+  BAND_LOST = 7,   // a wait ran out
+  BAND_NEAR = 8,   // the near-diagonal pool's ticket
+  BAND_FAIL = 9,   // a pivot not positive or not finite
+  BAND_CTRS = 10
+};
+
+// The factorisation's flags: tflag, tprog, counters, iflag.
+inline size_t band_flags(const BandShape& sh) {
+  return 2 * (size_t)sh.nb * (sh.bwt + 1) + BAND_CTRS + sh.nb;
 }
 
-__device__ __forceinline__ double* band_tile(const BandArgs& a, int I, int J) {
-  return a.T + band_index(a, I, J) * (BAND_TB * BAND_TB);
+template <typename S>
+__device__ __forceinline__ double* band_tile(const BandArgs<S>& a, int I, int J) {
+  return a.T + a.sh.index(I, J) * (BAND_TB * BAND_TB);
 }
 
-__device__ __forceinline__ int* band_flag(const BandArgs& a, int I, int J) { return a.tflag + band_index(a, I, J); }
+template <typename S>
+__device__ __forceinline__ int* band_flag(const BandArgs<S>& a, int I, int J) { return a.tflag + a.sh.index(I, J); }
 
-__device__ __forceinline__ int* band_prog(const BandArgs& a, int I, int J) { return a.tprog + band_index(a, I, J); }
-
-__device__ __forceinline__ int band_k0(const BandArgs& a, int I) { return max(0, I - a.bwt); }
+template <typename S>
+__device__ __forceinline__ int* band_prog(const BandArgs<S>& a, int I, int J) { return a.tprog + a.sh.index(I, J); }
 
 // Thread-0 wait until *flag >= v (acquire).  False when the wait ran out or
-// another one did (ctr[3]).
+// another one did (BAND_LOST).
 static __device__ __noinline__ bool band_wait(int* flag, int v, int* err) {
   cuda::atomic_ref<int, cuda::thread_scope_device> f(*flag), e(*err);
   unsigned int spins = 0;
@@ -209,22 +222,23 @@ static __device__ void band_potrf(BandSmem& s) {
 
 // D_J: the subdiagonal tile's solve, the last update of the diagonal tile
 // and its factorisation.
-static __device__ bool band_task_D(const BandArgs& a, BandSmem& s, int J) {
+template <typename S>
+static __device__ bool band_task_D(const BandArgs<S>& a, BandSmem& s, int J) {
   constexpr int TB = BAND_TB;
   const int tid = threadIdx.x;
-  if (J >= 1 && a.bwt >= 1) {
+  if (a.sh.chained(J)) {
     // tiles (J, J - 1) and (J, J) hold every update before K = J - 1
     // (the two tiles of row J usually finish first: stage them while
     // L_{J-1,J-1} is still being factored)
-    const int nupd = (J - 1) - band_k0(a, J);
     int w = 1;
     if (tid == 0)
-      w = band_wait(band_prog(a, J, J - 1), nupd, a.ctr + 3) && band_wait(band_prog(a, J, J), nupd, a.ctr + 3);
+      w = band_wait(band_prog(a, J, J - 1), a.sh.updates(J, J - 1, J - 1), a.ctr + BAND_LOST) &&
+          band_wait(band_prog(a, J, J), a.sh.updates(J, J, J - 1), a.ctr + BAND_LOST);
     if (!__syncthreads_and(w)) return false;
     band_stage(s.A, band_tile(a, J, J - 1));
     band_stage(s.C, band_tile(a, J, J));
     w = 1;
-    if (tid == 0) w = band_wait(band_flag(a, J - 1, J - 1), 1, a.ctr + 3);
+    if (tid == 0) w = band_wait(band_flag(a, J - 1, J - 1), 1, a.ctr + BAND_LOST);
     if (!__syncthreads_and(w)) return false;
     band_stage(s.B, band_tile(a, J - 1, J - 1));
     if (tid < TB) s.rs[tid] = __ldcg(a.rsd + (long long)(J - 1) * TB + tid);
@@ -248,19 +262,20 @@ static __device__ bool band_task_D(const BandArgs& a, BandSmem& s, int J) {
   band_potrf(s);  // s.C = L_JJ
   band_store(band_tile(a, J, J), s.C);
   if (tid < TB) a.rsd[(long long)J * TB + tid] = s.rs[tid];
-  if (tid == 0 && s.bad) atomicExch(a.fail, 1);
+  if (tid == 0 && s.bad) atomicExch(a.ctr + BAND_FAIL, 1);
   band_publish(band_flag(a, J, J), 1);
   return true;
 }
 
 // U: A_IJ -= L_IK L_JK^T for K = Ka .. Ka + cnt - 1, after the tile's
 // earlier updates.
-static __device__ bool band_task_U(const BandArgs& a, BandSmem& s, int I, int J, int Ka, int cnt) {
+template <typename S>
+static __device__ bool band_task_U(const BandArgs<S>& a, BandSmem& s, int I, int J, int Ka, int cnt) {
   constexpr int TB = BAND_TB, E = TB * TB / BAND_THREADS, RS = BAND_THREADS / TB;
   const int tid = threadIdx.x, col = tid % TB, row0 = tid / TB;
-  const int k0 = band_k0(a, I);
+  const int before = a.sh.updates(I, J, Ka);
   int w = 1;
-  if (tid == 0) w = band_wait(band_prog(a, I, J), Ka - k0, a.ctr + 3);
+  if (tid == 0) w = band_wait(band_prog(a, I, J), before, a.ctr + BAND_LOST);
   if (!__syncthreads_and(w)) return false;
   double* Tij = band_tile(a, I, J);
   double acc[E];
@@ -268,7 +283,7 @@ static __device__ bool band_task_U(const BandArgs& a, BandSmem& s, int I, int J,
   for (int m = 0; m < E; ++m) acc[m] = __ldcg(Tij + (row0 + m * RS) * TB + col);
   for (int K = Ka; K < Ka + cnt; ++K) {
     w = 1;
-    if (tid == 0) w = band_wait(band_flag(a, I, K), 1, a.ctr + 3) && band_wait(band_flag(a, J, K), 1, a.ctr + 3);
+    if (tid == 0) w = band_wait(band_flag(a, I, K), 1, a.ctr + BAND_LOST) && band_wait(band_flag(a, J, K), 1, a.ctr + BAND_LOST);
     if (!__syncthreads_and(w)) return false;
     band_stage(s.A, band_tile(a, I, K));
     if (I != J) band_stage(s.B, band_tile(a, J, K));
@@ -284,17 +299,18 @@ static __device__ bool band_task_U(const BandArgs& a, BandSmem& s, int I, int J,
   }
 #pragma unroll
   for (int m = 0; m < E; ++m) Tij[(row0 + m * RS) * TB + col] = acc[m];
-  band_publish(band_prog(a, I, J), Ka + cnt - k0);
+  band_publish(band_prog(a, I, J), before + cnt);
   return true;
 }
 
 // T: L_IJ = A_IJ L_JJ^{-T} (I >= J + 2) after the tile's updates.
-static __device__ bool band_task_T(const BandArgs& a, BandSmem& s, int I, int J) {
+template <typename S>
+static __device__ bool band_task_T(const BandArgs<S>& a, BandSmem& s, int I, int J) {
   constexpr int TB = BAND_TB;
   const int tid = threadIdx.x;
   int w = 1;
   if (tid == 0)
-    w = band_wait(band_flag(a, J, J), 1, a.ctr + 3) && band_wait(band_prog(a, I, J), J - band_k0(a, I), a.ctr + 3);
+    w = band_wait(band_flag(a, J, J), 1, a.ctr + BAND_LOST) && band_wait(band_prog(a, I, J), a.sh.updates(I, J, J), a.ctr + BAND_LOST);
   if (!__syncthreads_and(w)) return false;
   band_stage(s.A, band_tile(a, I, J));
   band_stage(s.B, band_tile(a, J, J));
@@ -307,11 +323,12 @@ static __device__ bool band_task_T(const BandArgs& a, BandSmem& s, int I, int J)
 }
 
 // I_J: U_J = L_JJ^{-T}, the solution of X L_JJ^T = identity.
-static __device__ bool band_task_I(const BandArgs& a, BandSmem& s, int J) {
+template <typename S>
+static __device__ bool band_task_I(const BandArgs<S>& a, BandSmem& s, int J) {
   constexpr int TB = BAND_TB;
   const int tid = threadIdx.x;
   int w = 1;
-  if (tid == 0) w = band_wait(band_flag(a, J, J), 1, a.ctr + 3);
+  if (tid == 0) w = band_wait(band_flag(a, J, J), 1, a.ctr + BAND_LOST);
   if (!__syncthreads_and(w)) return false;
   band_stage(s.B, band_tile(a, J, J));
   if (tid < TB) s.rs[tid] = __ldcg(a.rsd + (long long)J * TB + tid);
@@ -340,28 +357,40 @@ __device__ __forceinline__ bool band_wait_count(int* p, int v, int* known, int* 
 }
 
 // Forward block F_J: y_J = L_JJ^{-1} (b_J - sum_{K < J} L_JK y_K).
-static __device__ bool band_forward_task(const BandArgs& a, BandSmem& s, int J) {
+template <typename S>
+static __device__ bool band_forward_task(const BandArgs<S>& a, BandSmem& s, int J) {
   constexpr int TB = BAND_TB;
   const int tid = threadIdx.x, r = tid / 8, q = tid % 8;  // row r, columns 4q .. 4q + 3
-  int known = 0;                                         // forward blocks known done (thread 0)
+  int known[3] = {0, 0, 0};                              // forward blocks known done (thread 0)
   double part = 0.0;
-  for (int K = max(0, J - a.bwt); K < J; ++K) {
+  const int cj = a.sh.chain(J);
+  // the columns of row J: of the top, then the rest
+  int K = cj == 1 ? a.sh.first_rest(J) : a.sh.first_top(J);
+  while (K < J) {
+    if (cj == 2 && K == a.sh.top) K = a.sh.first_rest(J);
+    const int ck = a.sh.chain(K);
     int w = 1;
-    if (tid == 0)
-      w = band_wait(band_flag(a, J, K), 1, a.ctr + 3) && band_wait_count(a.ctr + 1, K + 1, &known, a.ctr + 3);
+    if (tid == 0) {
+      w = band_wait(band_flag(a, J, K), 1, a.ctr + BAND_LOST);
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        if (w && c == ck)
+          w = band_wait_count(a.ctr + BAND_FWD + c, K - a.sh.chain_begin(c) + 1, known + c, a.ctr + BAND_LOST);
+    }
     if (!__syncthreads_and(w)) return false;
     const double* L = band_tile(a, J, K) + r * TB + 4 * q;
     const double* yk = a.y + (long long)K * TB + 4 * q;
 #pragma unroll
     for (int c = 0; c < 4; ++c) part = fma(__ldcg(L + c), __ldcg(yk + c), part);
+    ++K;
   }
   part += __shfl_xor_sync(0xffffffffu, part, 4);
   part += __shfl_xor_sync(0xffffffffu, part, 2);
   part += __shfl_xor_sync(0xffffffffu, part, 1);
-  const long long row = (long long)J * TB + r;
+  const long long row = (long long)a.sh.row_of(J) * TB + r;
   if (q == 0) s.d[r] = (row < a.n ? a.rhs[row] : 0.0) - part;
   int w = 1;
-  if (tid == 0) w = band_wait(a.iflag + J, 1, a.ctr + 3);
+  if (tid == 0) w = band_wait(a.iflag + J, 1, a.ctr + BAND_LOST);
   if (!__syncthreads_and(w)) return false;
   {
     // y = U_J^T v: lane r, rows c = wp, wp + 8, ... of U_J, summed over the
@@ -383,27 +412,43 @@ static __device__ bool band_forward_task(const BandArgs& a, BandSmem& s, int J) 
       a.y[(long long)J * TB + lane] = v;
     }
   }
-  // blocks are published in order (F_{J-1} first)
+  // a chain's blocks are published in order
+  const int done = J - a.sh.chain_begin(cj);
   w = 1;
-  if (tid == 0) w = band_wait_count(a.ctr + 1, J, &known, a.ctr + 3);
+  if (tid == 0) w = band_wait(a.ctr + BAND_FWD + cj, done, a.ctr + BAND_LOST);
   if (!__syncthreads_and(w)) return false;
-  band_publish(a.ctr + 1, J + 1);
+  band_publish(a.ctr + BAND_FWD + cj, done + 1);
   return true;
 }
 
 // Backward block B_I: x_I = L_II^{-T} (y_I - sum_{K > I} L_KI^T x_K); x
 // overwrites y.
-static __device__ bool band_backward_task(const BandArgs& a, BandSmem& s, int I) {
+template <typename S>
+static __device__ bool band_backward_task(const BandArgs<S>& a, BandSmem& s, int I) {
   constexpr int TB = BAND_TB;
   const int tid = threadIdx.x, lane = tid % 32, wp = tid / 32;  // x row lane; L rows wp, wp + 8, ...
-  int known = 0;                                                // backward blocks known done (thread 0)
+  int known[3] = {0, 0, 0};                                     // backward blocks known done (thread 0)
+  const int ci = a.sh.chain(I), cl = a.sh.chain(a.sh.nb - 1);
   int w = 1;
-  if (tid == 0) w = band_wait(a.ctr + 1, a.nb, a.ctr + 3);  // every tile and y final
+  // every y final (the last chain's forward blocks come after the others'), so every tile
+  if (tid == 0) w = band_wait(a.ctr + BAND_FWD + cl, a.sh.nb - a.sh.chain_begin(cl), a.ctr + BAND_LOST);
   if (!__syncthreads_and(w)) return false;
   double part = 0.0;
-  for (int K = min(a.nb - 1, I + a.bwt); K > I; --K) {
+  // the rows of column I: of the middle, then of its own chain, descending
+  const int end = a.sh.chain_end(ci);
+  for (int K = a.sh.nb - 1; K > I; --K) {
+    if (K >= end && K < a.sh.joint) K = end - 1;                                    // the other end
+    if (K < end && K - I > a.sh.bwt) K = I + a.sh.bwt;
+    if (K <= I) break;
+    if (a.sh.slot(K, I) > a.sh.bwt) continue;
+    const int ck = a.sh.chain(K);
     w = 1;
-    if (tid == 0) w = band_wait_count(a.ctr + 2, a.nb - K, &known, a.ctr + 3);
+    if (tid == 0) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c)
+        if (c == ck)
+          w = band_wait_count(a.ctr + BAND_BWD + c, a.sh.chain_end(c) - K, known + c, a.ctr + BAND_LOST);
+    }
     if (!__syncthreads_and(w)) return false;
     const double* L = band_tile(a, K, I);
     const double* xk = a.y + (long long)K * TB;
@@ -433,22 +478,23 @@ static __device__ bool band_backward_task(const BandArgs& a, BandSmem& s, int I)
     p += __shfl_xor_sync(0xffffffffu, p, 4);
     p += __shfl_xor_sync(0xffffffffu, p, 2);
     p += __shfl_xor_sync(0xffffffffu, p, 1);
-    const long long row = (long long)I * TB + r;
+    const long long row = (long long)a.sh.row_of(I) * TB + r;
     if (q == 0) {
-      a.y[row] = p;
+      a.y[(long long)I * TB + r] = p;
       if (row < a.n) a.sol[row] = p;
     }
   }
   w = 1;
-  if (tid == 0) w = band_wait_count(a.ctr + 2, a.nb - 1 - I, &known, a.ctr + 3);
+  if (tid == 0) w = band_wait(a.ctr + BAND_BWD + ci, end - 1 - I, a.ctr + BAND_LOST);
   if (!__syncthreads_and(w)) return false;
-  band_publish(a.ctr + 2, a.nb - I);
+  band_publish(a.ctr + BAND_BWD + ci, end - I);
   return true;
 }
 
 // The whole factorisation and both solves; launched cooperatively so that
 // every block is resident.
-static __global__ void __launch_bounds__(BAND_THREADS, 1) k_band_chol(BandArgs a) {
+template <typename S>
+static __global__ void __launch_bounds__(BAND_THREADS, 1) k_band_chol(BandArgs<S> a) {
   __shared__ BandSmem s;
   for (int e = threadIdx.x; e < BAND_TRI; e += BAND_THREADS) {
     int r = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);  // FP32 guess, corrected below
@@ -460,7 +506,8 @@ static __global__ void __launch_bounds__(BAND_THREADS, 1) k_band_chol(BandArgs a
   const int lim = near ? a.ncrit : a.ntask;
   for (;;) {
     if (threadIdx.x == 0)
-      s.task = band_load(a.ctr + 3) ? lim : (near ? 0 : a.ncrit) + atomicAdd(a.ctr + (near ? 4 : 0), 1);
+      s.task = band_load(a.ctr + BAND_LOST) ? lim
+                                           : (near ? 0 : a.ncrit) + atomicAdd(a.ctr + (near ? BAND_NEAR : BAND_BULK), 1);
     __syncthreads();
     const int q = s.task;
     __syncthreads();
@@ -480,18 +527,17 @@ static __global__ void __launch_bounds__(BAND_THREADS, 1) k_band_chol(BandArgs a
 }
 
 // Identity rows of the padding (n .. nb TB - 1) on the zeroed tiles.
-static __global__ void k_band_pad(int n, int nb, int bwt, double* __restrict__ T) {
+static __global__ void k_band_pad(int n, BandShape sh, double* __restrict__ T) {
   const int R = n + blockIdx.x * blockDim.x + threadIdx.x;
-  if (R >= nb * BAND_TB) return;
-  const int I = R / BAND_TB;
-  T[(long long)I * (bwt + 1) * (BAND_TB * BAND_TB) + (R % BAND_TB) * (BAND_TB + 1)] = 1.0;
+  if (R >= sh.nb * BAND_TB) return;
+  const int J = sh.place_of(R / BAND_TB);
+  T[sh.index(J, J) * (BAND_TB * BAND_TB) + (R % BAND_TB) * (BAND_TB + 1)] = 1.0;
 }
 
 // After k_band_chol: a failed factorisation (a pivot not positive or not
 // finite) or a wait that ran out gives x = 0, counted; the solve's statistics.
-static __global__ void k_band_finish(int n, const int* __restrict__ fail, const int* __restrict__ ctr,
-                                     double* __restrict__ sol, DevState* st) {
-  const bool bad = *fail != 0 || ctr[3] != 0;
+static __global__ void k_band_finish(int n, const int* __restrict__ ctr, double* __restrict__ sol, DevState* st) {
+  const bool bad = ctr[BAND_FAIL] != 0 || ctr[BAND_LOST] != 0;
   const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (bad && i < n) sol[i] = 0.0;
   if (i == 0) {
@@ -500,6 +546,26 @@ static __global__ void k_band_finish(int n, const int* __restrict__ fail, const 
     st->pcg_rel = bad ? 1.0 : 0.0;
     if (bad) st->fallbacks += 1;
   }
+}
+
+// The factorisation and the solves (a cooperative launch of `blocks` blocks)
+// on zeroed flags, then k_band_finish.
+inline cudaError_t band_chol(const BandShape& sh, int n, int ntask, int ncrit, int ncta_crit, const int4* task, double* T,
+                             double* rsd, double* Ui, const double* rhs, double* y, double* sol, int* flags, int blocks,
+                             DevState* st, cudaStream_t s) {
+  const size_t ntile = (size_t)sh.nb * (sh.bwt + 1);
+  int* ctr = flags + 2 * ntile;
+  BandArgs<BandShape> a{sh, n, ntask, ncrit, ncta_crit, task, T, rsd, Ui, rhs, y, sol, flags, flags + ntile, ctr,
+                        ctr + BAND_CTRS};
+  BandArgs<BandTop> t{{sh.nb, sh.bwt, sh.top, sh.joint}, n, ntask, ncrit, ncta_crit, task, T, rsd, Ui, rhs, y, sol,
+                      flags, flags + ntile, ctr, ctr + BAND_CTRS};
+  const bool ends = sh.top < sh.nb;
+  void* args[] = {ends ? (void*)&a : (void*)&t};
+  const void* k = ends ? (const void*)k_band_chol<BandShape> : (const void*)k_band_chol<BandTop>;
+  const cudaError_t e = cudaLaunchCooperativeKernel(k, dim3(blocks), dim3(BAND_THREADS), args, 0, s);
+  if (e != cudaSuccess) return e;
+  k_band_finish<<<(n + 255) / 256, 256, 0, s>>>(n, ctr, sol, st);
+  return cudaGetLastError();
 }
 
 }  // namespace ba

@@ -173,9 +173,10 @@ struct ba_pgo {
   uint8_t* fixed = nullptr;
   // Cholesky: the band tiles of H + D (then L), 1 / L_cc, the inverses
   // L_JJ^{-T}, y / x in the padded factored order, and the flags of the
-  // factorisation's schedule (tile final and tile updates [bnb (bwt + 1)]
-  // each, counters [5], failure [1], inverse final [bnb])
-  int bnb = 0, bwt = 0, band_grid = 0, band_crit = 0, bntask = 0, bncrit = 0;
+  // factorisation's schedule (band_flags: tile final, tile updates,
+  // counters, inverse final)
+  BandShape bsh{0, 0, 0, 0};
+  int band_grid = 0, band_crit = 0, bntask = 0, bncrit = 0;
   size_t bT_bytes = 0, bflag_count = 0;
   double *bT = nullptr, *brs = nullptr, *bUi = nullptr, *dy = nullptr;
   int* bflag = nullptr;
@@ -342,10 +343,10 @@ ba_status enqueue_solve(ba_pgo* h, const double* lam_ptr, int maxiter, double to
     PCU(cudaMemsetAsync(h->bT, 0, h->bT_bytes, s));
     PCU(cudaMemsetAsync(h->bflag, 0, sizeof(int) * h->bflag_count, s));
     k_pgo_band<<<h->N, 64, 0, s>>>(h->N, h->rowptr, h->inc, h->ei, h->ej, h->B, h->Hd, h->D, h->pos, h->fixed,
-                                   h->bwt, h->bT);
+                                   h->bsh, h->bT);
     count_launch();
-    if (h->bnb * BAND_TB > n) {
-      k_band_pad<<<1, BAND_TB, 0, s>>>(n, h->bnb, h->bwt, h->bT);
+    if (h->bsh.nb * BAND_TB > n) {
+      k_band_pad<<<1, BAND_TB, 0, s>>>(n, h->bsh, h->bT);
       count_launch();
     }
     const double* rhs = h->r;
@@ -356,13 +357,8 @@ ba_status enqueue_solve(ba_pgo* h, const double* lam_ptr, int maxiter, double to
       rhs = h->rp;
       sol = h->xp;
     }
-    const size_t ntile = (size_t)h->bnb * (h->bwt + 1);
-    int* ctr = h->bflag + 2 * ntile;
-    BandArgs ba_{h->bnb, h->bwt, n, h->bntask, h->bncrit, h->band_crit, h->btask, h->bT, h->brs, h->bUi, rhs,
-                 h->dy, sol, h->bflag, h->bflag + ntile, ctr, ctr + 5, ctr + 6};
-    void* args[] = {&ba_};
-    PCU(cudaLaunchCooperativeKernel((const void*)k_band_chol, dim3(h->band_grid), dim3(BAND_THREADS), args, 0, s));
-    k_band_finish<<<nb(n, 256), 256, 0, s>>>(n, ctr + 5, ctr, sol, h->st);
+    PCU(band_chol(h->bsh, n, h->bntask, h->bncrit, h->band_crit, h->btask, h->bT, h->brs, h->bUi, rhs, h->dy, sol,
+                  h->bflag, h->band_grid, h->st, s));
     count_launch(2);
     if (h->pos) {
       k_pgo_permute<<<nb(n, 256), 256, 0, s>>>(h->N, h->pos, 1, h->xp, h->x);
@@ -548,32 +544,34 @@ ba_status ba_pgo_create(ba_pgo** out, int N, int E, const double* poses, const i
         hpos.clear();  // node order
       }
       // the band tiles and the schedule's flags
-      h->bnb = (int)((n6 + BAND_TB - 1) / BAND_TB);
-      h->bwt = std::min(h->bnb - 1, (h->band + BAND_TB - 1) / BAND_TB);
+      const int bnb = (int)((n6 + BAND_TB - 1) / BAND_TB);
+      const int bwt = std::min(bnb - 1, (h->band + BAND_TB - 1) / BAND_TB);
+      h->bsh = band_shape(bnb, bwt);
       // updates per task segment: one column, or more when the band is so
       // wide that the task list would pass 4M updates
-      const long long nupd = (long long)h->bnb * h->bwt * (h->bwt + 1) / 2;
+      const long long nupd = (long long)bnb * bwt * (bwt + 1) / 2;
       if (nupd > (1LL << 40))
         return bail(set_error(BA_ERR_INVALID_ARG, "the band of H is too wide for BA_SOLVER_CHOLESKY (%d x %d tiles)",
-                              h->bnb, h->bwt + 1));
+                              bnb, bwt + 1));
       const int s_upd = (int)std::max(1LL, (nupd + (4LL << 20) - 1) / (4LL << 20));
       // one block per SM: a task then has its SM's FP64 pipe to itself
       h->band_grid = std::max(1, nsm);
-      h->band_crit = h->band_grid >= 2 ? std::min(BAND_CRIT_BLOCKS, std::max(1, h->band_grid / 8)) : 0;
-      const std::vector<BandTask> tasks = band_tasks(h->bnb, h->bwt, s_upd, h->band_grid, h->band_crit, &h->bncrit);
+      const int crit = h->bsh.top < bnb ? 2 * BAND_CRIT_BLOCKS : BAND_CRIT_BLOCKS;  // for each chain
+      h->band_crit = h->band_grid >= 2 ? std::min(crit, std::max(1, h->band_grid / 8)) : 0;
+      const std::vector<BandTask> tasks = band_tasks(h->bsh, s_upd, h->band_grid, h->band_crit, &h->bncrit);
       static_assert(sizeof(BandTask) == sizeof(int4), "a task is read as an int4");
       if (h->bncrit == 0) h->band_crit = 0;
       h->bntask = (int)tasks.size();
-      h->bT_bytes = (size_t)h->bnb * (h->bwt + 1) * (BAND_TB * BAND_TB) * sizeof(double);
-      h->bflag_count = 2 * (size_t)h->bnb * (h->bwt + 1) + 6 + h->bnb;
+      h->bT_bytes = (size_t)bnb * (bwt + 1) * (BAND_TB * BAND_TB) * sizeof(double);
+      h->bflag_count = band_flags(h->bsh);
       int occb = 0;
-      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occb, k_band_chol, BAND_THREADS, 0)) != cudaSuccess ||
+      if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occb, k_band_chol<BandShape>, BAND_THREADS, 0)) != cudaSuccess ||
           occb < 1)
         return bail(set_error(BA_ERR_CUDA, "the Cholesky kernel cannot be resident"));
       if ((e = h->alloc(&h->bT, h->bT_bytes)) != cudaSuccess ||
-          (e = h->alloc(&h->brs, 8ull * h->bnb * BAND_TB)) != cudaSuccess ||
-          (e = h->alloc(&h->bUi, 8ull * h->bnb * BAND_TB * BAND_TB)) != cudaSuccess ||
-          (e = h->alloc(&h->dy, 8ull * h->bnb * BAND_TB)) != cudaSuccess ||
+          (e = h->alloc(&h->brs, 8ull * bnb * BAND_TB)) != cudaSuccess ||
+          (e = h->alloc(&h->bUi, 8ull * bnb * BAND_TB * BAND_TB)) != cudaSuccess ||
+          (e = h->alloc(&h->dy, 8ull * bnb * BAND_TB)) != cudaSuccess ||
           (e = h->alloc(&h->bflag, sizeof(int) * h->bflag_count)) != cudaSuccess ||
           (e = h->alloc(&h->btask, sizeof(int4) * tasks.size())) != cudaSuccess ||
           (e = cudaMemcpy(h->btask, tasks.data(), sizeof(int4) * tasks.size(), cudaMemcpyHostToDevice)) !=

@@ -1060,7 +1060,7 @@ static __global__ void __launch_bounds__(64)
 k_pgo_band(int N, const int32_t* __restrict__ rowptr, const int32_t* __restrict__ inc,
            const int32_t* __restrict__ ei, const int32_t* __restrict__ ej, const double* __restrict__ B,
            const double* __restrict__ Hd, const double* __restrict__ D, const int32_t* __restrict__ pos,
-           const uint8_t* __restrict__ fixed, int bwt, double* __restrict__ T) {
+           const uint8_t* __restrict__ fixed, BandShape sh, double* __restrict__ T) {
   const int i = blockIdx.x, t = threadIdx.x;
   if (t >= 36) return;
   const int a = t / 6, b = t % 6;
@@ -1068,8 +1068,11 @@ k_pgo_band(int N, const int32_t* __restrict__ rowptr, const int32_t* __restrict_
   const int R = 6 * pi + a;
   const bool fi = fixed && fixed[i];
   auto at = [&](int C) -> double& {
-    const int I = R / BAND_TB, J = C / BAND_TB;
-    return T[((long long)J * (bwt + 1) + (I - J)) * (BAND_TB * BAND_TB) + (R % BAND_TB) * BAND_TB + C % BAND_TB];
+    // block rows eliminated from the end come in reverse: their tiles transposed
+    const int I = sh.place_of(R / BAND_TB), J = sh.place_of(C / BAND_TB);
+    const int r = R % BAND_TB, c = C % BAND_TB;
+    return I >= J ? T[sh.index(I, J) * (BAND_TB * BAND_TB) + r * BAND_TB + c]
+                  : T[sh.index(J, I) * (BAND_TB * BAND_TB) + c * BAND_TB + r];
   };
   if (b <= a) at(6 * pi + b) = fi ? (a == b ? 1.0 : 0.0)
                                    : Hd[21LL * i + sym6(b, a)] + (a == b ? D[6LL * i + a] : 0.0);
