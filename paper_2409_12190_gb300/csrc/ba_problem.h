@@ -140,6 +140,9 @@ struct ba_problem {
     int4* parts = nullptr;
     unsigned long long* gx = nullptr;
   } sx;
+  // the PCG's vector work in one launch (ba_vec.cuh) where its blocks fit the GPU
+  unsigned long long* vec_gx = nullptr;  // exchange slots, then the error flag
+  double* vec_scal = nullptr;            // [4]
   bool batched = false;  // the concatenated problems of a batch: never solved as one
   ba::DevState* st = nullptr;
   ba_iter_stats* stats = nullptr;
