@@ -889,9 +889,8 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
     }
     h->bnb = (int)((n + BAND_TB - 1) / BAND_TB);
     h->bwt = h->bnb - 1;
-    const long long nupd = (long long)h->bnb * h->bwt * (h->bwt + 1) / 2;
-    const int s_upd = (int)std::max(1LL, (nupd + (4LL << 20) - 1) / (4LL << 20));
     h->band_grid = std::max(1, nsm);
+    const int s_upd = band_segment(BandShape{h->bnb, h->bwt, h->bnb, h->bnb}, h->band_grid);
     h->band_crit = h->band_grid >= 2 ? std::min(BAND_CRIT_BLOCKS, std::max(1, h->band_grid / 8)) : 0;
     const std::vector<BandTask> tasks = band_tasks(h->bnb, h->bwt, s_upd, h->band_grid, h->band_crit, &h->bncrit);
     static_assert(sizeof(BandTask) == sizeof(int4), "a task is read as an int4");

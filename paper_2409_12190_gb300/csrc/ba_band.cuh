@@ -120,6 +120,11 @@ static __device__ __noinline__ bool band_wait(int* flag, int v, int* err) {
   return true;
 }
 
+__device__ __forceinline__ int band_load(int* p) {
+  cuda::atomic_ref<int, cuda::thread_scope_device> f(*p);
+  return f.load(cuda::memory_order_acquire);
+}
+
 // Publish v after the block's writes (called by every thread).
 __device__ __forceinline__ void band_publish(int* flag, int v) {
   __syncthreads();
@@ -149,6 +154,7 @@ struct BandSmem {
   uint16_t tri[BAND_TRI];  // (r << 8) | c of the row-major lower triangle
   int task;
   int bad;
+  int ready;
 };
 
 // X L^T = A in place (s.A = A on entry, X on return), L = the staged tile
@@ -268,32 +274,64 @@ static __device__ bool band_task_D(const BandArgs<S>& a, BandSmem& s, int J) {
 }
 
 // U: A_IJ -= L_IK L_JK^T for K = Ka .. Ka + cnt - 1, after the tile's
-// earlier updates.
+// earlier updates.  A lane each looks at the flags of the first columns: those
+// that are final already (most, in the bulk) are not waited for, and their
+// tiles are fetched while the column before is multiplied (250 cameras, with
+// segments of four columns: 8.31 -> 6.95 ms, 7.63 without the fetching ahead;
+// the multiply-adds alone take 8.5 us a tile at the SM's FP64 rate, 3.6 ms).
 template <typename S>
 static __device__ bool band_task_U(const BandArgs<S>& a, BandSmem& s, int I, int J, int Ka, int cnt) {
   constexpr int TB = BAND_TB, E = TB * TB / BAND_THREADS, RS = BAND_THREADS / TB;
   const int tid = threadIdx.x, col = tid % TB, row0 = tid / TB;
   const int before = a.sh.updates(I, J, Ka);
   int w = 1;
-  if (tid == 0) w = band_wait(band_prog(a, I, J), before, a.ctr + BAND_LOST);
+  if (tid < 32) {
+    const int j = tid >> 1;
+    const bool there = j < cnt && band_load(band_flag(a, tid & 1 ? J : I, Ka + j)) != 0;
+    const unsigned int got = __ballot_sync(0xffffffffu, there);
+    if (tid == 0) {
+      s.ready = got == 0xffffffffu ? 16 : (__ffs(~got) - 1) >> 1;  // leading columns with both tiles final
+      w = band_wait(band_prog(a, I, J), before, a.ctr + BAND_LOST);
+    }
+  }
   if (!__syncthreads_and(w)) return false;
+  const int ready = s.ready;
   double* Tij = band_tile(a, I, J);
-  double acc[E];
+  double acc[E], fa[E], fb[E];
 #pragma unroll
   for (int m = 0; m < E; ++m) acc[m] = __ldcg(Tij + (row0 + m * RS) * TB + col);
-  for (int K = Ka; K < Ka + cnt; ++K) {
-    w = 1;
-    if (tid == 0) w = band_wait(band_flag(a, I, K), 1, a.ctr + BAND_LOST) && band_wait(band_flag(a, J, K), 1, a.ctr + BAND_LOST);
-    if (!__syncthreads_and(w)) return false;
-    band_stage(s.A, band_tile(a, I, K));
-    if (I != J) band_stage(s.B, band_tile(a, J, K));
+  auto fetch = [&](int K) {
+    const double *A = band_tile(a, I, K), *B = band_tile(a, J, K);
+#pragma unroll
+    for (int m = 0; m < E; ++m) fa[m] = __ldcg(A + tid + m * BAND_THREADS);
+    if (I != J) {
+#pragma unroll
+      for (int m = 0; m < E; ++m) fb[m] = __ldcg(B + tid + m * BAND_THREADS);
+    }
+  };
+  for (int k = 0; k < cnt; ++k) {
+    if (k >= ready) {
+      w = 1;
+      if (tid == 0)
+        w = band_wait(band_flag(a, I, Ka + k), 1, a.ctr + BAND_LOST) &&
+            band_wait(band_flag(a, J, Ka + k), 1, a.ctr + BAND_LOST);
+      if (!__syncthreads_and(w)) return false;
+    }
+    if (k == 0 || k >= ready) fetch(Ka + k);
+#pragma unroll
+    for (int m = 0; m < E; ++m) s.A[row0 + m * RS][col] = fa[m];
+    if (I != J) {
+#pragma unroll
+      for (int m = 0; m < E; ++m) s.B[row0 + m * RS][col] = fb[m];
+    }
     __syncthreads();
+    if (k + 1 < min(cnt, ready)) fetch(Ka + k + 1);
     const BandTile& LJ = (I != J) ? s.B : s.A;
 #pragma unroll 8
-    for (int k = 0; k < TB; ++k) {
-      const double b = LJ[col][k];
+    for (int kk = 0; kk < TB; ++kk) {
+      const double b = LJ[col][kk];
 #pragma unroll
-      for (int m = 0; m < E; ++m) acc[m] = fma(-s.A[row0 + m * RS][k], b, acc[m]);
+      for (int m = 0; m < E; ++m) acc[m] = fma(-s.A[row0 + m * RS][kk], b, acc[m]);
     }
     __syncthreads();
   }
@@ -338,11 +376,6 @@ static __device__ bool band_task_I(const BandArgs<S>& a, BandSmem& s, int J) {
   band_store(a.Ui + (long long)J * TB * TB, s.A);
   band_publish(a.iflag + J, 1);
   return true;
-}
-
-__device__ __forceinline__ int band_load(int* p) {
-  cuda::atomic_ref<int, cuda::thread_scope_device> f(*p);
-  return f.load(cuda::memory_order_acquire);
 }
 
 // Thread 0: wait until the counter *p reaches v; *known caches the last value

@@ -108,6 +108,22 @@ inline BandShape band_shape(int nb, int bwt) {
   return BandShape{nb, bwt, (nb - bwt + 1) / 2, nb - bwt};
 }
 
+// Columns per update segment: one where the chain of D tasks bounds (33 us a
+// step), four where the bulk updates do (12 us a column over `workers`
+// blocks): a segment reads and writes its tile and waits for its turn once.
+// One trial with S formed, one GB300, segments of 1 / 2 / 4 / 8 columns: 100
+// cameras (29 block rows) 2.22 / 2.23 / 2.29 / 2.52 ms, 160 (45 rows) 3.54 /
+// 3.39 / 3.52 / 3.99, 250 (71 rows) 7.79 / 7.22 / 6.95 / 6.98, 400 (113 rows)
+// 22.7 / 20.4 / 19.3 / 18.9; the line lies at 50 rows of a full triangle.  More
+// where the list would pass 4M updates.
+inline int band_segment(const BandShape& sh, int workers) {
+  const long long updates = (long long)sh.nb * sh.bwt * (sh.bwt + 1) / 2;
+  const long long chain = sh.top < sh.nb ? (sh.nb + sh.bwt) / 2 : sh.nb;
+  const double tiles = sh.bwt + 1 < sh.nb ? (double)updates : updates / 3.0;  // a triangle's columns get shorter
+  const int seg = 12.0 * tiles > 33.0 * (double)chain * workers ? 4 : 1;
+  return (int)std::max<long long>(seg, (updates + (4LL << 20) - 1) / (4LL << 20));
+}
+
 // One task, as the device reads it (an int4): x = type + 8 count (count:
 // U's columns), y = I, z = J, w = Ka (U's first column); for D, I, F:
 // y = z = J; for B: y = z = I.

@@ -547,15 +547,13 @@ ba_status ba_pgo_create(ba_pgo** out, int N, int E, const double* poses, const i
       const int bnb = (int)((n6 + BAND_TB - 1) / BAND_TB);
       const int bwt = std::min(bnb - 1, (h->band + BAND_TB - 1) / BAND_TB);
       h->bsh = band_shape(bnb, bwt);
-      // updates per task segment: one column, or more when the band is so
-      // wide that the task list would pass 4M updates
       const long long nupd = (long long)bnb * bwt * (bwt + 1) / 2;
       if (nupd > (1LL << 40))
         return bail(set_error(BA_ERR_INVALID_ARG, "the band of H is too wide for BA_SOLVER_CHOLESKY (%d x %d tiles)",
                               bnb, bwt + 1));
-      const int s_upd = (int)std::max(1LL, (nupd + (4LL << 20) - 1) / (4LL << 20));
       // one block per SM: a task then has its SM's FP64 pipe to itself
       h->band_grid = std::max(1, nsm);
+      const int s_upd = band_segment(h->bsh, h->band_grid);
       const int crit = h->bsh.top < bnb ? 2 * BAND_CRIT_BLOCKS : BAND_CRIT_BLOCKS;  // for each chain
       h->band_crit = h->band_grid >= 2 ? std::min(crit, std::max(1, h->band_grid / 8)) : 0;
       const std::vector<BandTask> tasks = band_tasks(h->bsh, s_upd, h->band_grid, h->band_crit, &h->bncrit);
