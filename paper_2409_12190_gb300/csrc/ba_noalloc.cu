@@ -35,11 +35,8 @@
 namespace {
 
 constexpr long long kMaxKeys = BA_NOALLOC_MAX_KEYS;
-constexpr long long kTile = 4096;  // keys per radix tile (the sort's tile size)
-constexpr long long kMaxTiles = (kMaxKeys + kTile - 1) / kTile;
-// temporary keys A/B and values A/B, then the [256][tiles] histogram, then the
-// error flag (own 256-byte line)
-constexpr long long kErrOffsetInts = 4 * kMaxKeys + 256 * kMaxTiles;
+// what the sort uses, then the error flag (own 256-byte line)
+constexpr long long kErrOffsetInts = ba::csr_scratch_ints(kMaxKeys);
 constexpr long long kScratchInts = kErrOffsetInts + 64;
 
 __device__ __align__(256) int32_t g_noalloc_scratch[kScratchInts];

@@ -25,6 +25,7 @@ constexpr int RS_WARPS = RS_THREADS / 32;
 constexpr int RS_ITEMS = 16;                       // keys per lane per tile
 constexpr int RS_PER_WARP = 32 * RS_ITEMS;         // 512
 constexpr int RS_TILE = RS_WARPS * RS_PER_WARP;    // 4096
+static_assert(RS_TILE == CSR_TILE, "the scratch is sized by it");
 
 __global__ void k_rs_check(const int32_t* __restrict__ keys, int n, int n_keys,
                            int* __restrict__ err) {
@@ -183,9 +184,7 @@ int bits_for(int n_keys) {
 }  // namespace
 
 size_t csr_scratch_bytes(int n) {
-  const long long ntiles = (n + RS_TILE - 1) / RS_TILE;
-  size_t b = 4 * (size_t)n * sizeof(int32_t) + 256 * (size_t)(ntiles + 1) * sizeof(int32_t);
-  return b + 256;
+  return (size_t)csr_scratch_ints(n) * sizeof(int32_t) + 256;
 }
 
 cudaError_t csr_build_async(const int32_t* keys, int n, int n_keys, int32_t* perm_out,
