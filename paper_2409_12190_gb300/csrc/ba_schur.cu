@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstring>
 #include <type_traits>
 #include <vector>
 
@@ -265,10 +266,37 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   btask.push_back((int)task.size());
   const int nblk = x.nblk = (int)bcam.size();
   x.ntask = (int)task.size();
-  auto up = [&](auto** p, const auto& v) {
-    cudaError_t r = h->alloc(p, v.size() * sizeof(v[0]));
-    if (r == cudaSuccess) r = cudaMemcpy(*p, v.data(), v.size() * sizeof(v[0]), cudaMemcpyHostToDevice);
-    return r;
+  // the lists and buffers of the formed system: one allocation, one copy (a
+  // call each was some 0.2 ms of a small problem's set-up of 4-8 ms)
+  struct Item {
+    void* p;  // the pointer's place
+    const void* src;
+    size_t bytes;
+  };
+  std::vector<Item> items;
+  auto up = [&](auto** p, const auto& v) { items.push_back({p, v.data(), v.size() * sizeof(v[0])}); };
+  auto room = [&](auto** p, size_t bytes) { items.push_back({p, nullptr, bytes}); };
+  auto place = [&] {
+    if (e != cudaSuccess) return;
+    auto al = [](size_t n) { return (n + 255) / 256 * 256; };
+    size_t copied = 0, all = 0;
+    for (const Item& i : items) {
+      copied += i.src ? al(i.bytes) : 0;
+      all += al(i.bytes);
+    }
+    char* base = nullptr;
+    e = h->alloc(&base, all);
+    if (e != cudaSuccess) return;
+    std::vector<char> host(copied);
+    size_t at = 0, free_at = copied;  // the copied ones first
+    for (const Item& i : items) {
+      size_t& o = i.src ? at : free_at;
+      const char* v = base + o;
+      std::memcpy(i.p, &v, sizeof v);
+      if (i.src) std::copy((const char*)i.src, (const char*)i.src + i.bytes, host.begin() + o);
+      o += al(i.bytes);
+    }
+    e = cudaMemcpy(base, host.data(), copied, cudaMemcpyHostToDevice);
   };
   auto keep = [&] {
     x.pk = pr.pk;
@@ -283,16 +311,20 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   const bool lean = !f32 && !h->mf;
   if (lean) {
     kernel_attr((const void*)k_schur_form_marked, sf_smem<double>());
-    if (e == cudaSuccess) e = h->alloc(&x.lean_w, 8ull * NLEAN * O);
-    if (e == cudaSuccess) e = h->alloc(&x.lean_t, 8ull * 6 * O);
-    if (e == cudaSuccess) e = h->alloc(&x.lean_marked, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemsetAsync(x.lean_marked, 0, sizeof(int), s);
+    room(&x.lean_w, 8ull * NLEAN * O);
+    room(&x.lean_t, 8ull * 6 * O);
+    room(&x.lean_marked, sizeof(int));
   }
-  if (e == cudaSuccess) e = up(&x.task, task);
-  if (e == cudaSuccess) e = up(&x.blk_cam, bcam);
-  if (e == cudaSuccess) e = up(&x.blk_task, btask);
-  if (e == cudaSuccess) e = h->alloc(&x.part, (size_t)x.ntask * SX_PART * vs);
+  up(&x.task, task);
+  up(&x.blk_cam, bcam);
+  up(&x.blk_task, btask);
+  room(&x.part, (size_t)x.ntask * SX_PART * vs);
+  auto unmark = [&] {
+    if (e == cudaSuccess && lean) e = cudaMemsetAsync(x.lean_marked, 0, sizeof(int), s);
+  };
   if (direct) {
+    place();
+    unmark();
     if (e != cudaSuccess) {
       cudaGetLastError();
       return BA_OK;
@@ -372,17 +404,19 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   SCU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, SX_THREADS, smem));
   if ((long long)occ * nsm < groups) return BA_OK;
   x.words = sx_words(groups, C) + 1;  // and the error flag
-  if (e == cudaSuccess) e = up(&x.blk_pos, pos);
-  if (e == cudaSuccess) e = up(&x.rowblk, rowblk);
-  if (e == cudaSuccess) e = up(&x.cams, list);
-  if (e == cudaSuccess) e = up(&x.cam_ptr, lptr);
-  if (e == cudaSuccess) e = up(&x.part_ptr, pptr);
-  if (e == cudaSuccess) e = up(&x.row_part, rpart);
-  if (e == cudaSuccess) e = up(&x.colloc, colloc);
-  if (e == cudaSuccess) e = up(&x.ownloc, ownloc);
-  if (e == cudaSuccess) e = up(&x.parts, parts);
-  if (e == cudaSuccess) e = h->alloc(&x.val, (size_t)rowblk[C] * SX_PART * vs);
-  if (e == cudaSuccess) e = h->alloc(&x.gx, 8 * x.words);
+  up(&x.blk_pos, pos);
+  up(&x.rowblk, rowblk);
+  up(&x.cams, list);
+  up(&x.cam_ptr, lptr);
+  up(&x.part_ptr, pptr);
+  up(&x.row_part, rpart);
+  up(&x.colloc, colloc);
+  up(&x.ownloc, ownloc);
+  up(&x.parts, parts);
+  room(&x.val, (size_t)rowblk[C] * SX_PART * vs);
+  room(&x.gx, 8 * x.words);
+  place();
+  unmark();
   if (e == cudaSuccess && !h->Sii) e = h->alloc(&h->Sii, 45ull * C * 8);
   if (e != cudaSuccess) {
     cudaGetLastError();
