@@ -425,9 +425,22 @@ def time_to_f_ref(prob, state0, f_ref, max_trials, stream):
             "final_cost": costs[-1], "rel_gap_at_end": costs[-1] / f_ref - 1.0}
 
 
-def kernel_table(per, C, P, O, lay, tsize, mf, huber, alu_peak):
+# operations per pair of observations of one point, where the reduced system
+# is formed: 157 FP64 multiply-adds from the lean form; FP32 the 9 x 3 by 3 x 9
+# product of the two couplings
+FORM_FLOPS_PER_PAIR = {"f64": 314, "f32": 486}
+
+
+def observation_pairs(pt_idx):
+    n = np.bincount(pt_idx).astype(np.int64)
+    return int((n * (n - 1) // 2).sum())
+
+
+def kernel_table(per, C, P, O, lay, tsize, mf, huber, alu_peak, form_flops=0):
     """Per kernel class: launches, mean CUDA-event time, share, algorithmic
-    GB/s and (PCG passes) TFLOP/s with their fractions."""
+    GB/s and (PCG passes) TFLOP/s with their fractions.  form_flops: the
+    arithmetic of forming S once, when it is formed: its launch is timed with
+    the Schur blocks' (two launches a trial in schur_cam)."""
     total = sum(v[0] for v in per.values())
     out = {}
     for name, (kms, n) in per.items():
@@ -437,7 +450,7 @@ def kernel_table(per, C, P, O, lay, tsize, mf, huber, alu_peak):
         avg = kms / n
         row = {"launches": n, "avg_us": 1000.0 * avg, "share": kms / total,
                "gbs": (b / (avg / 1000.0) / 1e9) if b else None, "bytes_per_launch": b or None}
-        fl = pass_flops(name, O, P, mf)
+        fl = form_flops / 2 if form_flops and name == "schur_cam" else pass_flops(name, O, P, mf)
         if fl:
             row["tflops"] = fl / (avg / 1000.0) / 1e12
             row["flops_per_launch"] = fl
@@ -515,7 +528,9 @@ def run_precision(args, prec, scene, ci, pi, pix, dev, world, f_ref, peaks_d, ba
         alu_peak = peaks_d["fp64_fma_tflops"]
         alu_source = "measured (ba_measure_fma_peak: FP64 FMA chains on every SM, best of 3)"
     huber = scene.huber_delta > 0
-    kernels = kernel_table(per, C, P, O, lay, tsize, mf, huber, alu_peak)
+    formed = per.get("pass_b", (0.0, 0))[1] == 0  # PCG ran without passes over the observations
+    kernels = kernel_table(per, C, P, O, lay, tsize, mf, huber, alu_peak,
+                           FORM_FLOPS_PER_PAIR[prec] * observation_pairs(scene.pt_idx) if formed else 0)
     it_bytes = sum(algorithmic_bytes(k, C, P, O, lay["pieces"], tsize, mf, huber) * per[k][1] for k in per)
     roof = roofline_of(kernels, per, peaks_d["hbm_gbs"], peaks_d["hbm_kind"], alu_peak, alu_source,
                        kernel_source_hash(), prof_ms, it_bytes, prec)
@@ -558,13 +573,14 @@ def run_precision(args, prec, scene, ci, pi, pix, dev, world, f_ref, peaks_d, ba
            "loss": "squared", "pcg": f"block-Jacobi, maxiter {PCG_MAXITER}, tol {PCG_TOL}",
            "pcg_iters_mean": statistics.mean(pcg) if pcg else None, "pcg_iters_total": sum(pcg),
            "accepted": sum(t["accepted"] for t in trials),
-           "l2": "inputs larger than L2 (each PCG pass streams >0.1 GB of per-observation data; L2 129 MB)",
+           "l2": "inputs larger than L2 (each pass streams >0.1 GB of per-observation data; L2 129 MB)",
            "parallelism": (f"points partitioned over {world} GPUs (cameras replicated, NCCL all-reduce at the "
                            f"six exchanges of a trial)" if part is not None else
                            ("replicas" if world > 1 else "single GPU")),
            "graph": "direct launches (exchanges)" if part is not None else "one CUDA graph per LM trial",
            "jacobian": "recomputed in every pass" if mf else "stored planes",
-           "schur_product": "fused point-major pass A + pass B" if lay["fused_a"] else "passes A1, A2, B"}
+           "schur_product": ("formed S, its PCG in one launch" if formed else
+                             "fused point-major pass A + pass B" if lay["fused_a"] else "passes A1, A2, B")}
     return {"value": value, "ms_per_step": ms / args.steps, "dtype": prec, "config": cfg, "gpu_launches": launches,
             "clocks": clk, "roofline": roof, "kernels": kernels, "e2e": e2e, "time_to_cost": ttc}
 
@@ -689,9 +705,8 @@ def run_ours(args):
 
 BATCH_N = 512
 BATCH_ITERS = 10
-# FP32 operations per observation and PCG iteration of the batched kernel's
-# passes A1 and B (recompute mode, as for the single-problem kernels)
-BATCH_FLOPS_PER_OBS_PCG = FLOPS_PER_OBS["pass_a1"] + FLOPS_PER_OBS["pass_b"]
+# operations of a 9 x 9 block of the formed system in a product
+BATCH_FLOPS_PER_BLOCK = 162
 
 
 def run_batch(args):
@@ -766,16 +781,17 @@ def run_batch(args):
     torch.cuda.synchronize()
     solve_ms = e0.elapsed_time(e1)
     st2 = bt.stats()
-    pcg_obs = sum(t["pcg_iters"] * s.O for st, s in zip(st2, scenes) for t in st)
-    flops = BATCH_FLOPS_PER_OBS_PCG * pcg_obs
+    # the windows' systems are formed once a trial (FP32, recomputed Jacobians)
+    flops = sum(len(st) * FORM_FLOPS_PER_PAIR["f32"] * observation_pairs(s.pt_idx)
+                + BATCH_FLOPS_PER_BLOCK * s.C * s.C * sum(t["pcg_iters"] for t in st) for st, s in zip(st2, scenes))
     sm_mhz = (clk or {}).get("sm_max_mhz") or 2070.0
     alu_peak = fp32_peak_tflops(sm_mhz)
     ach = flops / (solve_ms / 1000.0) / 1e12
     roofline = {"bound": "alu", "kernel": "k_batch_lm", "achieved": ach, "peak": alu_peak, "unit": "TFLOP/s",
                 "frac": ach / alu_peak, "flops_per_launch": flops,
                 "peak_source": f"152 SMs x 128 FP32 lanes x 2 x {sm_mhz:.0f} MHz",
-                "note": "PCG passes A1+B only (113+119 FP32 flops per observation and PCG iteration); "
-                        "each problem's arrays stay in L2 across its trials", "traffic": None}
+                "note": "forming (486 FP32 flops per pair of observations of a point) and the formed products "
+                        "(162 per camera pair and PCG iteration); each problem's arrays stay in L2", "traffic": None}
 
     # end to end: pinned host parameters in, solve, parameters out
     C, P = bt.C, bt.P
@@ -1310,7 +1326,7 @@ def run_pgo(args):
             "peak": peaks_d, "unit": "TFLOP/s", "frac": head["pcg"]["pcg_iteration_tflops"] / peaks_d,
             "flops_per_iteration": fl, "peak_source": "measured (ba_measure_fma_peak, FP64)", "traffic": None,
             "note": "the graph's arrays (B: 288 B per edge) stay in L2; the iteration is bound by FP64 issue and "
-                    "its two grid barriers"}
+                    "its two grid exchanges"}
     cpu = None
     if not args.no_cpu_baseline:
         import multiprocessing as mp
