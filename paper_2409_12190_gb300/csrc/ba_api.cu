@@ -320,15 +320,15 @@ void enqueue_dense_solve(ba_problem* h, const double* lam_ptr) {
     cudaMemsetAsync(h->bT, 0, h->bT_bytes, s);
     schur_to_band(h, lam_ptr);
   } else {
-  k_dense_w<T, MF><<<nblk(h->P, DENSE_THREADS), DENSE_THREADS, 0, s>>>(
-      h->P, h->rowptr_pt, h->pm_cam, h->pm2cm, (const T*)h->Jcm, (const T*)h->cm_sw, (const T*)h->camtab,
-      (const T*)h->pts, h->st, h->O, h->Wd);
-  k_schur_dense<T><<<h->C * h->nseg, DENSE_THREADS, 0, s>>>(
-      h->C, h->nseg, h->rowptr_cam, h->cm_pt, h->rowptr_pt, h->pm_cam, h->pm2cm, h->Wd, (const T*)h->Vinv, h->Spart);
-  cudaMemsetAsync(h->bT, 0, h->bT_bytes, s);
-  k_schur_to_band<<<n, 256, 0, s>>>(h->C, h->nseg, h->Spart, h->U, lam_ptr, h->opt.diag_min, h->opt.diag_max,
-                                    h->fixed, h->bwt, h->bT);
-  count_launch(3);
+    k_dense_w<T, MF><<<nblk(h->P, DENSE_THREADS), DENSE_THREADS, 0, s>>>(
+        h->P, h->rowptr_pt, h->pm_cam, h->pm2cm, (const T*)h->Jcm, (const T*)h->cm_sw, (const T*)h->camtab,
+        (const T*)h->pts, h->st, h->O, h->Wd);
+    k_schur_dense<T><<<h->C * h->nseg, DENSE_THREADS, 0, s>>>(
+        h->C, h->nseg, h->rowptr_cam, h->cm_pt, h->rowptr_pt, h->pm_cam, h->pm2cm, h->Wd, (const T*)h->Vinv, h->Spart);
+    cudaMemsetAsync(h->bT, 0, h->bT_bytes, s);
+    k_schur_to_band<<<n, 256, 0, s>>>(h->C, h->nseg, h->Spart, h->U, lam_ptr, h->opt.diag_min, h->opt.diag_max,
+                                      h->fixed, h->bwt, h->bT);
+    count_launch(3);
   }
   cudaMemsetAsync(h->bflag, 0, sizeof(int) * h->bflag_count, s);
   const BandShape sh{h->bnb, h->bwt, h->bnb, h->bnb};  // the whole triangle: from the top
