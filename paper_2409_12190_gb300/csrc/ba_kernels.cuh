@@ -899,8 +899,9 @@ static __global__ void k_compose_perm(int O, const int32_t* __restrict__ perm_a,
 //   W  = Jc'^T (M^T Jp),
 // Jc' without M: eight numbers (RX, p, q') and the six of M^T Jp.  It needs mu
 // away from 0 (where the distortion folds the image plane; the tangential
-// eigenvalue is A_0 + A_4 - mu): below an eighth of the other the observation
-// is marked, q'_0 = NaN, and takes the planes instead.
+// eigenvalue is A_0 + A_4 - mu): at 0 (a focal length of 0 makes all of M 0) or
+// below an eighth of the other the observation is marked, q'_0 = NaN, and takes
+// the planes instead.
 // Planes in pairs: (RX0, RX1) (RX2, p0) (p1, q'0) (q'1, q'2), then M^T Jp (3).
 constexpr int NLEAN = 14;
 template <typename T>
@@ -909,7 +910,7 @@ __device__ __forceinline__ bool lean_obs(const Fac<T>& o, const T (&pl)[NPLANE],
   const T m = o.A[2] * o.px + o.A[5] * o.py;  // mu r2
   const T im = r2 > T(0) ? r2 / m : T(0);     // 1 / mu (p = 0: p q' = 0 whatever q')
   const T mu = r2 > T(0) ? m / r2 : o.A[0];
-  const bool ok = fabs(mu) >= T(0.125) * fabs(o.A[0] + o.A[4] - mu);
+  const bool ok = mu != T(0) && fabs(mu) >= T(0.125) * fabs(o.A[0] + o.A[4] - mu);
   v[0] = o.RX0;
   v[1] = o.RX1;
   v[2] = o.RX2;

@@ -161,3 +161,24 @@ def test_observations_near_the_fold_of_the_distortion(solver, k1):
     with problem(sc, pix, "f64", solver=solver) as prob:
         dc, dp, _, _ = prob.damped_solve(1e-1, its, 0.0)
     assert rel_err(np64(dc), dc_ref) < 1e-9 and rel_err(np64(dp), dp_ref) < 1e-9
+
+
+@pytest.mark.parametrize("solver", ["pcg", "cholesky"])
+def test_camera_of_focal_length_zero(solver):
+    """Its projection's derivative by the point is 0 and so is the lean form's
+    factor: those observations take their planes (Jc keeps p q^T, Jp is 0)."""
+    sc = _ragged(8, 400, seed=11, lo=3, hi=6)
+    cams = sc.cams_init.copy()
+    cams[[2, 5], 6] = 0.0
+    pix = orc.pixels_from_scene(sc)
+    sc = scenegen.Scene(sc.cams_gt, sc.points_gt, sc.cam_idx, sc.pt_idx, sc.noise, cams, sc.points_init)
+    blk = orc.assemble(sc.cams_init, sc.points_init, sc.cam_idx, sc.pt_idx, pix)
+    its = 8
+    dc_ref, dp_ref, n_ref, _ = orc.solve_damped(blk, sc.cam_idx, sc.pt_idx, 1e-1,
+                                                orc.LMOptions(solver=solver, pcg_maxiter=its, pcg_tol=0.0))
+    assert np.all(np.isfinite(dc_ref)) and np.abs(dc_ref).max() > 0
+    with problem(sc, pix, "f64", solver=solver) as prob:
+        dc, dp, n, _ = prob.damped_solve(1e-1, its, 0.0)
+    if solver == "pcg":
+        assert n == n_ref
+    assert rel_err(np64(dc), dc_ref) < 1e-9 and rel_err(np64(dp), dp_ref) < 1e-9
