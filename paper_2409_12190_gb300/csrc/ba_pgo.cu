@@ -598,8 +598,15 @@ ba_status ba_pgo_create(ba_pgo** out, int N, int E, const double* poses, const i
     const size_t smem = pgo_res_smem(max_slots);
     int occ_res = 0;
     const int res_threads = std::max(64, gen_threads);  // (192 throughout: 2.65 ms against 2.54 ms a pass)
-    if (smem <= 220u * 1024u &&
-        cudaFuncSetAttribute(k_pgo_pcg_res, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+    // the kernel's limit of dynamic shared memory belongs to the process: always
+    // all that a block may have, so that no graph lowers it under another's
+    int block_max = 0;
+    cudaFuncAttributes fa{};
+    if (cudaDeviceGetAttribute(&block_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
+        cudaFuncGetAttributes(&fa, k_pgo_pcg_res) == cudaSuccess &&
+        smem + fa.sharedSizeBytes <= (size_t)block_max &&
+        cudaFuncSetAttribute(k_pgo_pcg_res, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             block_max - (int)fa.sharedSizeBytes) == cudaSuccess &&
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_res, k_pgo_pcg_res, res_threads, smem) == cudaSuccess &&
         groups <= (long long)occ_res * nsm) {
       h->pcg_res_smem = std::max<size_t>(smem, 16);

@@ -8,7 +8,7 @@ import paper_2409_12190_gb300 as ba
 import scenegen
 from oracle import LMOptions
 from oracle import pgo
-from paper_2409_12190_gb300.pgo import PoseGraph
+from paper_2409_12190_gb300.pgo import PoseGraph, synthesize
 
 pytestmark = pytest.mark.gpu
 
@@ -40,3 +40,23 @@ def test_iterates_over_the_block_layouts(N):
     assert gits == its == k
     assert np.max(np.abs(got - want)) < 1e-9 * np.max(np.abs(want))
     assert np.array_equal(got, again.cpu().numpy())  # fixed order: the same bits
+
+
+def _graph(g):
+    meas, poses0 = synthesize(g.poses_gt, g.ei, g.ej, g.noise, g.drift)
+    return PoseGraph(poses0, g.ei, g.ej, meas, g.info, fixed=(0,), options=ba.Options())
+
+
+def test_a_smaller_graph_leaves_a_larger_one_solvable():
+    """The larger graph's blocks hold more shared memory than the smaller one's:
+    creating and solving the smaller one in between changes nothing for it."""
+    large, small = scenegen.sphere_graph(20, 25, seed=1), scenegen.sphere_graph(2, 3, seed=2)
+    with _graph(large) as a:
+        want = a.damped_solve(1e-2, 12, 0.0)[0].cpu()
+        with _graph(small) as b:
+            b.damped_solve(1e-2, 12, 0.0)
+            got = a.damped_solve(1e-2, 12, 0.0)[0].cpu()
+            b.solve(2)
+        a.solve(2)
+        assert np.all(np.isfinite(a.poses().cpu().numpy()))
+    assert np.array_equal(got.numpy(), want.numpy())
