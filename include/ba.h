@@ -67,16 +67,16 @@ enum { BA_JAC_AUTO = 0, BA_JAC_RECOMPUTE = 1, BA_JAC_STORE = 2 };
  * factorisation).  BA_SOLVER_PCG: block-Jacobi PCG (pcg_maxiter,
  * pcg_tol) with the implicit S x product or, where the observation structure
  * makes that faster, on S formed once per trial (only the blocks of camera
- * pairs with common points; chosen at create, the same for every trial; a
- * bounded wait of its one launch that runs out, about a second, leaves dc = 0
- * for the trial).  BA_SOLVER_CHOLESKY: S formed explicitly
- * as a dense 9C x 9C FP64 matrix and factored by a tiled Cholesky on the
- * GPU (the factorisation and both triangular solves in one cooperative
- * launch), for problems with 9C <= BA_DENSE_MAX_DIM (the matrix and its
- * tiles take 81 C^2 x 8 bytes each, plus up to 8 partial copies of S while
- * it is built for small C); a trial whose S is not positive definite in
- * FP64 takes a zero step (rejected, counted in
- * ba_iter_stats.precond_fallbacks). */
+ * pairs with common points; chosen at create, the same for every trial).  A
+ * grid-wide wait of the PCG that runs out, about a second (ba_set_wait_limit),
+ * leaves dc = 0 for the trial, counted in ba_iter_stats.precond_fallbacks.
+ * BA_SOLVER_CHOLESKY: S formed explicitly as a dense 9C x 9C FP64 matrix
+ * and factored by a tiled Cholesky on the GPU (the factorisation and both
+ * triangular solves in one cooperative launch), for problems with
+ * 9C <= BA_DENSE_MAX_DIM (the matrix and its tiles take 81 C^2 x 8 bytes each,
+ * plus up to 8 partial copies of S while it is built for small C); a trial
+ * whose S is not positive definite in FP64 takes a zero step (rejected,
+ * counted in ba_iter_stats.precond_fallbacks). */
 enum { BA_SOLVER_PCG = 0, BA_SOLVER_CHOLESKY = 1 };
 #define BA_DENSE_MAX_DIM 18432
 
@@ -117,7 +117,8 @@ typedef struct {
   int32_t accepted;   /* 1 if theta <- theta + Delta */
   int32_t pcg_iters;  /* PCG iterations run */
   int32_t precond_fallbacks; /* cameras whose block-Jacobi block was not SPD;
-                                with BA_SOLVER_CHOLESKY: 1 if S was not */
+                                with BA_SOLVER_CHOLESKY: 1 if S was not;
+                                one more if a wait of the solve ran out */
   int32_t reserved;
 } ba_iter_stats;
 
@@ -348,6 +349,13 @@ ba_status ba_csr_build(const int32_t* keys, int n, int n_keys,
 ba_status ba_csr_build_noalloc(const int32_t* keys, int n, int n_keys,
                                int32_t* perm_out, int32_t* rowptr_out,
                                void* stream);
+
+/* The polls after which a grid-wide wait of h's PCG gives up (at least 0.7 us
+ * each; 0 or more than the default of 2^21, about a second or more: the
+ * default).  A wait that runs out ends the solve with dc = 0 for every camera,
+ * rel_res 1 and one count in ba_iter_stats.precond_fallbacks; no answer is a
+ * mixture of solved and unsolved cameras.  The paper has no counterpart. */
+ba_status ba_set_wait_limit(ba_problem* h, unsigned int polls);
 
 /* Number of kernel launches the library has issued in this process (for
  * launch accounting in benchmarks; graph replays count every node).

@@ -264,6 +264,11 @@ class Problem:
         names = ("pieces", "chunks", "fused_a", "stored")
         return {k: int(v) for k, v in zip(names, out)}
 
+    def set_wait_limit(self, polls: int):
+        """Polls after which a grid-wide wait of the PCG gives up (0: the
+        default, about a second); the solve then returns dc = 0."""
+        _lib.check(_L().ba_set_wait_limit(self._h, int(polls)))
+
     def profile_trials(self, iters: int):
         """Run iters LM trials with a CUDA event pair around every launch;
         returns {kernel class: (total ms, launches)} and the trials' total ms."""

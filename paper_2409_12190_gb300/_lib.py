@@ -93,6 +93,7 @@ SIGNATURES = {
     "ba_project": (_S, [_I, _I, _I, _I, _VP, _VP, _VP, _VP, _VP, _VP]),
     "ba_csr_build": (_S, [_VP, _I, _I, _VP, _VP, _VP]),
     "ba_csr_build_noalloc": (_S, [_VP, _I, _I, _VP, _VP, _VP]),
+    "ba_set_wait_limit": (_S, [_VP, ct.c_uint]),
     "ba_kernel_launch_count": (ct.c_uint64, []),
     "ba_profile_trials": (_S, [_VP, _I, ct.POINTER(ba_kernel_times)]),
     "ba_measure_fma_peak": (_S, [_I, ct.POINTER(_D), _VP]),

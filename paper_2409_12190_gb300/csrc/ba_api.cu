@@ -246,6 +246,11 @@ void enqueue_schur_product(ba_problem* h, const T* xc, int k, int check_done) {
 }
 
 // One PCG pass pair plus the vector updates of iteration k.
+// The error word of the vector launches' exchange, after its slots.
+int* vec_error(ba_problem* h) {
+  return h->vec_gx ? reinterpret_cast<int*>(h->vec_gx + gx_bytes(h->ncb) / 8) : nullptr;
+}
+
 template <typename T, bool MF>
 void enqueue_pcg_iter(ba_problem* h, const double* lam_ptr, int k, double tol) {
   cudaStream_t s = h->s;
@@ -255,7 +260,7 @@ void enqueue_pcg_iter(ba_problem* h, const double* lam_ptr, int k, double tol) {
     Prof pr(h, BA_K_OTHER, k);
     VecArgs<T> a{h->C, h->cam_piece_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr, dmin, dmax, h->Minv, h->fixed,
                  h->x, h->r, h->p, (T*)h->pT, h->dot_rz + h->ncb, h->dot_bb, h->vec_scal, k, tol,
-                 GridX{h->vec_gx, reinterpret_cast<int*>(h->vec_gx + gx_bytes(h->ncb) / 8)}, h->st};
+                 GridX{h->vec_gx, vec_error(h), h->wait_polls}, h->st};
     void* args[] = {&a};
     cudaLaunchCooperativeKernel((const void*)k_pcg_vectors<T, MF>, dim3(h->ncb), dim3(VT), args, 0, s);
     count_launch();
@@ -425,8 +430,12 @@ void enqueue_solve(ba_problem* h, const double* lam_ptr, int maxiter, double tol
   }
   {
     Prof pr(h, BA_K_OTHER);
+    // the error word of the exchange that this solve's PCG went through
+    const int* lost = nullptr;
+    if (h->opt.solver == BA_SOLVER_PCG && !h->xch)
+      lost = h->sx.pcg ? reinterpret_cast<const int*>(h->sx.gx + h->sx.words - 1) : vec_error(h);
     k_cam_trial<T, MF><<<h->ncb, CAM_THREADS, 0, s>>>(h->C, h->x, h->gc, (T*)h->cams, (const T*)h->camtab, h->st,
-                                                     (T*)h->xT, h->dot_gc);
+                                                     (T*)h->xT, h->dot_gc, lost);
   }
   if (MF && h->fa) {
     Prof pr(h, BA_K_BACKSUB);
@@ -1680,6 +1689,18 @@ ba_status ba_learn_slow_probes(ba_problem* h, double lambda, int n, const int* i
 }
 
 uint64_t ba_kernel_launch_count(void) { return ba::g_launches.load(); }
+
+ba_status ba_set_wait_limit(ba_problem* h, unsigned int polls) {
+  if (!h) return fail(BA_ERR_INVALID_ARG, "NULL problem");
+  h->wait_polls = polls ? std::min(polls, 1u << 21) : 1u << 21;
+  if (h->gexec) {
+    // the captured trial has the other limit: capture again on next use
+    CU(cudaStreamSynchronize(h->s));
+    cudaGraphExecDestroy(h->gexec);
+    h->gexec = nullptr;
+  }
+  return BA_OK;
+}
 
 ba_status ba_set_exchange(ba_problem* h, ba_exchange_fn fn, void* ctx, double* xbuf, size_t cap) {
   if (!h) return fail(BA_ERR_INVALID_ARG, "NULL problem");

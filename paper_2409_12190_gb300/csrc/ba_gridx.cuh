@@ -33,13 +33,14 @@ __host__ __device__ constexpr size_t gx_bytes(int blocks) {
   return 2ull * GX_COPIES * (size_t)blocks * GX_WORDS * sizeof(unsigned long long);
 }
 
-// Polls before a wait gives up (each at least an L2 round trip of about
-// 0.7 us: a second or more in all).
+// Polls before a wait gives up by default (each at least an L2 round trip of
+// about 0.7 us: a second or more in all).
 constexpr unsigned int GX_SPINS = 1u << 21;
 
 struct GridX {
   unsigned long long* slots;  // gx_bytes(gridDim.x)
   int* err;                   // set by a wait that ran out; every later wait returns
+  unsigned int spins;         // polls before a wait gives up
 };
 
 // Two 64-bit words at a 16-byte boundary; each word carries its own epoch, so
@@ -65,9 +66,10 @@ __device__ __forceinline__ double gx_value(unsigned long long a, unsigned long l
 }
 // Whether a wait of `spins` polls gives up (the caller then stops for good).
 __device__ __forceinline__ bool gx_give_up(const GridX& gx, unsigned int spins) {
-  if ((spins & 63) != 63) return false;
+  const bool out = spins >= gx.spins;
+  if (!out && (spins & 63) != 63) return false;
   cuda::atomic_ref<int, cuda::thread_scope_device> err(*gx.err);
-  if (spins < GX_SPINS && !err.load(cuda::memory_order_relaxed)) return false;
+  if (!out && !err.load(cuda::memory_order_relaxed)) return false;
   err.store(1, cuda::memory_order_relaxed);
   return true;
 }

@@ -2419,14 +2419,25 @@ __device__ __forceinline__ double cam_trial_one(const double* __restrict__ xc, c
 }
 
 // Trial cameras theta_c + dc (dc rounded to T), dc in the pass form, partial
-// gc . dc.
+// gc . dc.  lost (or NULL): set if a grid-wide wait of the PCG ran out; the
+// blocks it stopped and those that got through left a mixture, so dc becomes 0
+// for every camera, counted as the direct solver's failures are.
 template <typename T, bool MF>
 static __global__ void __launch_bounds__(CAM_THREADS)
-k_cam_trial(int C, const double* __restrict__ x, const double* __restrict__ gc, T* __restrict__ cams_buf,
-            const T* __restrict__ camtab, const DevState* __restrict__ st, T* __restrict__ xT,
-            double* __restrict__ dot_gc) {
+k_cam_trial(int C, double* __restrict__ x, const double* __restrict__ gc, T* __restrict__ cams_buf,
+            const T* __restrict__ camtab, DevState* __restrict__ st, T* __restrict__ xT,
+            double* __restrict__ dot_gc, const int* __restrict__ lost) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   double gd = 0.0;
+  if (lost && *lost) {
+    if (c < C)
+      for (int i = 0; i < 9; ++i) x[9LL * c + i] = 0.0;
+    if (c == 0) {
+      st->fallbacks += 1;
+      st->pcg_rel = 1.0;
+      st->pcg_done = 1;
+    }
+  }
   if (c < C) {
     const int cur = st->cur;
     gd = cam_trial_one<T, MF>(x + 9LL * c, gc + 9LL * c, cams_buf + (long long)cur * 9 * C + 9LL * c,

@@ -387,7 +387,7 @@ ba_status enqueue_solve(ba_pgo* h, const double* lam_ptr, int maxiter, double to
   a.maxiter = maxiter;
   a.tol = tol;
   a.bar = h->bar;
-  a.gx = GridX{h->gx_words, &h->bar->err};
+  a.gx = GridX{h->gx_words, &h->bar->err, GX_SPINS};
   a.st = h->st;
   void* args[] = {&a};
   if (h->pcg_res_smem) {

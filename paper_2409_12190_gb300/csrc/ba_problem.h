@@ -143,6 +143,7 @@ struct ba_problem {
   // the PCG's vector work in one launch (ba_vec.cuh) where its blocks fit the GPU
   unsigned long long* vec_gx = nullptr;  // exchange slots, then the error flag
   double* vec_scal = nullptr;            // [4]
+  unsigned int wait_polls = 1u << 21;    // of the PCG's grid-wide waits (ba_set_wait_limit)
   bool batched = false;  // the concatenated problems of a batch: never solved as one
   ba::DevState* st = nullptr;
   ba_iter_stats* stats = nullptr;

@@ -469,7 +469,7 @@ void pcg(ba_problem* h, int maxiter, double tol) {
   a.x = h->x;
   a.maxiter = maxiter;
   a.tol = tol;
-  a.gx = GridX{x.gx, reinterpret_cast<int*>(x.gx + x.words - 1)};
+  a.gx = GridX{x.gx, reinterpret_cast<int*>(x.gx + x.words - 1), h->wait_polls};
   a.st = h->st;
   void* args[] = {&a};
   cudaLaunchCooperativeKernel((const void*)k_schur_pcg<VT>, dim3(x.groups), dim3(SX_THREADS), args,

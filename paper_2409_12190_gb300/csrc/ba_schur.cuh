@@ -613,13 +613,13 @@ static __global__ void __launch_bounds__(SX_THREADS, 1) k_schur_pcg(SchurPcg<VT>
       break;
     }
   }
-  // a wait that ran out: no step, counted (as the direct solver does)
-  if (live) a.x[o] = lost ? 0.0 : xa;
+  // after a wait that ran out k_cam_trial makes it no step (each block knows
+  // only of its own waits, and some may have got through)
+  if (live) a.x[o] = xa;
   if (g == 0 && tid == 0) {
-    if (lost) a.st->fallbacks += 1;
     a.st->pcg_iters = it;
-    a.st->pcg_rel = lost ? 1.0 : it > 0 ? (bb > 0.0 ? sqrt(rr / bb) : 0.0) : done ? 0.0 : 1.0;
-    a.st->pcg_done = done | lost;
+    a.st->pcg_rel = it > 0 ? (bb > 0.0 ? sqrt(rr / bb) : 0.0) : done ? 0.0 : 1.0;
+    a.st->pcg_done = done;
   }
 }
 
