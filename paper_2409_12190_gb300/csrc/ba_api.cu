@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "ba.h"
+#include "ba_capture.h"
 #include "ba_internal.h"
 #include "ba_band.cuh"
 #include "ba_kernels.cuh"
@@ -1283,11 +1284,12 @@ ba_status ba_solve(ba_problem* h, int iters, void* stream) {
   }
   if (!h->gexec && iters > 0) {
     cudaGraph_t g = nullptr;
+    cudaGetLastError();
     CU(cudaStreamBeginCapture(h->s, cudaStreamCaptureModeThreadLocal));
     ba::g_capturing = true;
     enqueue_trial_any(h);
     ba::g_capturing = false;
-    cudaError_t e = cudaStreamEndCapture(h->s, &g);
+    cudaError_t e = end_capture(h->s, &g);
     if (e != cudaSuccess) return fail(BA_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(e));
     size_t n = 0;
     cudaGraphGetNodes(g, nullptr, &n);
@@ -1766,7 +1768,9 @@ ba_status ba_profile_trials(ba_problem* h, int iters, ba_kernel_times* out) {
   }
   CU(cudaEventRecord(eb, h->s));
   h->prof = nullptr;
-  cudaError_t e = cudaStreamSynchronize(h->s);
+  cudaError_t e = cudaGetLastError();
+  const cudaError_t es = cudaStreamSynchronize(h->s);
+  if (e == cudaSuccess) e = es;
   std::vector<ba_iter_stats> st(iters);
   for (int i = 0; i < iters && e == cudaSuccess; ++i)
     e = cudaMemcpy(&st[i], h->stats + ((t0 + i) % h->cap), sizeof(ba_iter_stats), cudaMemcpyDeviceToHost);
