@@ -368,7 +368,8 @@ enum {
   BA_LAYOUT_CHUNKS = 1,  /* point chunks (one CTA each in the point-major passes) */
   BA_LAYOUT_FUSED_A = 2, /* 1 if pass A runs fused (point-major, recompute mode) */
   BA_LAYOUT_STORED = 3,  /* 1 if the Jacobian blocks are stored (BA_JAC_STORE) */
-  BA_LAYOUT_COUNT = 4
+  BA_LAYOUT_PRODUCT_PIECES = 4, /* pieces of the implicit product's camera pass and of F */
+  BA_LAYOUT_COUNT = 5
 };
 
 /* Layout counts of problem h (see the enum above) into out[0 .. n) (host;

@@ -258,10 +258,11 @@ class Problem:
         return dpix, dc0, dp0, it.value, rel.value
 
     def layout(self):
-        """Layout counts: pieces, chunks, fused_a (1/0), stored (1/0)."""
-        out = (ct.c_int64 * 4)()
-        _lib.check(_L().ba_get_layout(self._h, out, 4))
-        names = ("pieces", "chunks", "fused_a", "stored")
+        """Layout counts: pieces, chunks, fused_a (1/0), stored (1/0),
+        product_pieces."""
+        names = ("pieces", "chunks", "fused_a", "stored", "product_pieces")
+        out = (ct.c_int64 * len(names))()
+        _lib.check(_L().ba_get_layout(self._h, out, len(names)))
         return {k: int(v) for k, v in zip(names, out)}
 
     def set_wait_limit(self, polls: int):

@@ -199,8 +199,8 @@ void enqueue_schur_product(ba_problem* h, const T* xc, int k, int check_done) {
       constexpr int UB = (MF && std::is_same<T, float>::value) ? 2 : 1;
       constexpr int NT = UB > 1 ? PASSB_THREADS : PIECE_THREADS;
       auto pb = h->cm_sw ? k_pass_b<T, MF, UB, (UB > 1), NT, true> : k_pass_b<T, MF, UB, (UB > 1), NT, false>;
-      pb<<<h->npieces, NT, 0, s>>>(
-          h->piece_cam, h->piece_beg, h->piece_end, h->cm_pt, (const T*)h->Jcm, (const T*)h->cm_sw,
+      pb<<<h->nlong, NT, 0, s>>>(
+          h->long_cam, h->long_beg, h->long_end, h->cm_pt, (const T*)h->Jcm, (const T*)h->cm_sw,
           (const T*)h->ptab, (const T*)h->camtab, h->st, check_done, h->O, h->part);
     }
     count_launch(2);
@@ -215,8 +215,8 @@ void enqueue_schur_product(ba_problem* h, const T* xc, int k, int check_done) {
     }
     {
       Prof pr(h, BA_K_PASS_B, k);
-      k_pass_b<T, MF><<<h->npieces, PIECE_THREADS, 0, s>>>(
-          h->piece_cam, h->piece_beg, h->piece_end, h->cm_pt, (const T*)h->Jcm, (const T*)h->cm_sw,
+      k_pass_b<T, MF><<<h->nlong, PIECE_THREADS, 0, s>>>(
+          h->long_cam, h->long_beg, h->long_end, h->cm_pt, (const T*)h->Jcm, (const T*)h->cm_sw,
           (const T*)h->ptab, (const T*)h->camtab, h->st, check_done, h->O, h->part);
     }
     count_launch(2);
@@ -224,8 +224,8 @@ void enqueue_schur_product(ba_problem* h, const T* xc, int k, int check_done) {
   }
   {
     Prof pr(h, BA_K_PASS_A, k);
-    k_pass_a1<T, MF><<<h->npieces, PIECE_THREADS, 0, s>>>(
-        h->piece_cam, h->piece_beg, h->piece_end, h->cm_pt, (const T*)h->Jcm, (const T*)h->cm_sw,
+    k_pass_a1<T, MF><<<h->nlong, PIECE_THREADS, 0, s>>>(
+        h->long_cam, h->long_beg, h->long_end, h->cm_pt, (const T*)h->Jcm, (const T*)h->cm_sw,
         (const T*)h->ptab, (const T*)h->camtab, xc, h->st, check_done, h->O, (T*)h->zbuf);
   }
   {
@@ -239,19 +239,19 @@ void enqueue_schur_product(ba_problem* h, const T* xc, int k, int check_done) {
     constexpr int UB = (MF && std::is_same<T, float>::value) ? 2 : 1;
     constexpr int NT = UB > 1 ? PASSB_THREADS : PIECE_THREADS;
     auto pb = h->cm_sw ? k_pass_b<T, MF, UB, (UB > 1), NT, true> : k_pass_b<T, MF, UB, (UB > 1), NT, false>;
-    pb<<<h->npieces, NT, 0, s>>>(
-        h->piece_cam, h->piece_beg, h->piece_end, h->cm_pt, (const T*)h->Jcm, (const T*)h->cm_sw,
+    pb<<<h->nlong, NT, 0, s>>>(
+        h->long_cam, h->long_beg, h->long_end, h->cm_pt, (const T*)h->Jcm, (const T*)h->cm_sw,
         (const T*)h->ptab, (const T*)h->camtab, h->st, check_done, h->O, h->part);
   }
   count_launch(3);
 }
 
-// One PCG pass pair plus the vector updates of iteration k.
 // The error word of the vector launches' exchange, after its slots.
 int* vec_error(ba_problem* h) {
   return h->vec_gx ? reinterpret_cast<int*>(h->vec_gx + gx_bytes(h->ncb) / 8) : nullptr;
 }
 
+// One PCG pass pair plus the vector updates of iteration k.
 template <typename T, bool MF>
 void enqueue_pcg_iter(ba_problem* h, const double* lam_ptr, int k, double tol) {
   cudaStream_t s = h->s;
@@ -259,7 +259,7 @@ void enqueue_pcg_iter(ba_problem* h, const double* lam_ptr, int k, double tol) {
   enqueue_schur_product<T, MF>(h, (const T*)h->pT, k, 1);
   if (h->vec_gx && !h->xch) {
     Prof pr(h, BA_K_OTHER, k);
-    VecArgs<T> a{h->C, h->cam_piece_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr, dmin, dmax, h->Minv, h->fixed,
+    VecArgs<T> a{h->C, h->cam_long_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr, dmin, dmax, h->Minv, h->fixed,
                  h->x, h->r, h->p, (T*)h->pT, h->dot_rz + h->ncb, h->dot_bb, h->vec_scal, k, tol,
                  GridX{h->vec_gx, vec_error(h), h->wait_polls}, h->st};
     void* args[] = {&a};
@@ -269,7 +269,7 @@ void enqueue_pcg_iter(ba_problem* h, const double* lam_ptr, int k, double tol) {
   }
   if (h->xch) {
     // the pass-B sums of every part (9C values), one row per camera
-    k_cam_sum_parts<<<nblk(9LL * h->C, 256), 256, 0, s>>>(h->C, h->cam_piece_ptr, h->part, 9, 9, h->camsum);
+    k_cam_sum_parts<<<nblk(9LL * h->C, 256), 256, 0, s>>>(h->C, h->cam_long_ptr, h->part, 9, 9, h->camsum);
     count_launch();
     xchg(h, h->camsum, 9ull * h->C);
     Prof pr(h, BA_K_OTHER, k);
@@ -277,7 +277,7 @@ void enqueue_pcg_iter(ba_problem* h, const double* lam_ptr, int k, double tol) {
                                            dmin, dmax, h->p, h->q, h->dot_pq, h->fixed, h->st, 1);
   } else {
     Prof pr(h, BA_K_OTHER, k);
-    k_pcg_q<T, MF><<<h->ncb, VT, 0, s>>>(h->C, h->cam_piece_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr,
+    k_pcg_q<T, MF><<<h->ncb, VT, 0, s>>>(h->C, h->cam_long_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr,
                                         dmin, dmax, h->p, h->q, h->dot_pq, h->fixed, h->st, 1);
   }
   count_launch(3);
@@ -305,7 +305,7 @@ void enqueue_coupling(ba_problem* h, const double* lam_ptr) {
   for (int k = 0; k < COUPLING_PROBES; ++k) {
     k_coup_probe_in<T, MF><<<nblk(h->C, 128), 128, 0, s>>>(h->C, k, h->Sii, (const T*)h->camtab, h->p, (T*)h->pT);
     enqueue_schur_product<T, MF>(h, (const T*)h->pT, -1, 0);
-    k_pcg_q<T, MF><<<h->ncb, VT, 0, s>>>(h->C, h->cam_piece_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr,
+    k_pcg_q<T, MF><<<h->ncb, VT, 0, s>>>(h->C, h->cam_long_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr,
                                         dmin, dmax, h->p, h->q, nullptr, h->fixed, h->st, 0);
     k_coup_acc<<<nblk(h->C, 128), 128, 0, s>>>(h->C, k, h->Sii, h->q, h->kap);
     count_launch(3);
@@ -467,19 +467,19 @@ void enqueue_solve(ba_problem* h, const double* lam_ptr, int maxiter, double tol
 template <typename T, bool MF>
 void enqueue_cost(ba_problem* h, bool gated = false) {
   const T delta = (T)(h->opt.huber_delta > 0 ? h->opt.huber_delta : 0.0);
-  k_cost_cam<T, false, MF><<<h->ncost, PIECE_THREADS, 0, h->s>>>(
-      h->cost_cam, h->cost_beg, h->cost_end, h->cm_pt, (const T*)h->cm_px, (const T*)h->cams,
+  k_cost_cam<T, false, MF><<<h->nlong, PIECE_THREADS, 0, h->s>>>(
+      h->long_cam, h->long_beg, h->long_end, h->cm_pt, (const T*)h->cm_px, (const T*)h->cams,
       (const T*)h->pts, h->st, gated ? 2 : 0, delta, h->C, h->P, h->O, nullptr, nullptr, nullptr, nullptr, nullptr,
       h->part);
   if (h->xch) {
     // the cost over every part (0 from each part when F is not stale)
-    k_part_cost_sum<<<1, 256, 0, h->s>>>(h->ncost, h->part, h->st, gated ? 1 : 0, h->xscal + 4);
+    k_part_cost_sum<<<1, 256, 0, h->s>>>(h->nlong, h->part, h->st, gated ? 1 : 0, h->xscal + 4);
     xchg(h, h->xscal + 4, 1);
     k_cost_set<<<1, 1, 0, h->s>>>(h->st, gated ? 1 : 0, h->xscal + 4);
     count_launch(3);
     return;
   }
-  k_cost_finalize<<<1, 256, 0, h->s>>>(h->ncost, h->part, h->st, gated ? 1 : 0);
+  k_cost_finalize<<<1, 256, 0, h->s>>>(h->nlong, h->part, h->st, gated ? 1 : 0);
   count_launch(2);
 }
 
@@ -574,7 +574,7 @@ void enqueue_matvec(ba_problem* h, const double* lam_ptr) {
                                                             (T*)h->y0, h->st);
   k_pass_vec<T, MF><<<nblk(h->C, 128), 128, 0, s>>>(h->C, h->p, (const T*)h->camtab, (T*)h->pT);
   enqueue_schur_product<T, MF>(h, (const T*)h->pT, -1, 0);
-  k_pcg_q<T, MF><<<h->ncb, VT, 0, s>>>(h->C, h->cam_piece_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr,
+  k_pcg_q<T, MF><<<h->ncb, VT, 0, s>>>(h->C, h->cam_long_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr,
                                       dmin, dmax, h->p, h->q, nullptr, h->fixed, h->st, 0);
   count_launch(3);
 }
@@ -783,13 +783,11 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
     if (sb != BA_OK) return sb;
   }
 
-  // pieces: each camera's slots cut into runs of at most piece_max.  The
-  // camera passes of one linearisation are then all a trial runs over the
-  // pieces when S is formed, one block of 64 threads each: about six blocks
-  // an SM keep the FP64 pipes busy (16 cameras: 16 pieces of 500 slots took
-  // 100 us a pass, 250 cameras: 250 pieces 375 us, twice what its arithmetic
-  // takes).  The implicit product runs over them in every iteration and adds a
-  // reduction for each: as long as they may be.
+  // pieces: each camera's slots cut into runs of at most piece_max.  Where S is
+  // formed the camera passes of one linearisation are all that a trial runs
+  // over them, one block of 64 threads each: about six blocks an SM keep the
+  // FP64 pipes busy (16 cameras: 16 pieces of 500 slots took 100 us a pass, 250
+  // cameras: 250 pieces 375 us, twice what its arithmetic takes).
   int piece_max = PIECE;
   if (h->sx.pcg || h->sx.direct) {
     int dev = 0, nsm = 1;
@@ -798,13 +796,14 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
     const long long per = O / (6LL * nsm);
     piece_max = (int)std::min<long long>(PIECE, std::max<long long>(LIN_THREADS, (per + LIN_THREADS - 1) / LIN_THREADS * LIN_THREADS));
   }
-  // F itself keeps the pieces of PIECE slots: a batch of problems adds it in
-  // the same order.
+  // The implicit product adds a reduction for each piece in every product: as
+  // long as they may be (250 cameras, 480,000 observations, FP64: a product
+  // 153 us with pieces of 2,048, 167 us with 576).  F keeps them too: a batch of
+  // problems adds it in the same order.
   std::vector<int32_t> rp(C + 1);
   CU(cudaMemcpy(rp.data(), h->rowptr_cam, (C + 1) * 4, cudaMemcpyDeviceToHost));
-  std::vector<int32_t> cpp(C + 1);
-  auto cut = [&](int most, int* count, int32_t** d_cam, int32_t** d_beg, int32_t** d_end) -> ba_status {
-    std::vector<int32_t> pc, pb, pe;
+  auto cut = [&](int most, int* count, int32_t** d_cam, int32_t** d_beg, int32_t** d_end, int32_t** d_ptr) -> ba_status {
+    std::vector<int32_t> pc, pb, pe, cpp(C + 1);
     for (long long c = 0; c < C; ++c) {
       cpp[c] = (int32_t)pc.size();
       const int n = rp[c + 1] - rp[c];
@@ -820,27 +819,27 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
     CU(h->alloc(d_cam, pc.size() * 4));
     CU(h->alloc(d_beg, pc.size() * 4));
     CU(h->alloc(d_end, pc.size() * 4));
+    CU(h->alloc(d_ptr, (C + 1) * 4));
     CU(cudaMemcpy(*d_cam, pc.data(), pc.size() * 4, cudaMemcpyHostToDevice));
     CU(cudaMemcpy(*d_beg, pb.data(), pb.size() * 4, cudaMemcpyHostToDevice));
     CU(cudaMemcpy(*d_end, pe.data(), pe.size() * 4, cudaMemcpyHostToDevice));
+    CU(cudaMemcpy(*d_ptr, cpp.data(), (C + 1) * 4, cudaMemcpyHostToDevice));
     return BA_OK;
   };
-  if (piece_max != PIECE) {
-    const ba_status cs = cut(PIECE, &h->ncost, &h->cost_cam, &h->cost_beg, &h->cost_end);
-    if (cs != BA_OK) return cs;
-  }
   {
-    const ba_status cs = cut(piece_max, &h->npieces, &h->piece_cam, &h->piece_beg, &h->piece_end);
+    const ba_status cs = cut(PIECE, &h->nlong, &h->long_cam, &h->long_beg, &h->long_end, &h->cam_long_ptr);
     if (cs != BA_OK) return cs;
   }
-  if (piece_max == PIECE) {
-    h->ncost = h->npieces;
-    h->cost_cam = h->piece_cam;
-    h->cost_beg = h->piece_beg;
-    h->cost_end = h->piece_end;
+  if (piece_max != PIECE) {
+    const ba_status cs = cut(piece_max, &h->npieces, &h->piece_cam, &h->piece_beg, &h->piece_end, &h->cam_piece_ptr);
+    if (cs != BA_OK) return cs;
+  } else {
+    h->npieces = h->nlong;
+    h->piece_cam = h->long_cam;
+    h->piece_beg = h->long_beg;
+    h->piece_end = h->long_end;
+    h->cam_piece_ptr = h->cam_long_ptr;
   }
-  CU(h->alloc(&h->cam_piece_ptr, (C + 1) * 4));
-  CU(cudaMemcpy(h->cam_piece_ptr, cpp.data(), (C + 1) * 4, cudaMemcpyHostToDevice));
 
   // linearisation and solver buffers
   CU(h->alloc(&h->camtab, CT * C * ts));
@@ -1042,7 +1041,7 @@ void enqueue_collect(ba_problem* h, const double* lam_ptr, int K, const float* z
     k_probe_in<T, MF><<<nblk(h->C, 128), 128, 0, s>>>(h->C, K, k, zhat, h->Dsc, (const T*)h->camtab, h->p,
                                                       (T*)h->pT);
     enqueue_schur_product<T, MF>(h, (const T*)h->pT, -1, 0);
-    k_pcg_q<T, MF><<<h->ncb, VT, 0, s>>>(h->C, h->cam_piece_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr, dmin,
+    k_pcg_q<T, MF><<<h->ncb, VT, 0, s>>>(h->C, h->cam_long_ptr, h->part, h->U, (const T*)h->camtab, lam_ptr, dmin,
                                         dmax, h->p, h->q, nullptr, h->fixed, h->st, 0);
     k_probe_out<<<nblk(h->C, 128), 128, 0, s>>>(h->C, K, k, h->q, h->Dsc, Yhat);
     count_launch(3);
@@ -1743,7 +1742,7 @@ ba_status ba_set_exchange(ba_problem* h, ba_exchange_fn fn, void* ctx, double* x
 
 ba_status ba_get_layout(const ba_problem* h, int64_t* out, int n) {
   if (!h || !out || n < 0) return fail(BA_ERR_INVALID_ARG, "bad argument");
-  const int64_t v[BA_LAYOUT_COUNT] = {h->npieces, h->nchunks, h->fa ? 1 : 0, h->mf ? 0 : 1};
+  const int64_t v[BA_LAYOUT_COUNT] = {h->npieces, h->nchunks, h->fa ? 1 : 0, h->mf ? 0 : 1, h->nlong};
   for (int i = 0; i < n; ++i) out[i] = i < BA_LAYOUT_COUNT ? v[i] : 0;
   return BA_OK;
 }

@@ -79,8 +79,8 @@ struct ba_problem {
   void *cm_px = nullptr, *pm_px = nullptr, *px_in = nullptr;
   int npieces = 0;
   int32_t *piece_cam = nullptr, *piece_beg = nullptr, *piece_end = nullptr, *cam_piece_ptr = nullptr;
-  int ncost = 0;  // pieces of F
-  int32_t *cost_cam = nullptr, *cost_beg = nullptr, *cost_end = nullptr;
+  int nlong = 0;  // pieces of F and of the implicit product (the same, or longer)
+  int32_t *long_cam = nullptr, *long_beg = nullptr, *long_end = nullptr, *cam_long_ptr = nullptr;
   // parameters, double-buffered (current / trial)
   void *cams = nullptr, *pts = nullptr;
   // linearisation
