@@ -141,6 +141,16 @@ ba_status ba_problem_create(ba_problem** out, int C, int P, int O,
                             const void* pixels, const ba_options* opt,
                             void* stream);
 
+/* ba_problem_create for a problem that ba_set_exchange makes one part of a
+ * partitioned problem: its PCG keeps the implicit product (a formed S would
+ * be this part's alone), so the pairs of observations are not sorted.  The
+ * paper has no counterpart. */
+ba_status ba_problem_create_part(ba_problem** out, int C, int P, int O,
+                                 const void* cams, const void* points,
+                                 const int32_t* cam_idx, const int32_t* pt_idx,
+                                 const void* pixels, const ba_options* opt,
+                                 void* stream);
+
 /* Free a problem and everything it owns (NULL is accepted).  Resource
  * management: no counterpart in the paper. */
 ba_status ba_problem_destroy(ba_problem* h);
@@ -273,7 +283,9 @@ typedef int (*ba_exchange_fn)(size_t n, void* stream, void* ctx);
  * exchange; the cost is re-evaluated (summed) at the next trial.  The
  * step-level entry points, the learned preconditioner, the direct solver and
  * ba_backward act on this part alone and are not for partitioned use.
- * Synchronises. */
+ * A problem whose PCG had S formed gives that up, also for when it is a
+ * problem of its own again (ba_problem_create_part does not form it in the
+ * first place).  Synchronises. */
 ba_status ba_set_exchange(ba_problem* h, ba_exchange_fn fn, void* ctx, double* xbuf, size_t cap);
 
 /* ---- step-level entry points (same arithmetic as ba_lm_step) ---------- */
@@ -369,7 +381,9 @@ enum {
   BA_LAYOUT_FUSED_A = 2, /* 1 if pass A runs fused (point-major, recompute mode) */
   BA_LAYOUT_STORED = 3,  /* 1 if the Jacobian blocks are stored (BA_JAC_STORE) */
   BA_LAYOUT_PRODUCT_PIECES = 4, /* pieces of the implicit product's camera pass and of F */
-  BA_LAYOUT_COUNT = 5
+  BA_LAYOUT_FORMED = 5,         /* S formed from pairs of observations: 1 for the PCG, 2 for the direct solver;
+                                   0: the implicit product, or the direct solver's other build */
+  BA_LAYOUT_COUNT = 6
 };
 
 /* Layout counts of problem h (see the enum above) into out[0 .. n) (host;

@@ -117,6 +117,8 @@ class Problem:
     int32, pixels [O, 2]; any device (copied), float dtype converted to the
     options' precision."""
 
+    _create = "ba_problem_create"
+
     def __init__(self, cams, points, cam_idx, pt_idx, pixels, options: Options | None = None,
                  device="cuda", stream=None):
         self.options = options or Options()
@@ -131,9 +133,9 @@ class Problem:
         self.C, self.P, self.O = int(cams.shape[0]), int(points.shape[0]), int(ci.shape[0])
         h = ct.c_void_p()
         o = self.options.to_c()
-        _lib.check(_L().ba_problem_create(ct.byref(h), self.C, self.P, self.O, _ptr(cams),
-                                          _ptr(points), _ptr(ci), _ptr(pi), _ptr(px), ct.byref(o),
-                                          _stream(stream)))
+        _lib.check(getattr(_L(), self._create)(ct.byref(h), self.C, self.P, self.O, _ptr(cams),
+                                               _ptr(points), _ptr(ci), _ptr(pi), _ptr(px), ct.byref(o),
+                                               _stream(stream)))
         self._h = h
 
     # -- lifetime ---------------------------------------------------------
@@ -259,8 +261,9 @@ class Problem:
 
     def layout(self):
         """Layout counts: pieces, chunks, fused_a (1/0), stored (1/0),
-        product_pieces."""
-        names = ("pieces", "chunks", "fused_a", "stored", "product_pieces")
+        product_pieces, formed (1: the PCG on formed S, 2: the direct solver's
+        S from pairs of observations, 0: neither)."""
+        names = ("pieces", "chunks", "fused_a", "stored", "product_pieces", "formed")
         out = (ct.c_int64 * len(names))()
         _lib.check(_L().ba_get_layout(self._h, out, len(names)))
         return {k: int(v) for k, v in zip(names, out)}

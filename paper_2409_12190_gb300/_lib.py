@@ -74,6 +74,8 @@ SIGNATURES = {
     "ba_options_default": (_S, [ct.POINTER(ba_options)]),
     "ba_problem_create": (_S, [ct.POINTER(_VP), _I, _I, _I, _VP, _VP, _VP, _VP, _VP,
                                ct.POINTER(ba_options), _VP]),
+    "ba_problem_create_part": (_S, [ct.POINTER(_VP), _I, _I, _I, _VP, _VP, _VP, _VP, _VP,
+                                    ct.POINTER(ba_options), _VP]),
     "ba_problem_destroy": (_S, [_VP]),
     "ba_lm_step": (_S, [_VP, _VP]),
     "ba_solve": (_S, [_VP, _I, _VP]),

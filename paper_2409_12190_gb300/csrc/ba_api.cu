@@ -597,6 +597,25 @@ ba_status check_options(const ba_options* o) {
   return BA_OK;
 }
 
+// One cooperative launch for an iteration's vector work while its blocks (32
+// cameras each) are resident at once (some 18,900 cameras; beyond, they cannot
+// wait for one another): 17.7 us against 27.7 at 4,000.
+template <typename T>
+ba_status vec_setup(ba_problem* h) {
+  int dev = 0, nsm = 0, coop = 0, occ = 0;
+  CU(cudaGetDevice(&dev));
+  CU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+  CU(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
+  const void* kern = h->mf ? (const void*)k_pcg_vectors<T, true> : (const void*)k_pcg_vectors<T, false>;
+  CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, VT, 0));
+  if (!coop || (long long)occ * nsm < h->ncb) return BA_OK;
+  unsigned long long* gx = nullptr;
+  CU(h->alloc(&gx, gx_bytes(h->ncb) + 8));
+  CU(h->alloc(&h->vec_scal, 4 * sizeof(double)));
+  h->vec_gx = gx;
+  return BA_OK;
+}
+
 template <typename T>
 ba_status create_impl(ba_problem* h, const void* cams, const void* points, const int32_t* cam_idx,
                       const int32_t* pt_idx, const void* pixels) {
@@ -922,19 +941,8 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
   CU(h->alloc(&h->dot_bb, h->ncb * 8));
   CU(h->alloc(&h->dot_gc, h->ncb * 8));
   if (h->opt.solver == BA_SOLVER_PCG && !h->batched && !h->sx.pcg) {
-    // one cooperative launch for an iteration's vector work while its blocks
-    // (32 cameras each) are resident at once (some 18,900 cameras; beyond,
-    // they cannot wait for one another): 17.7 us against 27.7 at 4,000
-    int dev = 0, nsm = 0, coop = 0, occ = 0;
-    CU(cudaGetDevice(&dev));
-    CU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    CU(cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev));
-    const void* kern = h->mf ? (const void*)k_pcg_vectors<T, true> : (const void*)k_pcg_vectors<T, false>;
-    CU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, VT, 0));
-    if (coop && (long long)occ * nsm >= h->ncb) {
-      CU(h->alloc(&h->vec_gx, gx_bytes(h->ncb) + 8));
-      CU(h->alloc(&h->vec_scal, 4 * sizeof(double)));
-    }
+    const ba_status vs = vec_setup<T>(h);
+    if (vs != BA_OK) return vs;
   }
   CU(h->alloc(&h->dot_gp, std::max(h->nchunks, 1) * 8));
   h->cap = h->opt.max_stats;
@@ -1171,7 +1179,7 @@ ba_status backward_via_f64(ba_problem* h, double lambda, int maxiter, double tol
 
 ba_status ba::problem_create(ba_problem** out, int C, int P, int O, const void* cams, const void* points,
                              const int32_t* cam_idx, const int32_t* pt_idx, const void* pixels,
-                             const ba_options* opt, void* stream, bool batched) {
+                             const ba_options* opt, void* stream, bool batched, bool may_form) {
   if (!out) return fail(BA_ERR_INVALID_ARG, "NULL output handle");
   *out = nullptr;
   if (C < 1 || P < 1 || O < 1) return fail(BA_ERR_INVALID_ARG, "C, P and O must be >= 1 (got %d, %d, %d)", C, P, O);
@@ -1193,6 +1201,7 @@ ba_status ba::problem_create(ba_problem** out, int C, int P, int O, const void* 
   h->tsize = o.precision == BA_PREC_F32 ? 4 : 8;
   h->opt = o;
   h->batched = batched;
+  h->may_form = may_form;
   cudaError_t e = cudaStreamCreateWithFlags(&h->s, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_out, cudaEventDisableTiming);
@@ -1243,7 +1252,13 @@ ba_status ba_options_default(ba_options* o) {
 ba_status ba_problem_create(ba_problem** out, int C, int P, int O, const void* cams, const void* points,
                             const int32_t* cam_idx, const int32_t* pt_idx, const void* pixels,
                             const ba_options* opt, void* stream) {
-  return ba::problem_create(out, C, P, O, cams, points, cam_idx, pt_idx, pixels, opt, stream, false);
+  return ba::problem_create(out, C, P, O, cams, points, cam_idx, pt_idx, pixels, opt, stream, false, true);
+}
+
+ba_status ba_problem_create_part(ba_problem** out, int C, int P, int O, const void* cams, const void* points,
+                                 const int32_t* cam_idx, const int32_t* pt_idx, const void* pixels,
+                                 const ba_options* opt, void* stream) {
+  return ba::problem_create(out, C, P, O, cams, points, cam_idx, pt_idx, pixels, opt, stream, false, false);
 }
 
 ba_status ba_problem_destroy(ba_problem* h) {
@@ -1720,9 +1735,21 @@ ba_status ba_set_exchange(ba_problem* h, ba_exchange_fn fn, void* ctx, double* x
     CU(h->alloc(&h->gc_loc, 9ull * h->C * 8));
     CU(h->alloc(&h->xscal, 8 * 8));
   }
-  // a part's PCG runs the implicit product: its fused pass A
-  if (fn && !h->mf && h->fa && !h->Jpm) CU(h->alloc(&h->Jpm, (size_t)NPLANE * h->O * h->tsize));
   CU(cudaStreamSynchronize(h->s));
+  // a part's PCG runs the implicit product: the formed system goes (its lists
+  // and an observation's 160 bytes of lean form, written by every linearisation
+  // and read by nothing), and the product gets its fused pass A and, for when
+  // the problem is alone again, its vector launch
+  if (fn && h->sx.pcg) {
+    if (h->gexec) {
+      cudaGraphExecDestroy(h->gexec);
+      h->gexec = nullptr;
+    }
+    schur_drop(h);
+    const ba_status vs = h->prec == BA_PREC_F32 ? vec_setup<float>(h) : vec_setup<double>(h);
+    if (vs != BA_OK) return vs;
+  }
+  if (fn && !h->mf && h->fa && !h->Jpm) CU(h->alloc(&h->Jpm, (size_t)NPLANE * h->O * h->tsize));
   h->xch = fn;
   h->xctx = ctx;
   h->xbuf = xbuf;
@@ -1742,7 +1769,8 @@ ba_status ba_set_exchange(ba_problem* h, ba_exchange_fn fn, void* ctx, double* x
 
 ba_status ba_get_layout(const ba_problem* h, int64_t* out, int n) {
   if (!h || !out || n < 0) return fail(BA_ERR_INVALID_ARG, "bad argument");
-  const int64_t v[BA_LAYOUT_COUNT] = {h->npieces, h->nchunks, h->fa ? 1 : 0, h->mf ? 0 : 1, h->nlong};
+  const int64_t v[BA_LAYOUT_COUNT] = {h->npieces, h->nchunks, h->fa ? 1 : 0, h->mf ? 0 : 1, h->nlong,
+                                      h->sx.pcg ? 1 : h->sx.direct ? 2 : 0};
   for (int i = 0; i < n; ++i) out[i] = i < BA_LAYOUT_COUNT ? v[i] : 0;
   return BA_OK;
 }

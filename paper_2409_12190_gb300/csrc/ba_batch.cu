@@ -405,7 +405,7 @@ ba_status ba_batch_create(ba_batch** out, int nprob, const int32_t* cam_counts, 
       e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e == cudaSuccess) st = problem_create(&b->h, C, P, O, cams, points, gci, gpi, pixels, opt, stream, true);
+    if (e == cudaSuccess) st = problem_create(&b->h, C, P, O, cams, points, gci, gpi, pixels, opt, stream, true, false);
     else st = set_error(e == cudaErrorMemoryAllocation ? BA_ERR_OOM : BA_ERR_CUDA, "batch set-up failed: %s",
                         cudaGetErrorString(e));
     cudaFree(gci);

@@ -14,10 +14,11 @@
 struct ba_problem;
 
 namespace ba {
-// ba_problem_create; batched: the concatenated problems of a batch.
+// ba_problem_create; batched: the concatenated problems of a batch; may_form:
+// the reduced system may be formed (ba_schur.cu).
 ba_status problem_create(ba_problem** out, int C, int P, int O, const void* cams, const void* points,
                          const int32_t* cam_idx, const int32_t* pt_idx, const void* pixels, const ba_options* opt,
-                         void* stream, bool batched);
+                         void* stream, bool batched, bool may_form);
 // The pairs of observations of each point, sorted by camera pair (device, n
 // each: camera-major slots of both, the point; freed with the object unless
 // kept), and where each camera pair begins.  n stays 0 above `most` pairs or
@@ -39,6 +40,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq);
 void schur_form(ba_problem* h);                                 // the pairs' partial blocks
 void schur_to_band(ba_problem* h, const double* lam_ptr);       // into the band tiles
 void schur_pcg(ba_problem* h, int maxiter, double tol);         // panels, then the PCG (S_ii, M and r given)
+void schur_drop(ba_problem* h);                                 // back to the implicit product (h->s idle)
 }  // namespace ba
 
 struct ba_problem {
@@ -140,11 +142,13 @@ struct ba_problem {
     int4* parts = nullptr;
     unsigned long long* gx = nullptr;
   } sx;
+  std::vector<void*> sx_allocs;  // its memory
   // the PCG's vector work in one launch (ba_vec.cuh) where its blocks fit the GPU
   unsigned long long* vec_gx = nullptr;  // exchange slots, then the error flag
   double* vec_scal = nullptr;            // [4]
   unsigned int wait_polls = 1u << 21;    // of the PCG's grid-wide waits (ba_set_wait_limit)
   bool batched = false;  // the concatenated problems of a batch: never solved as one
+  bool may_form = true;  // the reduced system may be formed
   ba::DevState* st = nullptr;
   ba_iter_stats* stats = nullptr;
   int cap = 0;
@@ -188,6 +192,7 @@ struct ba_problem {
     if (twin) ba_problem_destroy(twin);
     if (gexec) cudaGraphExecDestroy(gexec);
     for (void* v : allocs) cudaFree(v);
+    for (void* v : sx_allocs) cudaFree(v);
     if (ev_in) cudaEventDestroy(ev_in);
     if (ev_out) cudaEventDestroy(ev_out);
     if (s) cudaStreamDestroy(s);

@@ -210,7 +210,7 @@ ba_status schur_pairs(ba_problem* h, const std::vector<int32_t>& rq, bool self, 
 ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   const bool direct = h->opt.solver == BA_SOLVER_CHOLESKY;
   const bool f32 = h->prec == BA_PREC_F32;
-  if (h->batched) return BA_OK;
+  if (h->batched || !h->may_form) return BA_OK;
   const int C = h->C, O = h->O;
   const SchurCost cost{f32, h->opt.pcg_maxiter};
   int dev = 0, nsm = 0, coop = 0;
@@ -285,8 +285,9 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
       all += al(i.bytes);
     }
     char* base = nullptr;
-    e = h->alloc(&base, all);
+    e = cudaMalloc(&base, all);
     if (e != cudaSuccess) return;
+    h->sx_allocs.push_back(base);
     std::vector<char> host(copied);
     size_t at = 0, free_at = copied;  // the copied ones first
     for (const Item& i : items) {
@@ -302,7 +303,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
     x.pk = pr.pk;
     x.pl = pr.pl;
     x.pj = pr.pj;
-    pr.keep(h->allocs);
+    pr.keep(h->sx_allocs);
   };
   auto kernel_attr = [&](const void* k, int bytes) {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
@@ -327,6 +328,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
     unmark();
     if (e != cudaSuccess) {
       cudaGetLastError();
+      schur_drop(h);
       return BA_OK;
     }
     keep();
@@ -395,14 +397,20 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
     pptr.push_back((int32_t)parts.size());
     fits = x.nc_max < 65536 && sx_smem(x.nc_max, x.parts_max) <= 200u * 1024u;
   }
-  if (!fits) return BA_OK;
+  if (!fits) {
+    x = {};
+    return BA_OK;
+  }
   if (parts.empty()) parts.push_back(make_int4(0, 0, 0, 0));
   const size_t smem = sx_smem(x.nc_max, x.parts_max);
   const void* kern = f32 ? (const void*)k_schur_pcg<float> : (const void*)k_schur_pcg<double>;
   int occ = 0;
   SCU(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   SCU(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, SX_THREADS, smem));
-  if ((long long)occ * nsm < groups) return BA_OK;
+  if ((long long)occ * nsm < groups) {
+    x = {};
+    return BA_OK;
+  }
   x.words = sx_words(groups, C) + 1;  // and the error flag
   up(&x.blk_pos, pos);
   up(&x.rowblk, rowblk);
@@ -420,6 +428,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   if (e == cudaSuccess && !h->Sii) e = h->alloc(&h->Sii, 45ull * C * 8);
   if (e != cudaSuccess) {
     cudaGetLastError();
+    schur_drop(h);
     return BA_OK;
   }
   keep();
@@ -478,6 +487,12 @@ void pcg(ba_problem* h, int maxiter, double tol) {
 }
 
 }  // namespace
+
+void schur_drop(ba_problem* h) {
+  for (void* v : h->sx_allocs) cudaFree(v);
+  h->sx_allocs.clear();
+  h->sx = {};
+}
 
 void schur_form(ba_problem* h) {
   const bool f32 = h->prec == BA_PREC_F32;

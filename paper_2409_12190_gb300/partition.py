@@ -61,6 +61,10 @@ def part_arrays(cams, points, cam_idx, pt_idx, pixels, bounds, r: int):
             (pt_idx[obs] - lo).astype(np.int32), np.asarray(pixels)[obs], obs)
 
 
+class _Part(Problem):
+    _create = "ba_problem_create_part"
+
+
 class PartProblem:
     """One part of a point-partitioned problem: a ``Problem`` on the part's
     arrays whose exchanges call ``allreduce(t)``, which must sum the 1-D
@@ -69,7 +73,7 @@ class PartProblem:
 
     def __init__(self, cams, points, cam_idx, pt_idx, pixels, allreduce, options: Options | None = None,
                  device="cuda"):
-        self.problem = Problem(cams, points, cam_idx, pt_idx, pixels, options, device=device)
+        self.problem = _Part(cams, points, cam_idx, pt_idx, pixels, options, device=device)
         self.device = self.problem.device
         self._allreduce = allreduce
         self.xbuf = torch.zeros(exchange_cap(self.problem.C), dtype=torch.float64, device=self.device)

@@ -5,7 +5,10 @@ import pytest
 import torch
 
 import oracle as orc
+import paper_2409_12190_gb300 as ba
 from gpu_helpers import np64, problem, rel_err, small_ring
+from paper_2409_12190_gb300 import _lib
+from paper_2409_12190_gb300.partition import PartProblem, exchange_cap
 
 pytestmark = pytest.mark.gpu
 
@@ -24,3 +27,51 @@ def test_product_keeps_its_long_pieces(C, P):
         assert lay["product_pieces"] == np.sum(-(-per_cam // 2048)) < lay["pieces"]
         y = prob.schur_matvec(1e-3, x.cuda())
         assert rel_err(np64(y), np64(ref.schur_matvec(1e-3, x.cuda()))) < 1e-11
+
+
+def _one_part(C=97, P=9000):
+    sc = small_ring(C, P, seed=3)
+    pix = orc.pixels_from_scene(sc)
+    opts = ba.Options(precision="f64", pcg_maxiter=40, pcg_tol=0.0, huber_delta=sc.huber_delta)
+    return sc, (sc.cams_init, sc.points_init, sc.cam_idx, sc.pt_idx, pix), opts
+
+
+def test_a_part_holds_no_formed_system():
+    """Made as a part, or made alone and then given an exchange: the implicit
+    product, and the same trials (a sum over one part changes nothing).  Alone
+    again: trials to rounding of those of the formed system (1e-9)."""
+    sc, arrays, opts = _one_part()
+    with ba.Problem(*arrays, opts, device="cuda") as alone:
+        assert alone.layout()["formed"] == 1
+        alone.solve(3)
+        want = alone.stats()
+    with PartProblem(*arrays, lambda t: None, opts, device="cuda") as part:
+        lay = part.layout()
+        assert lay["formed"] == 0 and lay["pieces"] == lay["product_pieces"]
+        part.solve(3)
+        a = part.stats()
+        pa = [t.cpu() for t in part.params()]
+    prob = ba.Problem(*arrays, opts, device="cuda")
+    prob.solve(1)  # captured with the formed system
+    xbuf = torch.zeros(exchange_cap(sc.C), dtype=torch.float64, device="cuda")
+    fn = _lib.EXCHANGE_FN(lambda n, stream, ctx: 0)
+    _lib.check(_lib.load().ba_set_exchange(prob._h, fn, None, xbuf.data_ptr(), xbuf.numel()))
+    assert prob.layout()["formed"] == 0
+    prob.set_params(torch.from_numpy(sc.cams_init), torch.from_numpy(sc.points_init))
+    prob.set_lambda(opts.lambda0)
+    prob.solve(3)
+    b = prob.stats()[-3:]
+    pb = [t.cpu() for t in prob.params()]
+    _lib.check(_lib.load().ba_set_exchange(prob._h, _lib.EXCHANGE_FN(), None, None, 0))
+    prob.set_params(torch.from_numpy(sc.cams_init), torch.from_numpy(sc.points_init))
+    prob.set_lambda(opts.lambda0)
+    prob.solve(3)
+    c = prob.stats()[-3:]
+    prob.close()
+    for got in (a, b, c):
+        assert [s["pcg_iters"] for s in got] == [s["pcg_iters"] for s in want]
+        assert [s["accepted"] for s in got] == [s["accepted"] for s in want]
+        for s, w in zip(got, want):
+            assert abs(s["cost_trial"] - w["cost_trial"]) < 1e-9 * w["cost_trial"]
+    for x, y in zip(pa, pb):
+        assert rel_err(x.numpy(), y.numpy()) < 1e-9
