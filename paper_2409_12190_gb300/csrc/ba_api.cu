@@ -1216,8 +1216,14 @@ ba_status ba::problem_create(ba_problem** out, int C, int P, int O, const void* 
   }
   if (st != BA_OK) {
     std::string msg = g_err;
+    const bool formed = h->sx.pcg || h->sx.direct;
     cudaStreamSynchronize(h->s);
     delete h;
+    // the formed system took what something else needed: without it
+    if (st == BA_ERR_OOM && formed) {
+      cudaGetLastError();
+      return problem_create(out, C, P, O, cams, points, cam_idx, pt_idx, pixels, opt, stream, batched, false);
+    }
     g_err = msg;
     return st;
   }

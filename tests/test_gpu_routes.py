@@ -75,3 +75,59 @@ def test_a_part_holds_no_formed_system():
             assert abs(s["cost_trial"] - w["cost_trial"]) < 1e-9 * w["cost_trial"]
     for x, y in zip(pa, pb):
         assert rel_err(x.numpy(), y.numpy()) < 1e-9
+
+
+def _large_ring(C, P, views, seed):
+    """Points seen by `views` neighbouring cameras of a ring, on the GPU."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    f = dict(dtype=torch.float64, device="cuda")
+    cams = torch.zeros(C, 9, **f)
+    cams[:, 1] = -2 * np.pi * torch.arange(C, **f) / C
+    cams[:, 5], cams[:, 6] = -5.0, 500.0
+    pts = 2 * torch.rand(P, 3, generator=g, **f) - 1
+    pi = torch.arange(P, device="cuda").repeat_interleave(views)
+    ci = (torch.randint(0, C, (P,), generator=g, device="cuda")[:, None] + torch.arange(views, device="cuda")) % C
+    ci, pi = ci.reshape(-1).int(), pi.int()
+    pix = ba.project(cams, pts, ci, pi)
+    pix = pix + torch.randn(pix.shape, generator=g, **f)
+    return cams, pts + 0.01 * torch.randn(P, 3, generator=g, **f), ci, pi, pix
+
+
+def test_a_problem_that_fits_only_unformed_is_made():
+    """Memory for the problem with the implicit product, but not for the pairs
+    and the lean form that the formed system has instead of the point-major
+    planes: made without it."""
+    arrays = _large_ring(250, 300000, 12, seed=1)
+    opts = ba.Options(precision="f64", pcg_maxiter=30, pcg_tol=0.0)
+
+    class Part(ba.Problem):
+        _create = "ba_problem_create_part"
+
+    def run(make):
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        with make(*arrays, opts, device="cuda") as prob:
+            took = free - torch.cuda.mem_get_info()[0]
+            formed = prob.layout()["formed"]
+            prob.solve(1)
+            out = [t.clone() for t in prob.params()]
+        torch.cuda.synchronize()
+        return took, formed, out
+
+    for make in (Part, ba.Problem):
+        run(make)  # loads what it needs
+    torch.cuda.empty_cache()
+    plain, formed_0, want = run(Part)
+    formed, formed_1, _ = run(ba.Problem)
+    assert (formed_0, formed_1) == (0, 1) and formed - plain > 64 << 20
+    torch.cuda.empty_cache()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - (plain + formed) // 2, dtype=torch.uint8, device="cuda")
+    try:
+        with ba.Problem(*arrays, opts, device="cuda") as prob:
+            assert prob.layout()["formed"] == 0
+            prob.solve(1)
+            got = prob.params()
+        assert all(torch.equal(a, b) for a, b in zip(got, want))
+    finally:
+        del filler
+        torch.cuda.empty_cache()
