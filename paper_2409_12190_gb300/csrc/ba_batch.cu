@@ -305,6 +305,23 @@ int occupancy(const ba_batch* b, int variant) {
   return std::max(1, n);
 }
 
+// Two CTAs an SM (variant 1, half of the registers each) or one.  With the
+// systems formed one: the 81 sums of a block spill with half of them (512
+// windows 5.4 against 6.0 ms).  Otherwise two delay the largest window, which
+// bounds the batch unless every SM has that much to do, so the line is the
+// batch's observations an SM over the largest window's.  Time with two over that
+// with one, windows of 200-3,000, 60-500 and 1,000 points:
+//   stored planes, FP32   1.05 at 0.65, 0.98 at 0.79, 0.84 at 1.0, 0.70 at 1.7 and above
+//   stored planes, FP64   1.20 at 0.65, 1.04 at 0.92, 0.93-1.0 at 1.0, 0.87 at 1.7
+//   recomputed, FP64      1.42 at 0.65, 1.18 at 1.0, 1.01 at 1.26, 0.95 at 1.7
+int default_variant(const ba_batch* b) {
+  if (b->sx_val || b->nprob <= b->nsm || occupancy(b, 1) < 2) return 0;
+  int largest = 1;
+  for (int i = 0; i < b->nprob; ++i) largest = std::max(largest, b->obs_off[i + 1] - b->obs_off[i]);
+  const double fill = (double)b->obs_off[b->nprob] / ((double)largest * b->nsm);
+  return fill >= (b->h->prec == BA_PREC_F32 ? 0.8 : b->h->mf ? 1.3 : 1.0) ? 1 : 0;
+}
+
 template <typename T, bool MF>
 cudaError_t set_smem_attr(size_t bytes) {
   cudaError_t e = cudaFuncSetAttribute(k_batch_lm<T, MF, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
@@ -478,11 +495,7 @@ ba_status ba_batch_create(ba_batch** out, int nprob, const int32_t* cam_counts, 
   if (e == cudaSuccess) e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&b->nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return fail_out(BA_ERR_CUDA, "kernel attribute set-up failed");
-  // With the systems formed one CTA an SM with all of the registers (512
-  // windows 5.4 ms, two with half of them 6.0: the 81 sums of a block spill).
-  // Otherwise two CTAs an SM where there are problems for both (8.9 against
-  // 6.9 ms); with fewer problems than SMs one (8.9 against 9.8 ms).
-  b->variant = !b->sx_val && b->nprob > b->nsm && occupancy(b, 1) >= 2 ? 1 : 0;
+  b->variant = default_variant(b);
   b->ctas_per_sm = occupancy(b, b->variant);
   b->order = 0;
   st = upload_order(b);
