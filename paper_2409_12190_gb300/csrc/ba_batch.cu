@@ -215,7 +215,7 @@ ba_status form_setup(ba_batch* b, const std::vector<int32_t>& rq) {
                               q + 1 < pr.head.size() ? pr.head[q + 1] : pr.n));
     off.push_back((int32_t)blk.size());
     voff.push_back(vals);
-    vals += ((long long)9 * (c1 - c0) * sx_ld(c1 - c0) + 3) / 4 * 4;
+    vals += 2LL * 9 * (c1 - c0) * sx_ld(c1 - c0);
   }
   cudaError_t e = b->alloc(&b->sx_off, off.size() * 4);
   if (e == cudaSuccess) e = b->alloc(&b->sx_blk, blk.size() * sizeof(int4));
@@ -226,7 +226,7 @@ ba_status form_setup(ba_batch* b, const std::vector<int32_t>& rq) {
   void* val = nullptr;
   if (e == cudaSuccess) e = b->alloc(&val, vals * 4);
   // blocks of cameras without a common point stay zero
-  if (e == cudaSuccess) e = cudaMemset(val, 0, vals * 4);
+  if (e == cudaSuccess) e = cudaMemsetAsync(val, 0, vals * 4, h->s);
   if (e != cudaSuccess) {
     cudaGetLastError();  // no room: the implicit product
     return BA_OK;
@@ -307,7 +307,7 @@ int occupancy(const ba_batch* b, int variant) {
 
 // Two CTAs an SM (variant 1, half of the registers each) or one.  With the
 // systems formed one: the 81 sums of a block spill with half of them (512
-// windows 5.4 against 6.0 ms).  Otherwise two delay the largest window, which
+// windows 5.8 against 7.0 ms).  Otherwise two delay the largest window, which
 // bounds the batch unless every SM has that much to do, so the line is the
 // batch's observations an SM over the largest window's.  Time with two over that
 // with one, windows of 200-3,000, 60-500 and 1,000 points:

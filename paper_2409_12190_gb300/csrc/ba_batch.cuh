@@ -86,7 +86,8 @@ struct BatchArgs {
   // the reduced system of each problem formed explicitly (FP32 recompute
   // mode), or NULL: the camera-pair blocks (local cameras, entries e0 .. e1 of
   // the sorted pairs) of each problem, and its dense matrix without the
-  // diagonal blocks, rows of sx_ld(nc)
+  // diagonal blocks, rows of sx_ld(nc), the upper then the lower halves of
+  // float-float entries
   const int32_t* sx_off;  // [nprob + 1]
   const int4* sx_blk;
   const int32_t *sx_pk, *sx_pl, *sx_pj;
@@ -409,16 +410,28 @@ __device__ __forceinline__ void batch_stage_fxv(BShared<T>& S, const BRange<T>& 
 // Row stride of a formed system of nc cameras.
 __host__ __device__ constexpr int sx_ld(int nc) { return (9 * nc + 3) / 4 * 4; }
 
-// Warp reduce-scatter of 81 floats (padded to 96): lane l returns the totals
-// of values 3 l .. 3 l + 2.
-template <int N, int OFF>
-__device__ __forceinline__ void sx_rs96_step(float (&h)[48], int lane) {
-  const bool up = (lane & OFF) != 0;
+// Entries that a lane's plain FP32 sums of a block run over before they are
+// added up in float-float, times the lanes.
+constexpr int SX_RUN = 1024;
+
+// Warp reduce-scatter of 81 floats (padded to 96) in float-float: lane l
+// returns the totals of values 3 l .. 3 l + 2.
+__device__ __forceinline__ void sx_rs81_ff(const float (&v)[SX_PART], float (&h3)[3], float (&l3)[3], int lane) {
+  float h[48], l[48];
+  const bool up = (lane & 16) != 0;
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    const float k = up ? h[N + i] : h[i];
-    const float g = up ? h[i] : h[N + i];
-    h[i] = k + __shfl_xor_sync(0xffffffffu, g, OFF);
+  for (int i = 0; i < 48; ++i) {
+    const float lo = v[i], hi = 48 + i < SX_PART ? v[48 + i < SX_PART ? 48 + i : 0] : 0.f;
+    two_sum(up ? hi : lo, __shfl_xor_sync(0xffffffffu, up ? lo : hi, 16), h[i], l[i]);
+  }
+  rs_ff_step<24, 8>(h, l, lane);
+  rs_ff_step<12, 4>(h, l, lane);
+  rs_ff_step<6, 2>(h, l, lane);
+  rs_ff_step<3, 1>(h, l, lane);
+#pragma unroll
+  for (int u = 0; u < 3; ++u) {
+    h3[u] = h[u];
+    l3[u] = l[u];
   }
 }
 
@@ -427,13 +440,19 @@ __device__ __forceinline__ void sx_rs96_step(float (&h)[48], int lane) {
 // pair a lane (the arithmetic of k_schur_form).  The largest of 512 windows
 // (20 cameras, 20,900 observations) alone in its CTA took 1.8 ms a trial of ten
 // implicit iterations; a pair costs about what one observation of one
-// iteration does, and an iteration on the formed S reads 130 KB from L2.  The
+// iteration does, and an iteration on the formed S reads 260 KB from L2.  The
 // warps take the blocks from a counter.
+// Each entry is kept as a float-float pair (hi, then lo, each rows of sx_ld(nc)):
+// lanes add in FP32, what is added across lanes and runs is float-float.  Rounded
+// to FP32 and with plain sums the cameras of 512 windows were 4.3e-7 from the
+// 64-bit answer instead of the implicit product's 1.8e-7, now 2.0e-7 (512 windows
+// 8.9 ms with the implicit product, 5.4 with FP32 entries, 5.8 now).
 template <typename T>
 __device__ __noinline__ void batch_form(const BatchArgs<T>& a, const BRange<T>& R, BShared<T>& S, int b) {
   const int lane = threadIdx.x & 31;
   const int ld = sx_ld(R.nc);
   T* val = a.sx_val + a.sx_val_off[b];
+  T* val_lo = val + 9 * R.nc * ld;
   for (;;) {
     // the next block of the problem (each is summed by one warp whichever it is)
     int q = 0;
@@ -441,112 +460,139 @@ __device__ __noinline__ void batch_form(const BatchArgs<T>& a, const BRange<T>& 
     q = __shfl_sync(0xffffffffu, q, 0);
     if (q >= a.sx_off[b + 1]) break;
     const int4 blk = a.sx_blk[q];
-    T acc[SX_PART];
+    float H[3] = {0.f, 0.f, 0.f}, L[3] = {0.f, 0.f, 0.f};
+    for (int run = blk.z; run < blk.w; run += SX_RUN) {
+      T acc[SX_PART];
 #pragma unroll
-    for (int i = 0; i < SX_PART; ++i) acc[i] = T(0);
-    for (int e = blk.z + lane; e < blk.w; e += 32) {
-      const int j = a.sx_pj[e];
-      const int k = a.cm_sw ? a.sx_pk[e] : 0, l = a.cm_sw ? a.sx_pl[e] : 0;
-      T X0, X1, X2, pad;
-      load4(a.ptab + 8LL * j, X0, X1, X2, pad);
-      const T* vi = a.Vinv + 6LL * j;
-      const T v00 = vi[0], v01 = vi[1], v02 = vi[2], v11 = vi[3], v12 = vi[4], v22 = vi[5];
-      SfObs<T, true> u, w;
-      u.open(nullptr, 0, k, S.ct[blk.x], X0, X1, X2, a.cm_sw);
-      w.open(nullptr, 0, l, S.ct[blk.y], X0, X1, X2, a.cm_sw);
-      T K[4];
+      for (int i = 0; i < SX_PART; ++i) acc[i] = T(0);
+      for (int e = run + lane; e < min(blk.w, run + SX_RUN); e += 32) {
+        const int j = a.sx_pj[e];
+        const int k = a.cm_sw ? a.sx_pk[e] : 0, l = a.cm_sw ? a.sx_pl[e] : 0;
+        T X0, X1, X2, pad;
+        load4(a.ptab + 8LL * j, X0, X1, X2, pad);
+        const T* vi = a.Vinv + 6LL * j;
+        const T v00 = vi[0], v01 = vi[1], v02 = vi[2], v11 = vi[3], v12 = vi[4], v22 = vi[5];
+        SfObs<T, true> u, w;
+        u.open(nullptr, 0, k, S.ct[blk.x], X0, X1, X2, a.cm_sw);
+        w.open(nullptr, 0, l, S.ct[blk.y], X0, X1, X2, a.cm_sw);
+        T K[4];
 #pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const T* p = u.pl + NPLANE_JC + 3 * r;
-        const T t0 = p[0] * v00 + p[1] * v01 + p[2] * v02;
-        const T t1 = p[0] * v01 + p[1] * v11 + p[2] * v12;
-        const T t2 = p[0] * v02 + p[1] * v12 + p[2] * v22;
+        for (int r = 0; r < 2; ++r) {
+          const T* p = u.pl + NPLANE_JC + 3 * r;
+          const T t0 = p[0] * v00 + p[1] * v01 + p[2] * v02;
+          const T t1 = p[0] * v01 + p[1] * v11 + p[2] * v12;
+          const T t2 = p[0] * v02 + p[1] * v12 + p[2] * v22;
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const T* z = w.pl + NPLANE_JC + 3 * c;
-          K[2 * r + c] = t0 * z[0] + t1 * z[1] + t2 * z[2];
+          for (int c = 0; c < 2; ++c) {
+            const T* z = w.pl + NPLANE_JC + 3 * c;
+            K[2 * r + c] = t0 * z[0] + t1 * z[1] + t2 * z[2];
+          }
+        }
+        T k0[9], k1[9], l0[9], l1[9];
+        jc_rows(u.pl, k0, k1);
+        jc_rows(w.pl, l0, l1);
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+          const T g0 = K[0] * l0[c] + K[1] * l1[c], g1 = K[2] * l0[c] + K[3] * l1[c];
+#pragma unroll
+          for (int r = 0; r < 9; ++r) acc[9 * r + c] += k0[r] * g0 + k1[r] * g1;
         }
       }
-      T k0[9], k1[9], l0[9], l1[9];
-      jc_rows(u.pl, k0, k1);
-      jc_rows(w.pl, l0, l1);
+      float h[3], l[3];
+      sx_rs81_ff(acc, h, l, lane);
 #pragma unroll
-      for (int c = 0; c < 9; ++c) {
-        const T g0 = K[0] * l0[c] + K[1] * l1[c], g1 = K[2] * l0[c] + K[3] * l1[c];
-#pragma unroll
-        for (int r = 0; r < 9; ++r) acc[9 * r + c] += k0[r] * g0 + k1[r] * g1;
-      }
+      for (int u = 0; u < 3; ++u) ff_add(H[u], L[u], h[u], l[u]);
     }
-    float h[48];
-    {
-      const bool up = (lane & 16) != 0;
-#pragma unroll
-      for (int i = 0; i < 48; ++i) {
-        const float lo = acc[i], hi = 48 + i < SX_PART ? acc[48 + i < SX_PART ? 48 + i : 0] : 0.f;
-        h[i] = (up ? hi : lo) + __shfl_xor_sync(0xffffffffu, up ? lo : hi, 16);
-      }
-    }
-    sx_rs96_step<24, 8>(h, lane);
-    sx_rs96_step<12, 4>(h, lane);
-    sx_rs96_step<6, 2>(h, lane);
-    sx_rs96_step<3, 1>(h, lane);
     if (blk.x == blk.y) {
       // a camera that observes a point twice: with the transpose
+      float h[3], l[3];
 #pragma unroll
       for (int u = 0; u < 3; ++u) {
         const int v = 3 * lane + u, t = 9 * (v % 9) + v / 9, src = min(t / 3, 31);
-        const float t0 = __shfl_sync(0xffffffffu, h[0], src), t1 = __shfl_sync(0xffffffffu, h[1], src),
-                    t2 = __shfl_sync(0xffffffffu, h[2], src);
-        h[3 + u] = h[u] + (t % 3 == 0 ? t0 : t % 3 == 1 ? t1 : t2);
+        h[u] = l[u] = 0.f;
+#pragma unroll
+        for (int w = 0; w < 3; ++w) {
+          const float th = __shfl_sync(0xffffffffu, H[w], src), tl = __shfl_sync(0xffffffffu, L[w], src);
+          h[u] = t % 3 == w ? th : h[u];
+          l[u] = t % 3 == w ? tl : l[u];
+        }
       }
 #pragma unroll
-      for (int u = 0; u < 3; ++u) h[u] = h[3 + u];
+      for (int u = 0; u < 3; ++u) ff_add(h[u], l[u], H[u], L[u]);
+#pragma unroll
+      for (int u = 0; u < 3; ++u) {
+        H[u] = h[u];
+        L[u] = l[u];
+      }
     }
 #pragma unroll
     for (int u = 0; u < 3; ++u) {
       const int v = 3 * lane + u, r = 9 * blk.x + v / 9, c = 9 * blk.y + v % 9;
       if (v >= SX_PART) continue;
-      val[r * ld + c] = -h[u];
-      if (blk.x != blk.y) val[c * ld + r] = -h[u];
+      val[r * ld + c] = -H[u];
+      val_lo[r * ld + c] = -L[u];
+      if (blk.x != blk.y) {
+        val[c * ld + r] = -H[u];
+        val_lo[c * ld + r] = -L[u];
+      }
     }
   }
 }
 
+// (hi, lo) += (vh, vl) p: the product and the sum with their errors in lo
+// (Ogita, Rump and Oishi's compensated dot product).
+__device__ __forceinline__ void ff_mac(float& hi, float& lo, float vh, float vl, float p) {
+  const float q = vh * p;
+  const float eq = fmaf(vh, p, -q);
+  float es;
+  two_sum(hi, q, hi, es);
+  lo += fmaf(vl, p, eq + es);
+}
+
 // S.ss = (S without its diagonal blocks) pf: a warp takes eight rows at a time,
-// a lane four columns.
+// a lane up to eight columns, compensated; the lanes' sums are added in
+// float-float, a reduce-scatter over the rows.
 template <typename T>
 __device__ __forceinline__ void batch_formed_product(const BatchArgs<T>& a, const BRange<T>& R, BShared<T>& S, int b) {
   constexpr int RB = 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n = 9 * R.nc, l4 = sx_ld(R.nc) / 4;
   const float4* val = reinterpret_cast<const float4*>(a.sx_val + a.sx_val_off[b]);
+  const float4* val_lo = val + n * l4;
   const float4* pf = reinterpret_cast<const float4*>(S.pf);
   for (int r0 = RB * warp; r0 < n; r0 += RB * (BT / 32)) {
-    float acc[RB];
+    float h[RB], l[RB];
 #pragma unroll
-    for (int r = 0; r < RB; ++r) acc[r] = 0.f;
+    for (int r = 0; r < RB; ++r) h[r] = l[r] = 0.f;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
       const int c = lane + 32 * u;
       if (c >= l4) continue;
-      float4 v[RB];
+      float4 v[RB], w[RB];
 #pragma unroll
-      for (int r = 0; r < RB; ++r) v[r] = val[min(r0 + r, n - 1) * l4 + c];
+      for (int r = 0; r < RB; ++r) {
+        v[r] = val[min(r0 + r, n - 1) * l4 + c];
+        w[r] = val_lo[min(r0 + r, n - 1) * l4 + c];
+      }
       const float4 p = pf[c];
 #pragma unroll
-      for (int r = 0; r < RB; ++r) acc[r] += (v[r].x * p.x + v[r].y * p.y) + (v[r].z * p.z + v[r].w * p.w);
+      for (int r = 0; r < RB; ++r) {
+        ff_mac(h[r], l[r], v[r].x, w[r].x, p.x);
+        ff_mac(h[r], l[r], v[r].y, w[r].y, p.y);
+        ff_mac(h[r], l[r], v[r].z, w[r].z, p.z);
+        ff_mac(h[r], l[r], v[r].w, w[r].w, p.w);
+      }
     }
+    rs_ff_step<4, 16>(h, l, lane);
+    rs_ff_step<2, 8>(h, l, lane);
+    rs_ff_step<1, 4>(h, l, lane);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      float t[RB];
-#pragma unroll
-      for (int r = 0; r < RB; ++r) t[r] = __shfl_xor_sync(0xffffffffu, acc[r], off);
-#pragma unroll
-      for (int r = 0; r < RB; ++r) acc[r] += t[r];
+    for (int off = 2; off > 0; off >>= 1) {
+      const float gh = __shfl_xor_sync(0xffffffffu, h[0], off), gl = __shfl_xor_sync(0xffffffffu, l[0], off);
+      ff_add(h[0], l[0], gh, gl);
     }
-#pragma unroll
-    for (int r = 0; r < RB; ++r)
-      if (lane == r && r0 + r < n) S.ss[r0 + r] = (double)acc[r];
+    const int r = r0 + (lane >> 2);  // row lane / 4 of the eight
+    if (!(lane & 3) && r < n) S.ss[r] = (double)h[0] + (double)l[0];
   }
 }
 static_assert(sx_ld(BMAXC) <= 256, "a row of the formed system is two rounds of a warp's four-vectors");

@@ -171,8 +171,8 @@ __device__ __forceinline__ void ff_rcp(float bh, float bl, float& hi, float& lo)
 // of values 2l and 2l + 1 (after the step of offset o a lane keeps the upper
 // half iff its lane bit o is set, so the kept block starts at 2l).  The order
 // of the additions depends on the lane numbers only.
-template <int N, int OFF>
-__device__ __forceinline__ void rs_ff_step(float (&h)[32], float (&l)[32], int lane) {
+template <int N, int OFF, int M>
+__device__ __forceinline__ void rs_ff_step(float (&h)[M], float (&l)[M], int lane) {
   const bool up = (lane & OFF) != 0;
 #pragma unroll
   for (int i = 0; i < N; ++i) {

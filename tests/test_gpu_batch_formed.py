@@ -33,3 +33,27 @@ def test_point_observed_twice_by_a_camera(C, huber):
         assert drop > 0 and a["pcg_iters"] == b["pcg_iters"] == 10
         assert abs(a["cost_trial"] - b["cost_trial"]) < 1e-4 * drop
         assert abs(a["model"] - b["model"]) < 1e-4 * abs(b["model"])
+
+
+def test_formed_systems_are_as_accurate_as_the_implicit_product():
+    """Three trials of 48 windows from FP32-rounded inputs: the cameras'
+    distance from the FP64 batch, formed (recomputed Jacobians) against the
+    implicit product (stored ones).  Both round per observation; what the formed
+    system adds must stay below that: 1.5 times, over all windows."""
+    rng = np.random.default_rng(5)
+    inputs = []
+    for k in range(48):
+        C = int(rng.integers(5, 21))
+        sc = scenegen.arc_scene(C, int(rng.integers(200, 900)), seed=100 + k, views_lo=4, views_hi=min(C, 10))
+        pix = orc.pixels_from_scene(sc)
+        inputs.append([np.asarray(a, np.float32) for a in (sc.cams_init, sc.points_init)] + [sc.cam_idx, sc.pt_idx]
+                      + [np.asarray(pix, np.float32)])
+    cams = {}
+    for precision, jacobian in (("f64", "store"), ("f32", "store"), ("f32", "recompute")):
+        opts = ba.Options(precision=precision, jacobian=jacobian, pcg_maxiter=10, pcg_tol=0.0)
+        with ba.Batch(inputs, opts) as batch:
+            batch.solve(3)
+            cams[precision, jacobian] = batch.params(split=False)[0].cpu().double().numpy()
+    exact = cams["f64", "store"]
+    err = {j: np.linalg.norm(cams["f32", j] - exact) / np.linalg.norm(exact) for j in ("store", "recompute")}
+    assert err["recompute"] < 1.5 * err["store"], err
