@@ -424,10 +424,10 @@ __device__ __forceinline__ void sx_rs81_ff(const float (&v)[SX_PART], float (&h3
     const float lo = v[i], hi = 48 + i < SX_PART ? v[48 + i < SX_PART ? 48 + i : 0] : 0.f;
     two_sum(up ? hi : lo, __shfl_xor_sync(0xffffffffu, up ? lo : hi, 16), h[i], l[i]);
   }
-  rs_ff_step<24, 8>(h, l, lane);
-  rs_ff_step<12, 4>(h, l, lane);
-  rs_ff_step<6, 2>(h, l, lane);
-  rs_ff_step<3, 1>(h, l, lane);
+  rs_pair_step<24, 8>(h, l, lane);
+  rs_pair_step<12, 4>(h, l, lane);
+  rs_pair_step<6, 2>(h, l, lane);
+  rs_pair_step<3, 1>(h, l, lane);
 #pragma unroll
   for (int u = 0; u < 3; ++u) {
     h3[u] = h[u];
@@ -539,16 +539,6 @@ __device__ __noinline__ void batch_form(const BatchArgs<T>& a, const BRange<T>& 
   }
 }
 
-// (hi, lo) += (vh, vl) p: the product and the sum with their errors in lo
-// (Ogita, Rump and Oishi's compensated dot product).
-__device__ __forceinline__ void ff_mac(float& hi, float& lo, float vh, float vl, float p) {
-  const float q = vh * p;
-  const float eq = fmaf(vh, p, -q);
-  float es;
-  two_sum(hi, q, hi, es);
-  lo += fmaf(vl, p, eq + es);
-}
-
 // S.ss = (S without its diagonal blocks) pf: a warp takes eight rows at a time,
 // a lane up to eight columns, compensated; the lanes' sums are added in
 // float-float, a reduce-scatter over the rows.
@@ -583,13 +573,15 @@ __device__ __forceinline__ void batch_formed_product(const BatchArgs<T>& a, cons
         ff_mac(h[r], l[r], v[r].w, w[r].w, p.w);
       }
     }
-    rs_ff_step<4, 16>(h, l, lane);
-    rs_ff_step<2, 8>(h, l, lane);
-    rs_ff_step<1, 4>(h, l, lane);
+    rs_pair_step<4, 16>(h, l, lane);
+    rs_pair_step<2, 8>(h, l, lane);
+    rs_pair_step<1, 4>(h, l, lane);
 #pragma unroll
     for (int off = 2; off > 0; off >>= 1) {
       const float gh = __shfl_xor_sync(0xffffffffu, h[0], off), gl = __shfl_xor_sync(0xffffffffu, l[0], off);
-      ff_add(h[0], l[0], gh, gl);
+      float e;
+      two_sum(h[0], gh, h[0], e);
+      l[0] = (l[0] + gl) + e;
     }
     const int r = r0 + (lane >> 2);  // row lane / 4 of the eight
     if (!(lane & 3) && r < n) S.ss[r] = (double)h[0] + (double)l[0];

@@ -142,6 +142,16 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float h2, float l2)
   lo = e - (hi - s);
 }
 
+// (hi, lo) += (vh, vl) p: the product and the sum with their errors in lo
+// (Ogita, Rump and Oishi's compensated dot product).
+__device__ __forceinline__ void ff_mac(float& hi, float& lo, float vh, float vl, float p) {
+  const float q = vh * p;
+  const float eq = fmaf(vh, p, -q);
+  float es;
+  two_sum(hi, q, hi, es);
+  lo += fmaf(vl, p, eq + es);
+}
+
 // Float-float products (Dekker's product with the exact FMA remainder):
 // (hi, lo) = (ah, al) * (bh, bl), and the same with a plain float b.
 __device__ __forceinline__ void ff_mul(float ah, float al, float bh, float bl, float& hi, float& lo) {
@@ -171,8 +181,8 @@ __device__ __forceinline__ void ff_rcp(float bh, float bl, float& hi, float& lo)
 // of values 2l and 2l + 1 (after the step of offset o a lane keeps the upper
 // half iff its lane bit o is set, so the kept block starts at 2l).  The order
 // of the additions depends on the lane numbers only.
-template <int N, int OFF, int M>
-__device__ __forceinline__ void rs_ff_step(float (&h)[M], float (&l)[M], int lane) {
+template <int N, int OFF>
+__device__ __forceinline__ void rs_ff_step(float (&h)[32], float (&l)[32], int lane) {
   const bool up = (lane & OFF) != 0;
 #pragma unroll
   for (int i = 0; i < N; ++i) {
@@ -182,6 +192,21 @@ __device__ __forceinline__ void rs_ff_step(float (&h)[M], float (&l)[M], int lan
     ff_add(kh, kl, rh, rl);
     h[i] = kh;
     l[i] = kl;
+  }
+}
+// The same step for pairs of a float sum and what its additions rounded off:
+// the sums wait for one addition a step, not for the renormalisation.
+template <int N, int OFF, int M>
+__device__ __forceinline__ void rs_pair_step(float (&h)[M], float (&l)[M], int lane) {
+  const bool up = (lane & OFF) != 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const float kh = up ? h[N + i] : h[i], kl = up ? l[N + i] : l[i];
+    const float gh = up ? h[i] : h[N + i], gl = up ? l[i] : l[N + i];
+    const float rh = __shfl_xor_sync(0xffffffffu, gh, OFF), rl = __shfl_xor_sync(0xffffffffu, gl, OFF);
+    float e;
+    two_sum(kh, rh, h[i], e);
+    l[i] = (kl + rl) + e;
   }
 }
 // The same reduce-scatter for 16 plain floats (four steps, 15 shuffles):

@@ -238,7 +238,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   auto& x = h->sx;
   cudaStream_t s = h->s;
   cudaError_t e = cudaSuccess;
-  const size_t vs = direct || !f32 ? 8 : 4;
+  const size_t vs = f32 ? 4 : 8;  // the panels' values
   if (!direct && (cost.form_us((double)np) + cost.iters() * cost.iter_us(nhead) >= cost.implicit_us(O) ||
                   2ull * nhead * SX_PART * vs > (16ull << 30)))
     return BA_OK;
@@ -319,7 +319,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   up(&x.task, task);
   up(&x.blk_cam, bcam);
   up(&x.blk_task, btask);
-  room(&x.part, (size_t)x.ntask * SX_PART * vs);
+  room(&x.part, (size_t)x.ntask * SX_PART * 8);
   auto unmark = [&] {
     if (e == cudaSuccess && lean) e = cudaMemsetAsync(x.lean_marked, 0, sizeof(int), s);
   };
@@ -447,7 +447,7 @@ void form(ba_problem* h) {
   static_assert(sizeof(ACC) >= sizeof(T), "the sums hold what the Jacobians hold");
   k_schur_form<T, MF, ACC><<<nb_(x.ntask, SF_WARPS), 32 * SF_WARPS, sf_smem<ACC>(), h->s>>>(
       x.ntask, x.task, x.blk_cam, x.pk, x.pl, x.pj, (const T*)h->Jcm, h->O, (const T*)h->camtab, (const T*)h->ptab,
-      (const T*)h->cm_sw, (const T*)h->Vinv, (ACC*)x.part);
+      (const T*)h->cm_sw, (const T*)h->Vinv, (double*)x.part);
   count_launch();
 }
 
@@ -455,8 +455,8 @@ template <typename VT>
 void pcg(ba_problem* h, int maxiter, double tol) {
   auto& x = h->sx;
   cudaStream_t s = h->s;
-  k_schur_combine<VT, VT><<<x.nblk, 96, 0, s>>>(x.blk_cam, x.blk_pos, x.blk_task, x.rowblk, (const VT*)x.part,
-                                                (VT*)x.val, x.lean ? (const double*)h->camtab : nullptr);
+  k_schur_combine<VT><<<x.nblk, 96, 0, s>>>(x.blk_cam, x.blk_pos, x.blk_task, x.rowblk, (const double*)x.part,
+                                            (VT*)x.val, x.lean ? (const double*)h->camtab : nullptr);
   cudaMemsetAsync(x.gx, 0, 8 * x.words, s);
   SchurPcg<VT> a;
   a.C = h->C;

@@ -6,6 +6,7 @@ import torch
 
 import oracle as orc
 import paper_2409_12190_gb300 as ba
+import scenegen
 from gpu_helpers import np64, problem, rel_err, small_ring
 from paper_2409_12190_gb300 import _lib
 from paper_2409_12190_gb300.partition import PartProblem, exchange_cap
@@ -131,3 +132,35 @@ def test_a_problem_that_fits_only_unformed_is_made():
     finally:
         del filler
         torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("narrow", [False, True])
+def test_single_precision_formed_system_is_as_accurate_as_the_implicit_product(narrow):
+    """FP32 trials from FP32-rounded inputs on both routes: their distances from
+    the FP64 answer, cameras and points, over 16 problems.  Wide: arcs of 6-36
+    cameras, points seen by up to ten of them.  Narrow: rings of 100 whose points
+    three neighbours see.  Both routes round per observation; forming S may add
+    no more than their spread (15 % of the mean of 16)."""
+    class Implicit(ba.Problem):
+        _create = "ba_problem_create_part"
+
+    f32 = lambda a: torch.as_tensor(a).float()
+    ratios = []
+    for seed in range(16):
+        if narrow:
+            cams, pts, ci, pi, pix = _large_ring(100, 12000, 3, seed=seed + 1)
+        else:
+            C = 6 + 2 * seed
+            sc = scenegen.arc_scene(C, 40 * C, seed=seed, views_lo=4, views_hi=min(C, 10))
+            cams, pts, ci, pi, pix = sc.cams_init, sc.points_init, sc.cam_idx, sc.pt_idx, orc.pixels_from_scene(sc)
+        out = []
+        for make, precision, formed in ((ba.Problem, "f64", None), (Implicit, "f32", 0), (ba.Problem, "f32", 1)):
+            opts = ba.Options(precision=precision, pcg_maxiter=20, pcg_tol=0.0)
+            with make(f32(cams), f32(pts), ci, pi, f32(pix), opts, device="cuda") as prob:
+                assert formed is None or prob.layout()["formed"] == formed
+                prob.solve(1)
+                out.append([np64(t) for t in prob.params()])
+        exact, implicit, form = out
+        ratios.append([np.linalg.norm(f - e) / np.linalg.norm(i - e) for e, i, f in zip(exact, implicit, form)])
+    mean = np.exp(np.log(ratios).mean(0))
+    assert mean[0] < 1.15 and mean[1] < 1.15, mean
