@@ -16,6 +16,7 @@
 #include <stdint.h>
 
 #include "ba_kernels.cuh"
+#include "ba_rcp.h"
 
 namespace ba {
 
@@ -102,25 +103,6 @@ __device__ __forceinline__ bool gx_gather(const GridX& gx, const unsigned long l
       if (e0 + u * nt < n) dst[e0 + u * nt] = gx_value(a[u], b[u]);
   }
   return true;
-}
-
-// 1 / d: for a normal d well inside the range a third-order step
-// y (1 + r + r^2), r = 1 - m y, on the FP32 reciprocal of d's significand (error
-// 2^-23 -> below 2^-60, so the result is within an ulp), scaled and checked on
-// the integer side; else the division.  A warp issues an FP64 instruction in
-// some 70 cycles; the division's were on the PCG's critical path twice an
-// iteration (with 1 / rz taken while the sums travel and no square root in the
-// stopping test: sphere of 2,500 poses 2,514 -> 2,371 us, ring of 97 cameras
-// in FP32 757 -> 727 us).
-__device__ __forceinline__ double gx_rcp(double d) {
-  const int hi = __double2hiint(d), ex = hi >> 20;
-  if (ex < 23 || ex > 2023) return 1.0 / d;
-  const int up = (ex - 1023) * (1 << 20);
-  const double m = __hiloint2double(hi - up, __double2loint(d));
-  const double y = (double)(1.0f / (float)m);
-  const double r = fma(-m, y, 1.0);
-  const double z = fma(y, fma(r, r, r), y);  // in (1/2, 1]
-  return __hiloint2double(__double2hiint(z) - up, __double2loint(z));
 }
 
 // warp_sum of NV values, the trees interleaved (the shuffles of one keep their
