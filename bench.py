@@ -211,7 +211,7 @@ def parse_clock_samples(text):
             "sm_max_mhz": max(mx) if mx else None, "reasons": reasons, "samples": len(rows)}
 
 
-def algorithmic_bytes(kind, C, P, O, npieces, tsize, mf, huber=False):
+def algorithmic_bytes(kind, C, P, O, npieces, tsize, mf, huber=False, pairs=0):
     """Compulsory HBM bytes of one launch: every array element the kernel
     must read or write, each counted once (per-observation planes, indices
     and weights; per-point / per-camera vectors once)."""
@@ -237,6 +237,8 @@ def algorithmic_bytes(kind, C, P, O, npieces, tsize, mf, huber=False):
         return O * (2 * tsize + 8 + ob) + P * (4 + 3 * tsize + 9 * 8) + C * 32 * tsize
     if kind == "schur_cam":
         return O * (4 + ob) + P * ((3 * tsize if mf else 0) + 9 * tsize) + npieces * 54 * 8
+    if kind == "form":     # per pair its two slots (FP32 also its point); the lean planes, or points and V*^-1
+        return pairs * 12 + P * (8 + 6) * tsize + C * 32 * tsize if mf else pairs * 8 + O * 20 * tsize
     if kind == "cost":     # pixels, point index, (model) planes; trial + current points, dp
         return O * (2 * tsize + 4 + ob) + P * 9 * tsize + npieces * 2 * 8
     if kind == "backsub":  # A1 + A2 of the back-substitution (two launches per trial)
@@ -271,7 +273,7 @@ def fp32_peak_tflops(sm_mhz):
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("ba_kernels.cuh", "ba_api.cu"):
+    for f in ("ba_kernels.cuh", "ba_schur.cuh", "ba_vec.cuh", "ba_api.cu"):
         with open(os.path.join(ROOT, "paper_2409_12190_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -436,21 +438,20 @@ def observation_pairs(pt_idx):
     return int((n * (n - 1) // 2).sum())
 
 
-def kernel_table(per, C, P, O, lay, tsize, mf, huber, alu_peak, form_flops=0):
+def kernel_table(per, C, P, O, lay, tsize, mf, huber, alu_peak, pairs=0, flops_per_pair=0):
     """Per kernel class: launches, mean CUDA-event time, share, algorithmic
-    GB/s and (PCG passes) TFLOP/s with their fractions.  form_flops: the
-    arithmetic of forming S once, when it is formed: its launch is timed with
-    the Schur blocks' (two launches a trial in schur_cam)."""
+    GB/s and (PCG passes, forming S) TFLOP/s with their fractions."""
     total = sum(v[0] for v in per.values())
     out = {}
     for name, (kms, n) in per.items():
         if n == 0:
             continue
-        b = algorithmic_bytes(name, C, P, O, lay["pieces"], tsize, mf, huber)
+        pieces = lay["product_pieces" if name.startswith("pass_") else "pieces"]
+        b = algorithmic_bytes(name, C, P, O, pieces, tsize, mf, huber, pairs)
         avg = kms / n
         row = {"launches": n, "avg_us": 1000.0 * avg, "share": kms / total,
                "gbs": (b / (avg / 1000.0) / 1e9) if b else None, "bytes_per_launch": b or None}
-        fl = form_flops / 2 if form_flops and name == "schur_cam" else pass_flops(name, O, P, mf)
+        fl = flops_per_pair * pairs if name == "form" else pass_flops(name, O, P, mf)
         if fl:
             row["tflops"] = fl / (avg / 1000.0) / 1e12
             row["flops_per_launch"] = fl
@@ -528,10 +529,10 @@ def run_precision(args, prec, scene, ci, pi, pix, dev, world, f_ref, peaks_d, ba
         alu_peak = peaks_d["fp64_fma_tflops"]
         alu_source = "measured (ba_measure_fma_peak: FP64 FMA chains on every SM, best of 3)"
     huber = scene.huber_delta > 0
-    formed = per.get("pass_b", (0.0, 0))[1] == 0  # PCG ran without passes over the observations
-    kernels = kernel_table(per, C, P, O, lay, tsize, mf, huber, alu_peak,
-                           FORM_FLOPS_PER_PAIR[prec] * observation_pairs(scene.pt_idx) if formed else 0)
-    it_bytes = sum(algorithmic_bytes(k, C, P, O, lay["pieces"], tsize, mf, huber) * per[k][1] for k in per)
+    formed = lay["formed"] == 1
+    pairs = observation_pairs(scene.pt_idx) if formed else 0
+    kernels = kernel_table(per, C, P, O, lay, tsize, mf, huber, alu_peak, pairs, FORM_FLOPS_PER_PAIR[prec])
+    it_bytes = sum((k["bytes_per_launch"] or 0) * k["launches"] for k in kernels.values())
     roof = roofline_of(kernels, per, peaks_d["hbm_gbs"], peaks_d["hbm_kind"], alu_peak, alu_source,
                        kernel_source_hash(), prof_ms, it_bytes, prec)
 

@@ -412,7 +412,8 @@ enum {
   BA_K_OTHER = 7,     /* per-camera / per-point / scalar kernels */
   BA_K_PASS_A2 = 8,   /* a4 PCG pass A2 (point-major sum, V*^{-1}) */
   BA_K_PASS_FA = 9,   /* a4 fused point-major pass A (A1 + A2, recompute mode) */
-  BA_K_COUNT = 10
+  BA_K_FORM = 10,     /* forming S: its blocks' partial sums from pairs of observations */
+  BA_K_COUNT = 11
 };
 
 typedef struct {

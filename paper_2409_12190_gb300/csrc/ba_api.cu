@@ -412,7 +412,7 @@ void enqueue_solve(ba_problem* h, const double* lam_ptr, int maxiter, double tol
     enqueue_dense_solve<T, MF>(h, lam_ptr);
   } else if (h->sx.pcg && !h->xch) {
     {
-      Prof pr(h, BA_K_SCHUR_CAM);
+      Prof pr(h, BA_K_FORM);
       schur_form(h);
     }
     Prof pr(h, BA_K_OTHER);
