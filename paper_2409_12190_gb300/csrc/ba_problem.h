@@ -130,6 +130,7 @@ struct ba_problem {
     bool lean = false;    // S from the lean form (FP64, stored planes)
     void *lean_w = nullptr, *lean_t = nullptr;  // [O] x 14 and x 6, in pairs
     int* lean_marked = nullptr;                 // set: some observation takes the planes instead
+    int marked_grid = 0;
     int nblk = 0, ntask = 0, groups = 0, rpb = 0, nc_max = 0, parts_max = 0;
     size_t words = 0;
     int32_t *pk = nullptr, *pl = nullptr, *pj = nullptr;

@@ -29,11 +29,14 @@ inline unsigned nb_(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 constexpr long long MAX_PAIRS = 1ll << 27;  // 12 bytes each kept, 36 more while they are sorted
 
 // FP32: formed only where the implicit iteration is mostly launches (20 us of
-// which 12 are launches at this size).  Beyond it the formed S would still be
-// 1.4 times as fast on 8.0M observations, but its rounding is another one than
-// the implicit product's, and on rings of thousands of cameras the points of
-// three neighbouring views amplify FP32 rounding (V* conditioned 1e4) beyond
-// what a result may move.
+// which 12 are launches at this size).  Neither time nor accuracy sets this
+// line: on 4,000 cameras and 8.0M observations two trials take 10.7 ms with the
+// implicit product and 8.0 with S formed, both as far from the FP64 answer
+// (cameras 1.2e-6, points 3.1e-5, four seeds), and below it rings of 250-4,000
+// cameras with 4.5-8 views a point are as near on either route.  What moves is
+// the answer itself: points that three neighbouring views see amplify FP32
+// rounding, so that the two routes' are up to 3e-3 apart there, and larger
+// problems keep the answers of the implicit product.
 constexpr long long F32_MAX_OBS = 1ll << 19;
 
 // The pairs of each point's observations (with the observation itself when
@@ -105,7 +108,11 @@ const void* form_kernel(bool direct, bool f32, bool mf) {
 // Whether the PCG on the formed S takes less time than the implicit product
 // (us, one GB300; each constant beside what it was measured on).  An LM trial
 // at ordinary damping runs 30-80 iterations (rings of 64-4,000 cameras,
-// lambda 1e-4 to 2e-3, tol 1e-4), or maxiter: 32 are assumed.
+// lambda 1e-4 to 2e-3, tol 1e-4), or maxiter: 32 are assumed.  It weighs one
+// trial against another.  Set-up is not in it: sorting the pairs takes 0.3 ms for
+// 16 cameras, 0.7 for 97 (FP32, 108,000 observations), 0.7 for 250 (480,000),
+// which a trial or two earn back (1.7, 0.4 and 4 ms a trial) but a problem made
+// for one FP32 trial of a few iterations may not.
 struct SchurCost {
   bool f32;
   int maxiter;
@@ -312,6 +319,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   const bool lean = !f32 && !h->mf;
   if (lean) {
     kernel_attr((const void*)k_schur_form_marked, sf_smem<double>());
+    x.marked_grid = 2 * nsm;
     room(&x.lean_w, 8ull * NLEAN * O);
     room(&x.lean_t, 8ull * 6 * O);
     room(&x.lean_marked, sizeof(int));
@@ -501,7 +509,7 @@ void schur_form(ba_problem* h) {
     const unsigned g = nb_(x.ntask, SF_WARPS);
     k_schur_form_lean<<<g, 32 * SF_WARPS, sf_smem<double>(), h->s>>>(
         x.ntask, x.task, x.pk, x.pl, (const double2*)x.lean_w, (const double2*)x.lean_t, h->O, (double*)x.part);
-    k_schur_form_marked<<<std::min(g, 304u), 32 * SF_WARPS, sf_smem<double>(), h->s>>>(
+    k_schur_form_marked<<<std::min(g, (unsigned)x.marked_grid), 32 * SF_WARPS, sf_smem<double>(), h->s>>>(
         x.ntask, x.task, x.pk, x.pl, x.pj, (const double2*)x.lean_w, (const double*)h->Jcm, h->O,
         (const double*)h->Vinv, x.lean_marked, (double*)x.part);
     count_launch(2);

@@ -6,7 +6,7 @@
 // every iteration; S has one 9 x 9 block per pair of cameras that see a common
 // point, far fewer numbers.  Forming it costs a pass over the pairs of
 // observations of each point, so it pays from a number of iterations on
-// (schur_pays in ba_schur.cu).
+// (SchurCost in ba_schur.cu).
 //
 //   pairs      (k, l), k and l observations of one point by cameras i <= l's
 //              camera, sorted by (camera of k, camera of l): the entries of
@@ -273,7 +273,7 @@ k_schur_form_lean(int ntask, const int4* __restrict__ task, const int32_t* __res
 }
 
 // The pairs that k_schur_form_lean left out, from the planes, in the same
-// coordinates, added to its sums (a grid of a few blocks an SM strides over the tasks: it
+// coordinates, added to its sums (a grid of two blocks an SM strides over the tasks: it
 // returns at once when no observation is marked).
 static __global__ void __launch_bounds__(32 * SF_WARPS)
 k_schur_form_marked(int ntask, const int4* __restrict__ task, const int32_t* __restrict__ pk,
