@@ -3,8 +3,9 @@
 // host: tests/c/band_schedule.cpp prints it, and the tests execute it.
 #pragma once
 
+#include <stdint.h>
+
 #include <algorithm>
-#include <functional>
 #include <queue>
 #include <utility>
 #include <vector>
@@ -186,7 +187,7 @@ inline std::vector<BandTask> band_tasks(const BandShape& sh, int s_upd, int work
   if (!simulate) crit_workers = 0;
   std::vector<int> segid(seg0[ntile], -1), idD(nb), idI(nb), idF(nb), idB(nb), idT(ntile, -1);
   std::vector<BandTask> task;
-  std::vector<double> dur;
+  std::vector<int> dur;
   std::vector<int> pbeg(1, 0), pred;  // predecessors: id * 2 + (1: D's early output)
   auto prod = [&](int I, int K) {
     return I == K ? 2 * idD[K] : (I == K + 1 ? 2 * idD[K + 1] + 1 : 2 * idT[sh.index(I, K)]);
@@ -198,7 +199,7 @@ inline std::vector<BandTask> band_tasks(const BandShape& sh, int s_upd, int work
   auto dep = [&](int p2) {
     if (p2 >= 0 && simulate) pred.push_back(p2);
   };
-  auto add = [&](int type, int cnt, int I, int J, int Ka, double d) {
+  auto add = [&](int type, int cnt, int I, int J, int Ka, int d) {
     task.push_back(BandTask{type + 8 * cnt, I, J, Ka});
     dur.push_back(d);
     pbeg.push_back((int)pred.size());
@@ -211,9 +212,9 @@ inline std::vector<BandTask> band_tasks(const BandShape& sh, int s_upd, int work
       if (a >= 0) dep(2 * a);
       if (b >= 0) dep(2 * b);
     }
-    idD[st] = add(BAND_D, 0, st, st, 0, 20.0);
+    idD[st] = add(BAND_D, 0, st, st, 0, 20);
     dep(2 * idD[st]);
-    idI[st] = add(BAND_I, 0, st, st, 0, 8.0);
+    idI[st] = add(BAND_I, 0, st, st, 0, 8);
     if (st >= 1) {
       const int K = st - 1;  // the segments that end with column K
       rows(K, col);
@@ -230,7 +231,7 @@ inline std::vector<BandTask> band_tasks(const BandShape& sh, int s_upd, int work
             dep(prod(I, k));
             dep(prod(J, k));
           }
-          segid[seg0[sh.index(I, J)] + m] = add(BAND_U, st - Ka, I, J, Ka, 12.0 * (st - Ka));
+          segid[seg0[sh.index(I, J)] + m] = add(BAND_U, st - Ka, I, J, Ka, 12 * (st - Ka));
         }
     }
     rows(st, col);
@@ -239,7 +240,7 @@ inline std::vector<BandTask> band_tasks(const BandShape& sh, int s_upd, int work
       dep(2 * idD[st]);
       const int a = last_seg(I, st);
       if (a >= 0) dep(2 * a);
-      idT[sh.index(I, st)] = add(BAND_T, 0, I, st, 0, 7.0);
+      idT[sh.index(I, st)] = add(BAND_T, 0, I, st, 0, 7);
     }
     const int c = sh.chain(st);
     if (st > sh.chain_begin(c)) dep(2 * idF[st - 1]);
@@ -253,28 +254,27 @@ inline std::vector<BandTask> band_tasks(const BandShape& sh, int s_upd, int work
       for (int K = sh.first_rest(st); K < st; ++K) dep(prod(st, K));
     dep(prod(st, st));
     dep(2 * idI[st]);
-    idF[st] = add(BAND_F, 0, st, st, 0, 4.0);
+    idF[st] = add(BAND_F, 0, st, st, 0, 4);
   }
   for (int I = nb - 1; I >= 0; --I) {
     dep(2 * idF[nb - 1]);
     if (I + 1 < sh.chain_end(sh.chain(I))) dep(2 * idB[I + 1]);
     else if (I + 1 < nb) dep(2 * idB[sh.joint]);
-    idB[I] = add(BAND_B, 0, I, I, 0, 4.0);
+    idB[I] = add(BAND_B, 0, I, I, 0, 4);
   }
   const int nt = (int)task.size();
   if (!simulate) {
     *ncrit = 0;
     return task;
   }
-  const double lat = 1.0, early = 8.0;
-  auto out_time = [&](int p2, double start_or_len) { return (p2 & 1) ? early : start_or_len; };
+  const int lat = 1, early = 8;
   // longest path to the end
-  std::vector<double> bl(nt, 0.0);
+  std::vector<int> bl(nt, 0);
   for (int t = nt - 1; t >= 0; --t) {
     bl[t] = std::max(bl[t], dur[t]);
     for (int k = pbeg[t]; k < pbeg[t + 1]; ++k) {
       const int p = pred[k] >> 1;
-      bl[p] = std::max(bl[p], out_time(pred[k], dur[p]) + lat + bl[t]);
+      bl[p] = std::max(bl[p], ((pred[k] & 1) ? early : dur[p]) + lat + bl[t]);
     }
   }
   // the near-diagonal tasks (the chain D_J and what feeds it: updates that
@@ -289,7 +289,10 @@ inline std::vector<BandTask> band_tasks(const BandShape& sh, int s_upd, int work
               (type == BAND_T && sh.slot(q.y, q.z) <= 2);
   }
   // list scheduling: at each moment the idle blocks of a pool take its ready
-  // tasks, highest priority first
+  // tasks, highest priority (longest path, then first enumerated) first.  Times
+  // are whole numbers: the outputs that fall due are kept in a ring of one bucket
+  // a time, as long as the longest task, and what they release is ready `lat`
+  // later.
   std::vector<int> sbeg(nt + 1, 0), succ(pred.size()), npred(nt, 0);
   for (int p : pred) ++sbeg[(p >> 1) + 1];
   for (int t = 0; t < nt; ++t) {
@@ -299,64 +302,51 @@ inline std::vector<BandTask> band_tasks(const BandShape& sh, int s_upd, int work
   std::vector<int> sfill(sbeg.begin(), sbeg.end() - 1);
   for (int t = 0; t < nt; ++t)
     for (int k = pbeg[t]; k < pbeg[t + 1]; ++k) succ[sfill[pred[k] >> 1]++] = t * 2 + (pred[k] & 1);
-  std::vector<double> ready(nt, 0.0), start(nt, 0.0);
-  typedef std::pair<double, int> E;
-  std::priority_queue<E, std::vector<E>, std::greater<E>> pending, events;  // by time
-  auto higher = [&](int x, int y) { return bl[x] < bl[y] || (bl[x] == bl[y] && x > y); };
-  std::priority_queue<int, std::vector<int>, decltype(higher)> avail[2] = {
-      std::priority_queue<int, std::vector<int>, decltype(higher)>(higher),
-      std::priority_queue<int, std::vector<int>, decltype(higher)>(higher)};
+  std::vector<std::vector<int>> ring((size_t)std::max(early, *std::max_element(dur.begin(), dur.end())) + 1);
+  std::priority_queue<uint64_t> avail[2];
+  auto key = [&](int t) { return ((uint64_t)bl[t] << 32) | (uint32_t)~(uint32_t)t; };
   int idle[2] = {std::max(1, workers - crit_workers), crit_workers};
+  std::vector<int> due, soon, first;  // ready now, ready after lat, started now
   for (int t = 0; t < nt; ++t)
-    if (npred[t] == 0) pending.push(E(0.0, t));
-  double clock = 0.0;
-  int done = 0;
-  while (done < nt) {
-    // outputs due by now release their successors; ready tasks join their pool
-    while (!events.empty() && events.top().first <= clock) {
-      const int code = events.top().second;
-      const double tm = events.top().first;
-      events.pop();
+    if (npred[t] == 0) due.push_back(t);
+  std::vector<int> order[2];  // a pool's tasks by start, then by enumeration
+  size_t at = 0;              // the clock's place in the ring
+  while ((int)(order[0].size() + order[1].size()) < nt) {
+    // outputs due now release their successors; ready tasks join their pool
+    for (int code : ring[at]) {
       const int p = code >> 1, early_out = code & 1;
       if (!early_out) ++idle[crit[p]];
       for (int k = sbeg[p]; k < sbeg[p + 1]; ++k)
-        if ((succ[k] & 1) == early_out) {
-          const int q = succ[k] >> 1;
-          ready[q] = std::max(ready[q], tm + lat);
-          if (--npred[q] == 0) pending.push(E(ready[q], q));
-        }
+        if ((succ[k] & 1) == early_out && --npred[succ[k] >> 1] == 0) soon.push_back(succ[k] >> 1);
     }
-    while (!pending.empty() && pending.top().first <= clock) {
-      avail[crit[pending.top().second]].push(pending.top().second);
-      pending.pop();
-    }
-    for (int pl = 0; pl < 2; ++pl)
-      while (idle[pl] > 0 && !avail[pl].empty()) {
-        const int t = avail[pl].top();
+    ring[at].clear();
+    for (int t : due) avail[crit[t]].push(key(t));
+    for (int pl = 0; pl < 2; ++pl) {
+      first.clear();
+      for (; idle[pl] > 0 && !avail[pl].empty(); --idle[pl]) {
+        const int t = (int)~(uint32_t)avail[pl].top();
         avail[pl].pop();
-        --idle[pl];
-        start[t] = clock;
-        events.push(E(clock + dur[t], 2 * t));
-        if ((task[t].x & 7) == BAND_D) events.push(E(clock + early, 2 * t + 1));
-        ++done;
+        first.push_back(t);
+        ring[(at + dur[t]) % ring.size()].push_back(2 * t);
+        if ((task[t].x & 7) == BAND_D) ring[(at + early) % ring.size()].push_back(2 * t + 1);
       }
-    double nxt = 1e300;
-    if (!events.empty()) nxt = std::min(nxt, events.top().first);
-    if (!pending.empty()) nxt = std::min(nxt, pending.top().first);
-    if (nxt == 1e300) break;  // not reached: the enumeration is acyclic
-    clock = std::max(clock, nxt);
+      std::sort(first.begin(), first.end());
+      order[pl].insert(order[pl].end(), first.begin(), first.end());
+    }
+    due.clear();
+    due.swap(soon);
+    // to the next moment at which something is due
+    size_t step = 1;
+    while (due.empty() && step < ring.size() && ring[(at + step) % ring.size()].empty()) ++step;
+    if (due.empty() && step == ring.size()) break;  // not reached: the enumeration is acyclic
+    at = (at + step) % ring.size();
   }
-  // tickets: the critical pool's tasks, then the bulk pool's, each by
-  // simulated start
-  std::vector<int> order(nt);
-  for (int t = 0; t < nt; ++t) order[t] = t;
-  std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
-    return crit[x] != crit[y] ? crit[x] > crit[y] : start[x] < start[y];
-  });
-  *ncrit = 0;
-  for (int t = 0; t < nt; ++t) *ncrit += crit[t];
-  std::vector<BandTask> out(nt);
-  for (int t = 0; t < nt; ++t) out[t] = task[order[t]];
+  // tickets: the near-diagonal pool's tasks, then the bulk pool's
+  *ncrit = (int)order[1].size();
+  std::vector<BandTask> out;
+  out.reserve(nt);
+  for (int pl = 1; pl >= 0; --pl)
+    for (int t : order[pl]) out.push_back(task[t]);
   return out;
 }
 
