@@ -821,7 +821,13 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
   // problems adds it in the same order.
   std::vector<int32_t> rp(C + 1);
   CU(cudaMemcpy(rp.data(), h->rowptr_cam, (C + 1) * 4, cudaMemcpyDeviceToHost));
-  auto cut = [&](int most, int* count, int32_t** d_cam, int32_t** d_beg, int32_t** d_end, int32_t** d_ptr) -> ba_status {
+  // one cut's lists, then the other's, in one allocation and one copy
+  std::vector<int32_t> cuts;
+  struct Cut {
+    size_t cam, beg, end, ptr;
+    int n;
+  };
+  auto cut = [&](int most) {
     std::vector<int32_t> pc, pb, pe, cpp(C + 1);
     for (long long c = 0; c < C; ++c) {
       cpp[c] = (int32_t)pc.size();
@@ -834,31 +840,29 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
       }
     }
     cpp[C] = (int32_t)pc.size();
-    *count = (int)pc.size();
-    CU(h->alloc(d_cam, pc.size() * 4));
-    CU(h->alloc(d_beg, pc.size() * 4));
-    CU(h->alloc(d_end, pc.size() * 4));
-    CU(h->alloc(d_ptr, (C + 1) * 4));
-    CU(cudaMemcpy(*d_cam, pc.data(), pc.size() * 4, cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(*d_beg, pb.data(), pb.size() * 4, cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(*d_end, pe.data(), pe.size() * 4, cudaMemcpyHostToDevice));
-    CU(cudaMemcpy(*d_ptr, cpp.data(), (C + 1) * 4, cudaMemcpyHostToDevice));
-    return BA_OK;
+    auto put = [&](const std::vector<int32_t>& v) {
+      const size_t at = cuts.size();
+      cuts.insert(cuts.end(), v.begin(), v.end());
+      cuts.resize((cuts.size() + 63) / 64 * 64);
+      return at;
+    };
+    Cut r{put(pc), put(pb), put(pe), put(cpp), (int)pc.size()};
+    return r;
   };
-  {
-    const ba_status cs = cut(PIECE, &h->nlong, &h->long_cam, &h->long_beg, &h->long_end, &h->cam_long_ptr);
-    if (cs != BA_OK) return cs;
-  }
-  if (piece_max != PIECE) {
-    const ba_status cs = cut(piece_max, &h->npieces, &h->piece_cam, &h->piece_beg, &h->piece_end, &h->cam_piece_ptr);
-    if (cs != BA_OK) return cs;
-  } else {
-    h->npieces = h->nlong;
-    h->piece_cam = h->long_cam;
-    h->piece_beg = h->long_beg;
-    h->piece_end = h->long_end;
-    h->cam_piece_ptr = h->cam_long_ptr;
-  }
+  const Cut lc = cut(PIECE), sc = piece_max != PIECE ? cut(piece_max) : lc;
+  int32_t* d_cuts = nullptr;
+  CU(h->alloc(&d_cuts, cuts.size() * 4));
+  CU(cudaMemcpy(d_cuts, cuts.data(), cuts.size() * 4, cudaMemcpyHostToDevice));
+  h->nlong = lc.n;
+  h->long_cam = d_cuts + lc.cam;
+  h->long_beg = d_cuts + lc.beg;
+  h->long_end = d_cuts + lc.end;
+  h->cam_long_ptr = d_cuts + lc.ptr;
+  h->npieces = sc.n;
+  h->piece_cam = d_cuts + sc.cam;
+  h->piece_beg = d_cuts + sc.beg;
+  h->piece_end = d_cuts + sc.end;
+  h->cam_piece_ptr = d_cuts + sc.ptr;
 
   // linearisation and solver buffers
   CU(h->alloc(&h->camtab, CT * C * ts));

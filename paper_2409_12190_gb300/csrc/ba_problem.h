@@ -25,6 +25,7 @@ ba_status problem_create(ba_problem** out, int C, int P, int O, const void* cams
 // when there is no room.
 struct SchurPairs {
   int n = 0;
+  int32_t* mem = nullptr;  // the three lists' memory
   int32_t *pk = nullptr, *pl = nullptr, *pj = nullptr;
   std::vector<int32_t> head;
   std::vector<int2> cam;

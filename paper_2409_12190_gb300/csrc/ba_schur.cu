@@ -132,15 +132,11 @@ struct SchurCost {
 
 }  // namespace
 
-SchurPairs::~SchurPairs() {
-  for (int32_t* p : {pk, pl, pj}) cudaFree(p);
-}
+SchurPairs::~SchurPairs() { cudaFree(mem); }
 
 void SchurPairs::keep(std::vector<void*>& allocs) {
-  for (int32_t** p : {&pk, &pl, &pj}) {
-    allocs.push_back(*p);
-    *p = nullptr;
-  }
+  allocs.push_back(mem);
+  mem = nullptr;
 }
 
 ba_status schur_pairs(ba_problem* h, const std::vector<int32_t>& rq, bool self, long long most, SchurPairs& out) {
@@ -157,15 +153,14 @@ ba_status schur_pairs(ba_problem* h, const std::vector<int32_t>& rq, bool self, 
   if (np == 0) return BA_OK;
   cudaStream_t s = h->s;
   const int n = (int)np;
-  // one allocation for everything that is not kept
+  // two allocations, what is kept and what is not (each takes some 50 us)
   const size_t scratch_bytes = csr_scratch_bytes(n);
   auto al = [](size_t b) { return (b + 255) / 256 * 256; };
   const size_t need = al(4ull * (P + 1)) + 7 * al(4ull * n) + al(4ull * (std::max(C, 2) + 1)) + al(8ull * n) +
                       al(scratch_bytes);
   char* base = nullptr;
   cudaError_t e = cudaMalloc(&base, need);
-  for (int32_t** p : {&out.pk, &out.pl, &out.pj})
-    if (e == cudaSuccess) e = cudaMalloc(p, 4ull * n);
+  if (e == cudaSuccess) e = cudaMalloc(&out.mem, 3 * al(4ull * n));
   struct Free {
     char* p;
     ~Free() { cudaFree(p); }
@@ -174,6 +169,9 @@ ba_status schur_pairs(ba_problem* h, const std::vector<int32_t>& rq, bool self, 
     cudaGetLastError();  // no room: the implicit product (or the dense build) as before
     return BA_OK;
   }
+  out.pk = out.mem;
+  out.pl = out.pk + al(4ull * n) / 4;
+  out.pj = out.pl + al(4ull * n) / 4;
   size_t off = 0;
   auto take = [&](size_t bytes) {
     char* p = base + off;
