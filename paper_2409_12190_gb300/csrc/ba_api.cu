@@ -756,23 +756,28 @@ ba_status create_impl(ba_problem* h, const void* cams, const void* points, const
   // if no chunk has more than FA_CAMS of them
   {
     std::vector<int32_t> pmc(O), list, ptr(h->nchunks + 1), tmp;
-    std::vector<int16_t> lc(O);
+    std::vector<int32_t> in(C, -1);  // the last chunk that sees a camera
+    std::vector<int16_t> lc(O), place(C);
     CU(cudaMemcpy(pmc.data(), h->pm_cam, O * 4, cudaMemcpyDeviceToHost));
     bool ok = true;
     for (int k = 0; k < h->nchunks && ok; ++k) {
       const int s0 = rq[pch[k]], s1 = rq[pch[k + 1]];
-      tmp.assign(pmc.begin() + s0, pmc.begin() + s1);
-      std::sort(tmp.begin(), tmp.end());
-      tmp.erase(std::unique(tmp.begin(), tmp.end()), tmp.end());
+      tmp.clear();
+      for (int q = s0; q < s1; ++q)
+        if (in[pmc[q]] != k) {
+          in[pmc[q]] = k;
+          tmp.push_back(pmc[q]);
+        }
       if ((int)tmp.size() > FA_CAMS) {
         ok = false;
         break;
       }
+      std::sort(tmp.begin(), tmp.end());
       ptr[k] = (int32_t)list.size();
       list.insert(list.end(), tmp.begin(), tmp.end());
       h->fa_nc = std::max(h->fa_nc, (int)tmp.size());
-      for (int q = s0; q < s1; ++q)
-        lc[q] = (int16_t)(std::lower_bound(tmp.begin(), tmp.end(), pmc[q]) - tmp.begin());
+      for (size_t i = 0; i < tmp.size(); ++i) place[tmp[i]] = (int16_t)i;
+      for (int q = s0; q < s1; ++q) lc[q] = place[pmc[q]];
     }
     if (ok) {
       ptr[h->nchunks] = (int32_t)list.size();
