@@ -122,8 +122,19 @@ struct SchurCost {
   double implicit_us(double O) const {
     return iters() * (12.0 + O * (f32 ? 1.5e-5 : 1.28e-4)) + (maxiter - iters()) * 6.0;
   }
-  // forming: FP64 pipe (13 ns per 32 pairs), FP32 arithmetic and gathers
-  double form_us(double pairs) const { return 25.0 + pairs * (f32 ? 5.0e-5 : 3.1e-4); }
+  // forming: FP64 pipe (13 ns per 32 pairs), FP32 arithmetic and gathers.  In
+  // FP64 both sides are understated, an implicit iteration by the latency of its
+  // passes (24 us), forming by the lean form (2e-4 us an observation, in the
+  // linearisation and the Schur blocks) and by short tasks (1e-4 a pair); what the
+  // second exceeds the first by counts.  Formed over implicit without it, and
+  // what it chooses: 2,500 cameras, 2.0M observations, 2.6 pairs each, 8 iterations
+  // 1.06 (implicit), 10 0.97 (formed); 5.4 pairs each, 16 1.12 (implicit), 20
+  // 1.01 and 30 0.83 (formed); 1,000 cameras, 0.9M, 10 1.05 (implicit), 12
+  // 0.97 (formed); 4,000 cameras, 4.7M, 12 1.07 (implicit), 16 0.94 (formed).
+  double form_us(double pairs, double O) const {
+    const double more = f32 ? 0.0 : std::max(0.0, 2.0e-4 * O + 1.0e-4 * pairs - 24.0 * iters());
+    return 25.0 + pairs * (f32 ? 5.0e-5 : 3.1e-4) + more;
+  }
   // more pairs than this and forming alone takes longer
   long long most_pairs(double O) const { return (long long)(std::max(0.0, implicit_us(O) - 25.0) / (f32 ? 5.0e-5 : 3.1e-4)); }
   // two exchanges, then 81 multiply-adds or 324 bytes a block
@@ -244,7 +255,7 @@ ba_status schur_build(ba_problem* h, const std::vector<int32_t>& rq) {
   cudaStream_t s = h->s;
   cudaError_t e = cudaSuccess;
   const size_t vs = f32 ? 4 : 8;  // the panels' values
-  if (!direct && (cost.form_us((double)np) + cost.iters() * cost.iter_us(nhead) >= cost.implicit_us(O) ||
+  if (!direct && (cost.form_us((double)np, O) + cost.iters() * cost.iter_us(nhead) >= cost.implicit_us(O) ||
                   2ull * nhead * SX_PART * vs > (16ull << 30)))
     return BA_OK;
 
