@@ -515,6 +515,10 @@ ba_status ba_batch_set_launch(ba_batch* h, int ctas_per_sm, int variant, int ord
  * outputs, any may be NULL; no counterpart in the paper). */
 ba_status ba_batch_get_launch(ba_batch* h, int* ctas_per_sm, int* variant, int* order,
                               int* grid);
+/* *formed (host): 1 if the problems' reduced systems are formed in their CTAs
+ * (FP32, recomputed Jacobians), 0 if they take the implicit product.
+ * Measurement aid: no counterpart in the paper. */
+ba_status ba_batch_get_formed(const ba_batch* h, int* formed);
 
 /* Segment sizes of the batched solve (no counterpart in the paper; the
  * symbolic phase's cut, Sec. IV-B): each camera's observations in equal

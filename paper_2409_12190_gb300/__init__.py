@@ -473,6 +473,12 @@ class Batch:
         _lib.check(_L().ba_batch_get_launch(self._h, ct.byref(c), ct.byref(v), ct.byref(o), ct.byref(g)))
         return dict(ctas_per_sm=c.value, variant=v.value, order=o.value, grid=g.value)
 
+    def formed(self):
+        """Whether the problems' reduced systems are formed in their CTAs."""
+        f = ct.c_int()
+        _lib.check(_L().ba_batch_get_formed(self._h, ct.byref(f)))
+        return bool(f.value)
+
     def set_segments(self, piece_max: int = 2048, chunk_slots: int = 1024, chunk_pts: int = 512):
         """Segment sizes of the solve (pieces of camera-major slots, point
         chunks); another cut moves results by rounding."""

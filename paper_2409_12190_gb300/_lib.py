@@ -115,6 +115,7 @@ SIGNATURES = {
     "ba_batch_get_scalars": (_S, [_VP, _VP, _VP]),
     "ba_batch_set_launch": (_S, [_VP, _I, _I, _I]),
     "ba_batch_get_launch": (_S, [_VP, ct.POINTER(_I), ct.POINTER(_I), ct.POINTER(_I), ct.POINTER(_I)]),
+    "ba_batch_get_formed": (_S, [_VP, ct.POINTER(_I)]),
     "ba_batch_autotune": (_S, [_VP, _I, ct.c_char_p, ct.POINTER(_D)]),
     "ba_batch_set_segments": (_S, [_VP, _I, _I, _I]),
     "ba_batch_get_segments": (_S, [_VP, ct.POINTER(_I), ct.POINTER(_I), ct.POINTER(_I)]),

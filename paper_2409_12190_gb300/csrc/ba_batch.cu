@@ -699,6 +699,12 @@ ba_status ba_batch_get_launch(ba_batch* b, int* ctas_per_sm, int* variant, int* 
   return BA_OK;
 }
 
+ba_status ba_batch_get_formed(const ba_batch* b, int* formed) {
+  if (!b || !formed) return set_error(BA_ERR_INVALID_ARG, "NULL argument");
+  *formed = b->sx_val ? 1 : 0;
+  return BA_OK;
+}
+
 ba_status ba_batch_autotune(ba_batch* b, int iters, const char* cache_path, double* best_ms) {
   if (!b || iters < 1) return set_error(BA_ERR_INVALID_ARG, "NULL batch or iters < 1");
   if (best_ms) *best_ms = 0.0;

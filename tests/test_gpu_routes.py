@@ -173,3 +173,34 @@ def test_the_formed_system_is_chosen_where_it_was_measured_to_pay(maxiter, forme
     opts = ba.Options(precision="f64", pcg_maxiter=maxiter, pcg_tol=0.0)
     with ba.Problem(*_large_ring(1000, 112500, 8, seed=2), opts, device="cuda") as prob:
         assert prob.layout()["formed"] == formed
+
+
+@pytest.mark.parametrize("C,P", [(2, 5), (7, 33), (30, 700), (151, 900), (153, 1200), (310, 1500)])
+def test_small_problems_take_the_formed_route(C, P):
+    """The sizes at which the formed system is compared with the oracle do form
+    it, in one launch for the whole PCG; the implicit product takes three an
+    iteration."""
+    sc = scenegen.arc_scene(C, P, seed=C, views_lo=1, views_hi=9)
+    pix = orc.pixels_from_scene(sc)
+    for precision in ("f64", "f32"):
+        with problem(sc, pix, precision) as prob:
+            assert prob.layout()["formed"] == 1
+            prob.damped_solve(1e-2, 8, 0.0)
+            torch.cuda.synchronize()
+            n = ba.kernel_launch_count()
+            prob.damped_solve(1e-2, 8, 0.0)
+            assert ba.kernel_launch_count() - n < 20
+    with problem(sc, pix, "f64", jacobian="recompute") as prob:
+        assert prob.layout()["formed"] == 0
+    with problem(sc, pix, "f64", solver="cholesky") as prob:
+        assert prob.layout()["formed"] == 2
+
+
+def test_windows_are_formed_in_single_precision():
+    inputs = []
+    for C in (2, 6, 20):
+        sc = scenegen.arc_scene(C, 40 * C, seed=C, views_lo=2, views_hi=min(C, 6))
+        inputs.append((sc.cams_init, sc.points_init, sc.cam_idx, sc.pt_idx, orc.pixels_from_scene(sc)))
+    for precision, jacobian, formed in (("f32", "auto", True), ("f32", "store", False), ("f64", "auto", False)):
+        with ba.Batch(inputs, ba.Options(precision=precision, jacobian=jacobian, pcg_maxiter=10)) as batch:
+            assert batch.formed() == formed
