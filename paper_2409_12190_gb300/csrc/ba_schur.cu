@@ -31,7 +31,7 @@ constexpr long long MAX_PAIRS = 1ll << 27;  // 12 bytes each kept, 36 more while
 // FP32: formed only where the implicit iteration is mostly launches (20 us of
 // which 12 are launches at this size).  Neither time nor accuracy sets this
 // line: on 4,000 cameras and 8.0M observations two trials take 10.7 ms with the
-// implicit product and 8.0 with S formed, both as far from the FP64 answer
+// implicit product and 7.8 with S formed, both as far from the FP64 answer
 // (cameras 1.2e-6, points 3.1e-5, four seeds), and below it rings of 250-4,000
 // cameras with 4.5-8 views a point are as near on either route.  What moves is
 // the answer itself: points that three neighbouring views see amplify FP32
