@@ -8,7 +8,8 @@ import paper_2409_12190_gb300 as ba
 import scenegen
 from oracle import LMOptions
 from oracle import pgo
-from paper_2409_12190_gb300.pgo import PoseGraph, synthesize
+from paper_2409_12190_gb300.pgo import PoseGraph
+from paper_2409_12190_gb300.pgo import synthesize
 
 pytestmark = pytest.mark.gpu
 
