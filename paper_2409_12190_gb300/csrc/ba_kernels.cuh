@@ -2454,18 +2454,22 @@ k_cam_trial(int C, double* __restrict__ x, const double* __restrict__ gc, T* __r
             double* __restrict__ dot_gc, const int* __restrict__ lost) {
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   double gd = 0.0;
-  if (lost && *lost) {
-    if (c < C)
-      for (int i = 0; i < 9; ++i) x[9LL * c + i] = 0.0;
-    if (c == 0) {
-      st->fallbacks += 1;
-      st->pcg_rel = 1.0;
-      st->pcg_done = 1;
-    }
+  const bool none = lost && *lost;
+  if (none && c == 0) {
+    st->fallbacks += 1;
+    st->pcg_rel = 1.0;
+    st->pcg_done = 1;
   }
   if (c < C) {
     const int cur = st->cur;
-    gd = cam_trial_one<T, MF>(x + 9LL * c, gc + 9LL * c, cams_buf + (long long)cur * 9 * C + 9LL * c,
+    double xc[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) xc[i] = none ? 0.0 : x[9LL * c + i];
+    if (none) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) x[9LL * c + i] = 0.0;
+    }
+    gd = cam_trial_one<T, MF>(xc, gc + 9LL * c, cams_buf + (long long)cur * 9 * C + 9LL * c,
                               cams_buf + (long long)(1 - cur) * 9 * C + 9LL * c, camtab + (long long)CT * c,
                               xT + (long long)pass_vec_stride(MF) * c);
   }
